@@ -71,8 +71,9 @@ SCALE_ROT_BYTES = (21 + 9 + 3) * 4
 # kernel's committed ncu summary (profiles/) only while these are unchanged.
 KERNEL_SOURCES = {
     "blend_fused_kernel": ["raster.cu"], "blend_bwd_kernel": ["raster.cu"], "blend_fwd_kernel": ["raster.cu"],
-    "project_fwd_kernel": ["project.cu", "cond.cuh", "sh.cuh", "mat3.cuh", "stage.cuh"],
-    "onesweep_kernel": ["sort.cu"], "emit_expand_kernel": ["sort.cu"], "compact_kernel": ["sort.cu"],
+    "project_fwd_kernel": ["project.cu", "bin.cuh", "cond.cuh", "sh.cuh", "mat3.cuh", "stage.cuh"],
+    "bin_scan_kernel": ["sort.cu", "bin.cuh"], "bin_scatter_kernel": ["sort.cu", "bin.cuh"],
+    "bin_sort_kernel": ["sort.cu", "bin.cuh"],
     "geom_bwd_kernel": ["project_bwd.cu", "cond.cuh", "mat3.cuh"],
     "sh_bwd_kernel": ["project_bwd.cu", "cond.cuh", "mat3.cuh", "sh.cuh"],
     "scale_rotation_kernel": ["scale_rotation.cu", "cond.cuh", "mat3.cuh"],
@@ -433,11 +434,20 @@ def hbm_peak():
 
 
 def launches_per_frame(plan, n_cams):
-    """Kernels of ours one fwd+bwd frame launches: camera upload (one per 48
-    cameras), projection, compaction, depth passes, emission (scan + expand),
-    tile passes, ranges, fused blend forward + L1 + blend backward, SH
-    backward, geometry backward."""
+    """Kernels of one frame whose lists are sorted by one radix pass per digit
+    (camera upload, projection, compaction, depth passes, emission scan +
+    expand, tile passes, ranges, fused blend, SH and geometry backward): what a
+    plan's digit counts stand for, and the launches that the tile-first binning
+    (step_launches) is compared with."""
     return (n_cams + 47) // 48 + 1 + 1 + plan.depth_passes + 2 + plan.tile_passes + 1 + 1 + 1 + 1
+
+
+def step_launches(n_cams):
+    """Kernels of ours one fwd+bwd frame launches: camera upload (one per 48
+    cameras), projection, list scan, scatter and sort, fused blend forward + L1
+    + blend backward, SH backward, geometry backward."""
+    return (n_cams + 47) // 48 + 1 + 3 + 1 + 1 + 1
+
 
 def build_inputs(args):
     w = synth.make_workload(args.config, n_override=args.n or None)
@@ -609,7 +619,7 @@ def run_ours(args, world, rank, local):
         ms_plain = max_over_ranks(sum(t_plain) / len(t_plain), world)
         rp0 = next(iter(plain_r.values()))
         plain = {"value": V * 1000.0 / ms_plain * world, "unit": UNIT, "ms_per_step": ms_plain,
-                 "launches_per_step": V * launches_per_frame(rp0.plan, 1), "graph": False}
+                 "launches_per_step": V * step_launches(1), "graph": False}
         g_rel = {k: float((grads_p[k] - grads_batched[k]).norm() / grads_batched[k].norm().clamp_min(1e-30))
                  for k in grads_p}
         equiv = {"image_max_abs": float((images - img_batched).abs().max()),
@@ -799,7 +809,7 @@ def run_ours(args, world, rank, local):
         "config": workload_config(w, kw["tile"], world),
         "e2e": e2e, "roofline": roofline, "cpu_baseline": cpu,
         "clocks": {k: clk[k] for k in ("sm_mhz", "sm_max_mhz", "reasons")},
-        "gpu_launches": launches_per_frame(r.plan, V) * args.steps,
+        "gpu_launches": step_launches(V) * args.steps,
         "megapixels_per_s": round(r.total_pixels * world / (ms_batched * 1e-3) / 1e6, 1),
         "loss": loss_batched,
         "autotuned": None if tuned is None else {k: tuned[k] for k in ("tile", "batch", "persistent", "ms", "cached")},

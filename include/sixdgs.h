@@ -11,8 +11,8 @@
  *   bin_sort          : duplicate every visible Gaussian into the screen tiles
  *                       of its tile rectangle (settings.alpha_footprint: the
  *                       3-sigma square, by default intersected with the box
- *                       of its alpha >= 1/255 ellipse) and radix-sort the
- *                       (tile, depth) keys (section 4.4, inherited 3DGS step);
+ *                       of its alpha >= 1/255 ellipse) and sort them by
+ *                       (tile, depth) (section 4.4, inherited 3DGS step);
  *   raster_fwd        : blend every tile front to back (section 4.4), with an
  *                       optional fused L1 loss (the 3DGS loss section 4.4
  *                       keeps);
@@ -167,8 +167,8 @@ typedef struct sixdgs_plan {
   int64_t total_tiles;    /* screen tiles over all cameras                    */
   int64_t total_pixels;   /* pixels over all cameras                          */
   int64_t dup_capacity;   /* room for (Gaussian, tile) duplicates             */
-  int32_t depth_passes;   /* radix passes over the depth key                  */
-  int32_t tile_passes;    /* radix passes over the tile key                   */
+  int32_t depth_passes;   /* bytes of the depth key                           */
+  int32_t tile_passes;    /* bytes of the global tile id                      */
   int64_t ws_bytes;       /* required workspace size                          */
   int64_t off[32];        /* byte offsets of the workspace sections           */
 } sixdgs_plan;
@@ -236,13 +236,14 @@ sixdgs_status sixdgs_condition_project(const sixdgs_plan* plan, const sixdgs_sce
                                        size_t ws_bytes, int32_t* status_dev,
                                        sixdgs_stream_t stream);
 
-/* Stage 2 -- binning and sort (section 4.4).  Visible (view, Gaussian) pairs
- * are radix-sorted by depth (stable, so equal depths keep Gaussian-id
- * order), duplicated once per touched tile in that order, and stably
- * radix-sorted by global tile id: an LSD sort of the composite
- * (tile, depth, id) key whose depth digits run before duplication.  Both
- * sorts are single-pass-per-digit "onesweep" sorts with decoupled look-back.
- * Writes SORTED, RANGES and COUNTS.  Device: CAPACITY, TIMEOUT. */
+/* Stage 2 -- binning and sort (section 4.4).  Every visible (view, Gaussian)
+ * pair is duplicated once per touched tile, and each tile's list is sorted by
+ * (depth, Gaussian id): the ranges from a scan of the tile counts that
+ * condition_project left, the duplicates scattered to their tiles, then every
+ * list sorted on chip (lists above 4,096 entries in runs that a cluster of
+ * CTAs merges).  May be called again on the same projection.
+ * Writes SORTED, SORTEDKEY, RANGES and COUNTS.  Device: CAPACITY (lists beyond
+ * the capacity are cut), TIMEOUT (a look-back wait of the scan). */
 sixdgs_status sixdgs_bin_sort(const sixdgs_plan* plan, void* ws_dev, size_t ws_bytes,
                               int32_t* status_dev, sixdgs_stream_t stream);
 

@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "stage.cuh"
 
 using namespace sixdgs;
 
@@ -12,31 +13,21 @@ namespace {
 
 // Internal workspace sections (after the public ones of sixdgs.h).
 enum {
-  WS_ZERO = 11,        // start of the region cleared by bin_sort
-  WS_ZERO_END = 12,
-  WS_COUNTERS = 13,    // uint32 tile counters of the persistent kernels
-  WS_SCAN_C = 14,      // compaction scan state
-  WS_SCAN_E = 15,      // emission scan state
-  WS_HIST = 16,        // (depth + tile passes) x 256 digit counts
-  WS_LB_DEPTH = 17,    // look-back words of the depth passes
-  WS_LB_TILE = 18,     // look-back words of the tile passes
-  WS_DEPTH_A_K = 19,
-  WS_DEPTH_A_V = 20,
-  WS_DEPTH_B_K = 21,
-  WS_DEPTH_B_V = 22,
-  WS_DUP_A_K = 23,
-  WS_DUP_A_V = 24,
-  WS_DUP_B_K = 25,
-  WS_DUP_B_V = 26,
-  WS_CHUNK_FIRST = 27, // first pair of every emission chunk
-  WS_COUNT = 28
+  WS_ZERO = 11,        // start of the region condition_project clears
+  WS_STATE = 12,       // words of the binning (kernels.cuh, BinWord)
+  WS_SCAN = 13,        // look-back words of the list scan
+  WS_TILE = 14,        // counters of every tile
+  WS_ZERO_END = 15,
+  WS_COUNTERS = 16,    // word 32: persistent blend queue
+  WS_ORDER = 18,       // tiles, longest lists first
+  WS_VIS = 19,         // visible queue of the projection (16 bytes an entry)
+  WS_DUP = 20,         // (depth, pair) of every duplicate, grouped by tile
+  WS_SORT_K = 21,      // SIXDGS_WS_SORTEDKEY
+  WS_SORT_V = 22,      // SIXDGS_WS_SORTED
+  WS_VIS_COUNT = 23    // entries of every segment of the visible queue
 };
 
 constexpr int kMaxCams = 256;
-// WS_COUNTERS words: 0 compaction, 1-4 depth passes, 8 emission, 9-12 tile
-// passes, 32 persistent blend queue, 40-44 depth-pass buffer parities
-constexpr int kDepthParityWord = 40;
-constexpr int kCamsPerUpload = 48;   // 6 KB of kernel parameters per upload
 
 int64_t align_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
@@ -52,13 +43,36 @@ int sm_count() {
   return cached[dev];
 }
 
+template <int kCams>
 struct CamUpload {
-  CamRec cams[kCamsPerUpload];
-  int32_t count;
+  CamRec cams[kCams];
+  int32_t first, count;
 };
 
-__global__ void upload_cams_kernel(CamUpload up, CamRec* dst) {
-  for (int i = threadIdx.x; i < up.count; i += blockDim.x) dst[i] = up.cams[i];
+// Camera records from the kernel parameters, and the words that the
+// projection and the binning count in set to zero (zero_quads 16-byte words;
+// grid-stride).
+template <int kCams>
+__global__ void upload_cams_kernel(const __grid_constant__ CamUpload<kCams> up, CamRec* dst, uint4* zero,
+                                   int64_t zero_quads) {
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i0 < up.count) dst[up.first + i0] = up.cams[i0];
+  for (int64_t i = i0; i < zero_quads; i += (int64_t)gridDim.x * blockDim.x) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// One launch per kCams cameras; the first also clears.
+template <int kCams, typename Make>
+void upload_cams(int n_cams, Make make, CamRec* dst, void* zero, int64_t zero_bytes, int sms, cudaStream_t stream) {
+  for (int first = 0; first < n_cams; first += kCams) {
+    CamUpload<kCams> up;
+    std::memset(&up, 0, sizeof(up));
+    up.first = first;
+    up.count = std::min(kCams, n_cams - first);
+    for (int i = 0; i < up.count; ++i) up.cams[i] = make(first + i);
+    const int64_t quads = first == 0 ? zero_bytes / 16 : 0;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((quads + 1023) / 1024, 2 * sms));
+    upload_cams_kernel<kCams><<<grid, 256, 0, stream>>>(up, dst, static_cast<uint4*>(zero), quads);
+  }
 }
 
 CamRec make_cam_rec(const sixdgs_camera& c, const sixdgs_settings& st, int32_t tile_offset,
@@ -189,9 +203,6 @@ sixdgs_status sixdgs_plan_init(int64_t n, int32_t sh_degree, const sixdgs_camera
   plan->tile_passes = (bits + 7) / 8;
 
   const int64_t np4 = align_up(n_pairs, 4);
-  const int64_t scan_tiles = (n_pairs + kScanTile - 1) / kScanTile + 1;
-  const int64_t sort_tiles_d = (n_pairs + kSortTile - 1) / kSortTile + 1;
-  const int64_t sort_tiles_t = (dup_capacity + kSortTile - 1) / kSortTile + 1;
   int64_t o = 0;
   auto take = [&](int section, int64_t bytes) {
     plan->off[section] = o;
@@ -205,28 +216,22 @@ sixdgs_status sixdgs_plan_init(int64_t n, int32_t sh_degree, const sixdgs_camera
   take(SIXDGS_WS_GRADREC, st->inference ? 0 : n_pairs * 48);
   take(SIXDGS_WS_RANGES, tiles * 8);
   take(SIXDGS_WS_NWALK, st->store_aux ? pixels * 4 : 0);
-  // cleared at the start of every bin_sort
-  plan->off[WS_ZERO] = o;
   take(SIXDGS_WS_COUNTS, 48);
   take(WS_COUNTERS, 64 * 4);
-  take(WS_SCAN_C, scan_tiles * 8);
-  take(WS_SCAN_E, scan_tiles * 8);
-  take(WS_HIST, (int64_t)(plan->depth_passes + plan->tile_passes) * 256 * 4);
-  take(WS_LB_DEPTH, (int64_t)plan->depth_passes * sort_tiles_d * 256 * 4);
-  take(WS_LB_TILE, (int64_t)plan->tile_passes * sort_tiles_t * 256 * 4);
+  // cleared by condition_project (the binning leaves its own words clean)
+  plan->off[WS_ZERO] = o;
+  take(WS_STATE, kBinWords * 4);
+  take(WS_SCAN, (tiles + kScanTile - 1) / kScanTile * 8);
+  take(WS_TILE, tiles * (int64_t)sizeof(TileCounters));
   plan->off[WS_ZERO_END] = o;
-  take(WS_DEPTH_A_K, n_pairs * 4);
-  take(WS_DEPTH_A_V, n_pairs * 4);
-  take(WS_DEPTH_B_K, n_pairs * 4);
-  take(WS_DEPTH_B_V, n_pairs * 4);
-  take(WS_DUP_A_K, dup_capacity * 4);
-  take(WS_DUP_A_V, dup_capacity * 4);
-  take(WS_DUP_B_K, dup_capacity * 4);
-  take(WS_DUP_B_V, dup_capacity * 4);
-  take(WS_CHUNK_FIRST, (dup_capacity / kEmitChunk + 2) * 4);
-  const bool odd = plan->tile_passes & 1;
-  plan->off[SIXDGS_WS_SORTED] = plan->off[odd ? WS_DUP_B_V : WS_DUP_A_V];
-  plan->off[SIXDGS_WS_SORTEDKEY] = plan->off[odd ? WS_DUP_B_K : WS_DUP_A_K];
+  take(WS_ORDER, tiles * 4);
+  take(WS_VIS, n_pairs * 16);
+  take(WS_VIS_COUNT, (n + kStageTile - 1) / kStageTile * 4);
+  take(WS_DUP, dup_capacity * 8);
+  take(WS_SORT_K, dup_capacity * 4);
+  take(WS_SORT_V, dup_capacity * 4);
+  plan->off[SIXDGS_WS_SORTED] = plan->off[WS_SORT_V];
+  plan->off[SIXDGS_WS_SORTEDKEY] = plan->off[WS_SORT_K];
   plan->ws_bytes = o;
   return SIXDGS_OK;
 }
@@ -243,19 +248,27 @@ sixdgs_status sixdgs_condition_project(const sixdgs_plan* p, const sixdgs_scene*
   CamRec* dcams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
   int32_t tile_offset = 0;
   int64_t pixel_base = 0;
-  for (int first = 0; first < p->n_cams; first += kCamsPerUpload) {
-    CamUpload up;
-    std::memset(&up, 0, sizeof(up));
-    up.count = std::min(kCamsPerUpload, p->n_cams - first);
-    for (int i = 0; i < up.count; ++i) {
-      const sixdgs_camera& c = cams[first + i];
-      up.cams[i] = make_cam_rec(c, p->settings, tile_offset, pixel_base);
-      tile_offset += up.cams[i].tiles_x * up.cams[i].tiles_y;
-      pixel_base += (int64_t)c.width * c.height;
-    }
-    upload_cams_kernel<<<1, 64, 0, stream>>>(up, dcams + first);
+  for (int i = 0; i < p->n_cams; ++i) {
+    const CamRec r = make_cam_rec(cams[i], p->settings, 0, 0);
+    tile_offset += r.tiles_x * r.tiles_y;
+    pixel_base += (int64_t)r.width * r.height;
   }
   if (tile_offset != p->total_tiles || pixel_base != p->total_pixels) return SIXDGS_ERR_INVALID_ARG;
+  tile_offset = 0;
+  pixel_base = 0;
+  auto next_cam = [&](int i) {
+    const CamRec r = make_cam_rec(cams[i], p->settings, tile_offset, pixel_base);
+    tile_offset += r.tiles_x * r.tiles_y;
+    pixel_base += (int64_t)r.width * r.height;
+    return r;
+  };
+  char* zero = static_cast<char*>(ws) + p->off[WS_ZERO];
+  const int64_t zero_bytes = p->off[WS_ZERO_END] - p->off[WS_ZERO];
+  // kernel parameters of 128 bytes a camera: the launch copies no more of
+  // them than the frame needs
+  if (p->n_cams == 1) upload_cams<1>(1, next_cam, dcams, zero, zero_bytes, sm_count(), stream);
+  else if (p->n_cams <= 8) upload_cams<8>(p->n_cams, next_cam, dcams, zero, zero_bytes, sm_count(), stream);
+  else upload_cams<48>(p->n_cams, next_cam, dcams, zero, zero_bytes, sm_count(), stream);
   ProjectArgs a;
   a.cams = dcams;
   a.n_cams = p->n_cams;
@@ -276,6 +289,9 @@ sixdgs_status sixdgs_condition_project(const sixdgs_plan* p, const sixdgs_scene*
   a.ntiles = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NTILES);
   a.rect = ws_ptr<ushort4>(ws, p, SIXDGS_WS_RECT);
   a.depth_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_DEPTHKEY);
+  a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
+  a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
+  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
   a.grad_rec = p->settings.inference ? nullptr : ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
   a.bulk = bulk_planes(p->n, {a.mu_p, a.mu_d, a.sh, a.lambda_raw, a.cond_cache,
                               a.cond_cache ? nullptr : a.l_raw, a.cond_cache ? nullptr : a.opacity_logit});
@@ -290,124 +306,27 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
   sixdgs_status e = check_ws(p, ws, ws_bytes);
   if (e != SIXDGS_OK) return e;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  const int sms = sm_count();
-  char* base = static_cast<char*>(ws);
-  if (cudaMemsetAsync(base + p->off[WS_ZERO], 0, p->off[WS_ZERO_END] - p->off[WS_ZERO], stream) != cudaSuccess)
-    return SIXDGS_ERR_CUDA;
-  uint32_t* counts = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_COUNTS);
-  uint32_t* counters = ws_ptr<uint32_t>(ws, p, WS_COUNTERS);
-  uint32_t* hist = ws_ptr<uint32_t>(ws, p, WS_HIST);
-  const int64_t budget = spin_budget(p);
-  const int64_t sort_tiles_d = (p->n_pairs + kSortTile - 1) / kSortTile + 1;
-  const int64_t sort_tiles_t = (p->dup_capacity + kSortTile - 1) / kSortTile + 1;
-
-  // 1. compaction of visible pairs + depth histograms
-  {
-    CompactArgs a;
-    a.ntiles = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NTILES);
-    a.depth_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_DEPTHKEY);
-    a.n_pairs = p->n_pairs;
-    a.keys_out = ws_ptr<uint32_t>(ws, p, WS_DEPTH_A_K);
-    a.vals_out = ws_ptr<uint32_t>(ws, p, WS_DEPTH_A_V);
-    a.n_vis_out = counts + 0;
-    a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN_C);
-    a.tile_counter = counters + 0;
-    a.hist = hist;
-    a.passes = p->depth_passes;
-    a.spin_budget = budget;
-    a.status = status_dev;
-    const int64_t tiles = (p->n_pairs + kCompactTile - 1) / kCompactTile;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms * 8));
-    launch_compact(a, grid, stream);
-  }
-  // 2. depth passes between buffers A and B; each pass records in a parity
-  // word where its output is, so that a pass whose digit is the same for
-  // every key (the high byte of depths within a factor of two) moves nothing
-  uint32_t* depth_parity = counters + kDepthParityWord;   // zeroed above: input in A
-  const int depth_grid = (int)std::max<int64_t>(1, std::min<int64_t>((p->n_pairs + kSortTile - 1) / kSortTile, (int64_t)sms * 4));
-  for (int pass = 0; pass < p->depth_passes; ++pass) {
-    OnesweepArgs a;
-    a.keys[0] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_A_K);
-    a.vals[0] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_A_V);
-    a.keys[1] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_B_K);
-    a.vals[1] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_B_V);
-    a.parity = depth_parity + pass;
-    a.n_ptr = counts + 0;
-    a.capacity = (uint32_t)p->n_pairs;
-    a.hist = hist + pass * 256;
-    a.lookback = ws_ptr<uint32_t>(ws, p, WS_LB_DEPTH) + (int64_t)pass * sort_tiles_d * 256;
-    a.tile_counter = counters + 1 + pass;
-    a.shift = 8 * pass;
-    a.spin_budget = budget;
-    a.status = status_dev;
-    launch_onesweep(a, depth_grid, stream);
-  }
-  // 3. duplicate emission in depth order + tile histograms
-  {
-    EmitArgs a;
-    a.pairs[0] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_A_V);
-    a.pairs[1] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_B_V);
-    a.depth_parity = depth_parity + p->depth_passes;
-    a.n_vis = counts + 0;
-    a.ntiles = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NTILES);
-    a.rect = ws_ptr<ushort4>(ws, p, SIXDGS_WS_RECT);
-    a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
-    a.n = p->n;
-    a.n_pairs = (uint32_t)p->n_pairs;
-    a.keys_out = ws_ptr<uint32_t>(ws, p, WS_DUP_A_K);
-    a.vals_out = ws_ptr<uint32_t>(ws, p, WS_DUP_A_V);
-    // the depth keys are not needed once the depth passes are done
-    a.dup_off[0] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_A_K);
-    a.dup_off[1] = ws_ptr<uint32_t>(ws, p, WS_DEPTH_B_K);
-    a.chunk_first = ws_ptr<uint32_t>(ws, p, WS_CHUNK_FIRST);
-    a.capacity = (uint64_t)p->dup_capacity;
-    a.k_out = counts + 1;
-    a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN_E);
-    a.tile_counter = counters + 8;
-    a.hist = hist + p->depth_passes * 256;
-    a.passes = p->tile_passes;
-    a.spin_budget = budget;
-    a.status = status_dev;
-    const int64_t tiles = (p->n_pairs + kScanTile - 1) / kScanTile;
-    const int scan_grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms * 8));
-    const int64_t chunks = (p->dup_capacity + kEmitChunk - 1) / kEmitChunk;
-    const int expand_grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, (int64_t)sms * 6));
-    launch_emit(a, scan_grid, expand_grid, stream);
-  }
-  // 4. tile passes
-  const int tile_grid = (int)std::max<int64_t>(1, std::min<int64_t>((p->dup_capacity + kSortTile - 1) / kSortTile, (int64_t)sms * 4));
-  for (int pass = 0; pass < p->tile_passes; ++pass) {
-    // fixed ping-pong: the sorted duplicates end in the buffer the plan names
-    OnesweepArgs a;
-    const bool even = (pass % 2) == 0;
-    a.keys[0] = ws_ptr<uint32_t>(ws, p, even ? WS_DUP_A_K : WS_DUP_B_K);
-    a.vals[0] = ws_ptr<uint32_t>(ws, p, even ? WS_DUP_A_V : WS_DUP_B_V);
-    a.keys[1] = ws_ptr<uint32_t>(ws, p, even ? WS_DUP_B_K : WS_DUP_A_K);
-    a.vals[1] = ws_ptr<uint32_t>(ws, p, even ? WS_DUP_B_V : WS_DUP_A_V);
-    a.parity = nullptr;
-    a.n_ptr = counts + 1;
-    a.capacity = (uint32_t)p->dup_capacity;
-    a.hist = hist + (p->depth_passes + pass) * 256;
-    a.lookback = ws_ptr<uint32_t>(ws, p, WS_LB_TILE) + (int64_t)pass * sort_tiles_t * 256;
-    a.tile_counter = counters + 9 + pass;
-    a.shift = 8 * pass;
-    a.spin_budget = budget;
-    a.status = status_dev;
-    launch_onesweep(a, tile_grid, stream);
-  }
-  // 5. tile ranges
-  if (cudaMemsetAsync(base + p->off[SIXDGS_WS_RANGES], 0, p->total_tiles * 8, stream) != cudaSuccess)
-    return SIXDGS_ERR_CUDA;
-  {
-    RangesArgs a;
-    a.keys = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTEDKEY);
-    a.k_ptr = counts + 1;
-    a.capacity = (uint32_t)p->dup_capacity;
-    a.total_tiles = (uint32_t)p->total_tiles;
-    a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((p->dup_capacity + 255) / 256, (int64_t)sms * 8));
-    launch_ranges(a, grid, stream);
-  }
+  BinArgs a;
+  a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
+  a.n = (uint32_t)p->n;
+  a.total_tiles = (uint32_t)p->total_tiles;
+  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
+  a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
+  a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
+  a.segments = (uint32_t)((p->n + kStageTile - 1) / kStageTile);
+  a.segment_size = (uint32_t)(kStageTile * p->n_cams);
+  a.state = ws_ptr<uint32_t>(ws, p, WS_STATE);
+  a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN);
+  a.order = ws_ptr<uint32_t>(ws, p, WS_ORDER);
+  a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
+  a.capacity = (uint64_t)p->dup_capacity;
+  a.dup = ws_ptr<uint64_t>(ws, p, WS_DUP);
+  a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
+  a.sorted_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTEDKEY);
+  a.counts = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_COUNTS);
+  a.spin_budget = spin_budget(p);
+  a.status = status_dev;
+  if (launch_bin(a, sm_count(), stream) != cudaSuccess) return SIXDGS_ERR_CUDA;
   return launch_status();
 }
 

@@ -5,6 +5,15 @@
 
 namespace sixdgs {
 
+// Counters of one tile, a 32-byte sector of their own: the tiles of a scene's
+// silhouette take most of the atomics, and packed counters put them on a few
+// L2 slices.
+struct __align__(32) TileCounters {
+  uint32_t count;    // duplicates, counted by the projection
+  uint32_t cursor;   // next free place of the tile's list
+  uint32_t pad[6];
+};
+
 struct ProjectArgs {
   const CamRec* cams;
   int32_t n_cams;
@@ -24,76 +33,46 @@ struct ProjectArgs {
   uint32_t* ntiles;
   ushort4* rect;
   uint32_t* depth_key;
+  uint4* vis;             // visible queue of the binning (bin.cuh)
+  uint32_t* vis_count;
+  TileCounters* tile;     // their counts are added to
   float* grad_rec;   // zeroed for every visible pair (read by the backward); null: inference plan
   int32_t bulk;      // 1: every parameter plane segment can be staged with bulk copies
   int64_t spin_budget;
   int32_t* status;
 };
 
-// Visible-pair compaction (scan of ntiles > 0) feeding the depth sort.
-struct CompactArgs {
-  const uint32_t* ntiles;
-  const uint32_t* depth_key;
-  int64_t n_pairs;
-  uint32_t* keys_out;
-  uint32_t* vals_out;
-  uint32_t* n_vis_out;
-  unsigned long long* scan_state;  // one word per scan tile
-  uint32_t* tile_counter;
-  uint32_t* hist;                  // passes x 256
-  int32_t passes;
-  int64_t spin_budget;
-  int32_t* status;
+// Words of the binning's state section (uint32).
+enum BinWord {
+  kBinClass = 0,         // tiles of every list-length class
+  kBinCursor = 64,       // next place of every class in the tile order
+  kBinTicket = 128,      // scan tile counter
+  kBinQueue = 129,       // sort work counter
+  kBinOver = 130,        // tiles with lists above 4096, 2048, 1024, 512 and 0 entries
+  kBinWords = 192
 };
 
-struct OnesweepArgs {
-  uint32_t* keys[2];       // the two key buffers; data moves from one to the other
-  uint32_t* vals[2];
-  // null: input in keys[0], output in keys[1]; else *parity is the input
-  // buffer and the pass writes its output buffer to parity[1] (an identity
-  // pass leaves the data where it is)
-  uint32_t* parity;
-  const uint32_t* n_ptr;   // element count (device)
-  uint32_t capacity;       // buffer size; counts above it are clamped
-  const uint32_t* hist;    // 256 digit counts of this pass
-  uint32_t* lookback;      // tiles x 256 status words of this pass
-  uint32_t* tile_counter;
-  int32_t shift;
-  int64_t spin_budget;
-  int32_t* status;
-};
-
-// Duplicate emission in depth order (scan of ntiles over the depth-sorted
-// visible pairs) feeding the tile sort.
-struct EmitArgs {
-  const uint32_t* pairs[2];   // depth-sorted visible pair indices: pairs[*depth_parity]
-  const uint32_t* depth_parity;
-  const uint32_t* n_vis;
-  const uint32_t* ntiles;
-  const ushort4* rect;
+// Per-tile lists from the projection's tile counts and visible queue.
+struct BinArgs {
   const CamRec* cams;
-  int64_t n;                  // Gaussians per camera
-  uint32_t n_pairs;
-  uint32_t* keys_out;         // global tile id
-  uint32_t* vals_out;         // pair index
-  uint32_t* dup_off[2];       // first output of each depth-sorted pair (n_vis): dup_off[*depth_parity]
-  uint32_t* chunk_first;      // pair owning the first output of each chunk
+  uint32_t n;                      // Gaussians per camera
+  uint32_t total_tiles;
+  TileCounters* tile;
+  const uint4* vis;                // visible queue (bin.cuh)
+  const uint32_t* vis_count;
+  uint32_t segments;               // of the queue
+  uint32_t segment_size;
+  uint32_t* state;                 // kBinWords words
+  unsigned long long* scan_state;  // one word per scan block
+  uint32_t* order;                 // tiles, longest list class first
+  uint2* ranges;
   uint64_t capacity;
-  uint32_t* k_out;            // number of duplicates (may exceed capacity)
-  unsigned long long* scan_state;
-  uint32_t* tile_counter;
-  uint32_t* hist;
-  int32_t passes;
+  uint64_t* dup;                   // (depth, pair) of every duplicate, grouped by tile
+  uint32_t* sorted;                // pair index, by (tile, depth, pair)
+  uint32_t* sorted_key;            // global tile id of the same
+  uint32_t* counts;                // the public counts section
   int64_t spin_budget;
   int32_t* status;
-};
-
-struct RangesArgs {
-  const uint32_t* keys;
-  const uint32_t* k_ptr;
-  uint32_t capacity;
-  uint32_t total_tiles;
-  uint2* ranges;
 };
 
 struct BlendArgs {
@@ -172,32 +151,14 @@ void launch_project_fwd(const ProjectArgs& a, cudaStream_t stream);
 void launch_scale_rotation(const ScaleRotationArgs& a, cudaStream_t stream);
 void launch_cond_cache(const CondCacheArgs& a, cudaStream_t stream);
 void launch_peak_probe(int kind, int64_t iters, float* out, int blocks, cudaStream_t stream);
-void launch_compact(const CompactArgs& a, int grid, cudaStream_t stream);
-void launch_onesweep(const OnesweepArgs& a, int grid, cudaStream_t stream);
-void launch_emit(const EmitArgs& a, int scan_grid, int expand_grid, cudaStream_t stream);
-void launch_ranges(const RangesArgs& a, int grid, cudaStream_t stream);
+cudaError_t launch_bin(const BinArgs& a, int sms, cudaStream_t stream);
 void launch_blend_fwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_blend_fused(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_blend_bwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_sh_bwd(const ProjectBwdArgs& a, cudaStream_t stream);
 void launch_geom_bwd(const ProjectBwdArgs& a, cudaStream_t stream);
 
-// Tile geometry of the scans and sorts (elements per block tile).
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
-// the visible-pair compaction: more items per thread (loads in flight, fewer
-// look-back steps); a multiple of 4, so its tiles never outnumber the scan
-// tiles the workspace has state for
-#ifndef SIXDGS_COMPACT_ITEMS
-#define SIXDGS_COMPACT_ITEMS 16
-#endif
-constexpr int kCompactItems = SIXDGS_COMPACT_ITEMS;
-constexpr int kCompactTile = kScanThreads * kCompactItems;
-static_assert(kCompactItems % 4 == 0 && kCompactTile >= kScanTile, "compaction tile");
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 12;
-constexpr int kSortTile = kSortThreads * kSortItems;
-constexpr int kEmitChunk = 512;    // duplicates written per expansion chunk
+// Tiles per block of the list scan.
+constexpr int kScanTile = 256;
 
 }  // namespace sixdgs

@@ -15,6 +15,7 @@
 // the two variants give bit-identical records.
 #include "common.cuh"
 #include "kernels.cuh"
+#include "bin.cuh"
 #include "cond.cuh"
 #include "mat3.cuh"
 #include "sh.cuh"
@@ -113,8 +114,7 @@ __device__ __forceinline__ M3 sym_upper(const M3& m) {
 // Per-Gaussian state the second phase reads from shared memory, written over
 // the tile's conditioning planes once a thread has read its own: A (9), the
 // upper triangles of Sigma_d^-1 and Sigma_cond (6 each: 00 01 02 11 12 22),
-// alpha, lambda.
-constexpr int kCsPlanes = 23;
+// alpha, lambda (23 planes).
 
 __device__ __forceinline__ void store_sym(float* cp, int k0, const M3& m) {
   cp[(k0 + 0) * kStageTile] = m(0, 0);
@@ -136,18 +136,44 @@ __device__ __forceinline__ M3 load_sym(const float* cp, int k0) {
   return m;
 }
 
+// Pairs of a CTA with more tiles than one thread should count alone.
+struct BigRects {
+  static constexpr int kMax = 128;
+  static constexpr uint32_t kTiles = 16;   // above: a warp counts them together
+  uint32_t count;
+  const uint4* at[kMax];
+};
+
+// Adds one pair's duplicates to the counts of its view's tiles (no result is
+// waited for).
+__device__ __forceinline__ void count_tiles(TileCounters* c, int32_t tiles_x, uint4 e, uint32_t ntiles, const uint4* vis,
+                                            BigRects& big) {
+  if (ntiles > BigRects::kTiles) {
+    const uint32_t k = atomicAdd(&big.count, 1u);
+    if (k < BigRects::kMax) {
+      big.at[k] = vis;
+      return;
+    }
+  }
+  const uint32_t x0 = e.z & 0xffffu, x1 = e.z >> 16;
+  for (uint32_t y = e.w & 0xffffu; y < e.w >> 16; ++y)
+    for (uint32_t x = x0; x < x1; ++x) atomicAdd(&c[y * (uint32_t)tiles_x + x].count, 1u);
+}
+
 // EWA projection, colour and tile rectangle of one pair that passed the
 // visibility test (section 4.4, section 4.2): writes the pair's record, depth
 // key, rect and tile count (0 when the 2D covariance, the footprint or a
-// value is degenerate).  beta(k, c): SH coefficient k of colour channel c.
+// value is degenerate), and its entry of the visible queue.  beta(k, c): SH
+// coefficient k of colour channel c.
 template <typename Beta>
 __device__ __forceinline__ void project_pair(const ProjectArgs& a, Beta beta, const float* mp,
                                              const float* md, const M3& A, const M3& Sdi, const M3& Sc, float alpha,
-                                             float lam, const CamRec& cam, int64_t pair, int K) {
+                                             float lam, const CamRec& cam, int64_t pair, int K, uint4* vis, BigRects& big) {
   const SliceView sv = slice_view(mp, md, A, Sdi, alpha, lam, cam);
   const float* t = sv.t;
   const float alpha_cond = sv.alpha_cond;
   uint32_t ntiles = 0;
+  uint4 entry = make_uint4((uint32_t)pair, 0u, 0u, 0u);
   // ---- projection (section 4.4, EWA) ----
   float iz = 1.f / t[2];
   float rx = fminf(cam.limx, fmaxf(-cam.limx, t[0] * iz));
@@ -226,9 +252,30 @@ __device__ __forceinline__ void project_pair(const ProjectArgs& a, Beta beta, co
       a.depth_key[pair] = __float_as_uint(t[2]);
       a.rect[pair] =
           make_ushort4((unsigned short)x0, (unsigned short)x1, (unsigned short)y0, (unsigned short)y1);
+      entry = vis_entry((uint32_t)pair, __float_as_uint(t[2]), (uint32_t)x0, (uint32_t)x1, (uint32_t)y0, (uint32_t)y1);
+      count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, vis, big);
     }
   }
   a.ntiles[pair] = ntiles;
+  *vis = entry;
+}
+
+// The rest of the counting: the pairs of the CTA with many tiles, a warp each.
+// Called by the whole CTA after its pairs.
+__device__ __forceinline__ void count_big(const ProjectArgs& a, const CamRec* cams, const BigRects& big) {
+  __syncthreads();
+  const uint32_t nb = min(big.count, (uint32_t)BigRects::kMax);
+  for (uint32_t i = threadIdx.x >> 5; i < nb; i += kStageTile / 32) {
+    const uint4 e = *big.at[i];
+    const CamRec& cam = cams[e.x / (uint32_t)a.n];
+    const uint32_t x0 = e.z & 0xffffu, y0 = e.w & 0xffffu, w = max((e.z >> 16) - x0, 1u);
+    const uint32_t nt = w * ((e.w >> 16) - y0);
+    TileCounters* c = a.tile + cam.tile_offset + y0 * cam.tiles_x + x0;
+    for (uint32_t o = threadIdx.x & 31u; o < nt; o += 32) {
+      const uint32_t row = rect_row(o, w);
+      atomicAdd(&c[row * cam.tiles_x + (o - row * w)].count, 1u);
+    }
+  }
 }
 
 // kStageTile Gaussians per CTA in two phases:
@@ -249,7 +296,8 @@ template <bool kCached, bool kStaged>
 __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kernel(ProjectArgs a) {
   extern __shared__ float4 s_dyn[];
   __shared__ uint64_t s_bars[2];
-  __shared__ uint32_t s_count;
+  __shared__ uint32_t s_count;   // the CTA's visible pairs
+  __shared__ BigRects s_big;
   CamRec* s_cams = reinterpret_cast<CamRec*>(s_dyn);
   float* tile = reinterpret_cast<float*>(s_cams + a.n_cams);
   const int64_t n = a.n;
@@ -259,8 +307,9 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
   float* s_cs = tile + pp.cond * kStageTile;
   uint16_t* s_queue = reinterpret_cast<uint16_t*>(tile + pp.count * kStageTile);
   for (int i = threadIdx.x; i < a.n_cams; i += blockDim.x) s_cams[i] = a.cams[i];
-  if (threadIdx.x == 0) s_count = 0;
+  if (threadIdx.x == 0) s_count = s_big.count = 0;
   const int64_t g0 = (int64_t)blockIdx.x * kStageTile;
+  uint4* vis_seg = a.vis + g0 * a.n_cams;   // this CTA's segment of the visible queue
   const int m = (int)min((int64_t)kStageTile, n - g0);
   // group 0: mu_p, mu_d, the conditioning planes and lambda (phase A);
   // group 1: the SH coefficients, in flight while phase A runs
@@ -330,52 +379,58 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
       // with the same symmetric state the queued path reads
       const M3 Sdi = sym_upper(cs.Sdi), Sc = sym_upper(cs.Sc);
       const int K = (a.sh_degree + 1) * (a.sh_degree + 1);
+      bool vis = false;
+      if (ok) {
+        const SliceView sv = slice_view(mp, md, cs.A, Sdi, cs.alpha, lam, s_cams[0]);
+        vis = (sv.alpha_cond >= kAlphaMin) && (sv.t[2] > s_cams[0].znear);
+      }
+      if (vis) {
+        const uint32_t slot = atomicAdd(&s_count, 1u);
+        project_pair(a, [&](int k, int c) { return bt[k][c]; }, mp, md, cs.A, Sdi, Sc, cs.alpha, lam, s_cams[0], g, K,
+                     vis_seg + slot, s_big);
+      } else {
+        a.ntiles[g] = 0u;
+      }
+    } else {
+      // this thread's own column of the conditioning planes is read: reuse it
+      float* cp = s_cs + tid;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) cp[k * kStageTile] = cs.A.m[k];
+      store_sym(cp, 9, cs.Sdi);
+      store_sym(cp, 15, cs.Sc);
+      cp[21 * kStageTile] = cs.alpha;
+      cp[22 * kStageTile] = lam;
+      const int lane = tid & 31;
+      const M3 Sdi = sym_upper(cs.Sdi);   // as phase B reads it back
       for (int v = 0; v < a.n_cams; ++v) {
-        const int64_t pair = (int64_t)v * n + g;
         bool vis = false;
         if (ok) {
           const SliceView sv = slice_view(mp, md, cs.A, Sdi, cs.alpha, lam, s_cams[v]);
           vis = (sv.alpha_cond >= kAlphaMin) && (sv.t[2] > s_cams[v].znear);
         }
-        if (vis) project_pair(a, [&](int k, int c) { return bt[k][c]; }, mp, md, cs.A, Sdi, Sc, cs.alpha, lam,
-                              s_cams[v], pair, K);
-        else a.ntiles[pair] = 0u;
+        if (!vis) a.ntiles[(int64_t)v * n + g] = 0u;
+        // warp-aggregated append to the queue
+        const uint32_t active = __activemask();
+        const uint32_t bal = __ballot_sync(active, vis);
+        uint32_t base = 0;
+        const int leader = __ffs(active) - 1;
+        if (lane == leader && bal) base = atomicAdd(&s_count, (uint32_t)__popc(bal));
+        base = __shfl_sync(active, base, leader);
+        if (vis) s_queue[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(tid | (v << 7));
       }
-      return;
-    }
-    // this thread's own column of the conditioning planes is read: reuse it
-    float* cp = s_cs + tid;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) cp[k * kStageTile] = cs.A.m[k];
-    store_sym(cp, 9, cs.Sdi);
-    store_sym(cp, 15, cs.Sc);
-    cp[21 * kStageTile] = cs.alpha;
-    cp[22 * kStageTile] = lam;
-    const int lane = tid & 31;
-    const M3 Sdi = sym_upper(cs.Sdi);   // as phase B reads it back
-    for (int v = 0; v < a.n_cams; ++v) {
-      bool vis = false;
-      if (ok) {
-        const SliceView sv = slice_view(mp, md, cs.A, Sdi, cs.alpha, lam, s_cams[v]);
-        vis = (sv.alpha_cond >= kAlphaMin) && (sv.t[2] > s_cams[v].znear);
-      }
-      if (!vis) a.ntiles[(int64_t)v * n + g] = 0u;
-      // warp-aggregated append to the queue
-      const uint32_t active = __activemask();
-      const uint32_t bal = __ballot_sync(active, vis);
-      uint32_t base = 0;
-      const int leader = __ffs(active) - 1;
-      if (lane == leader && bal) base = atomicAdd(&s_count, (uint32_t)__popc(bal));
-      base = __shfl_sync(active, base, leader);
-      if (vis) s_queue[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(tid | (v << 7));
     }
   }
-  if (!kStaged) return;
+  if (!kStaged) {
+    count_big(a, s_cams, s_big);
+    if (tid == 0) a.vis_count[blockIdx.x] = s_count;
+    return;
+  }
   if (!stage_wait(s_bars, 1, bulk, a.spin_budget)) raise_status(a.status, SIXDGS_ERR_TIMEOUT);
   __syncthreads();
 
   // ---- phase B: one visible pair per thread ----
   const uint32_t count = s_count;
+  if (tid == 0) a.vis_count[blockIdx.x] = count;
   const int K = (a.sh_degree + 1) * (a.sh_degree + 1);
   for (uint32_t qi = tid; qi < count; qi += kStageTile) {
     const uint32_t e = s_queue[qi];
@@ -393,8 +448,9 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
     const float md[3] = {P(pp.mu_d), P(pp.mu_d + 1), P(pp.mu_d + 2)};
     const CamRec& cam = s_cams[v];
     project_pair(a, [&](int k, int c) { return P(pp.sh + k * 3 + c); }, mp, md, A, Sdi, Sc, cp[21 * kStageTile],
-                 cp[22 * kStageTile], cam, pair, K);
+                 cp[22 * kStageTile], cam, pair, K, vis_seg + qi, s_big);
   }
+  count_big(a, s_cams, s_big);
 }
 
 template <bool kCached, bool kStaged>
@@ -405,7 +461,7 @@ static void launch_project(const ProjectArgs& a, cudaStream_t stream) {
                       (kStaged ? (size_t)pp.count * kStageTile * sizeof(float) +
                                      (size_t)kStageTile * a.n_cams * sizeof(uint16_t)
                                : 0);
-  if (smem > 48 * 1024)
+  if (smem > 40 * 1024)   // the static shared memory counts towards the 48 KB as well
     cudaFuncSetAttribute(project_fwd_kernel<kCached, kStaged>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   project_fwd_kernel<kCached, kStaged><<<(unsigned)blocks, kStageTile, smem, stream>>>(a);
 }

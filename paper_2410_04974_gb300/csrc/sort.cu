@@ -1,28 +1,44 @@
-// Stage 2: binning and sorting of (view, Gaussian) pairs into per-tile lists
-// ordered by depth (the 3DGS duplicate/sort step kept by 6DGS section 4.4).
+// Stage 2: per-tile lists of (view, Gaussian) pairs ordered by depth (the
+// 3DGS duplicate/sort step kept by 6DGS section 4.4).
 //
-// The composite key (global tile, depth, Gaussian id) is sorted LSD-first:
-//   1. compact_kernel   -- visible pairs in (view, id) order, with the depth
-//                          digits' histograms (single-pass scan, decoupled
-//                          look-back);
-//   2. onesweep passes  -- stable 8-bit digit passes over the depth key;
-//   3. emit_kernel      -- duplicate each pair once per touched tile, in depth
-//                          order, with the tile digits' histograms;
-//   4. onesweep passes  -- stable passes over the global tile id;
-//   5. ranges_kernel    -- [start, end) of every tile's list.
-// Because every pass is stable and the depth passes run before duplication,
-// the result equals one LSD sort of the full key while the depth passes
-// touch each visible pair once instead of once per tile.
+// The composite order (global tile, depth, Gaussian id) is built tile first:
+//   1. the projection counts every tile's duplicates and queues its visible
+//      pairs (project.cu);
+//   2. bin_scan_kernel    -- exclusive scan of the counts: every tile's range
+//                            (single pass, decoupled look-back) and the
+//                            number of tiles of every list-length class;
+//   3. bin_scatter_kernel -- every duplicate (depth, pair) to the next free
+//                            place of its tile's range, and the order of the
+//                            tiles, longest lists first;
+//   4. bin_sort_kernel    -- every tile's entries sorted on chip by (depth,
+//                            pair).
+// The entries of a tile are distinct and all of one view, whose pair index
+// grows with the Gaussian id, so sorting (depth, pair) gives the stable
+// (depth, id) order whatever order the scatter's atomics left.
 //
-// The per-digit passes follow the single-pass "onesweep" design (Adinets and
-// Merrill, 2022): a tile's digit counts are published with decoupled
-// look-back (Merrill and Garland, 2016) so each pass reads and writes the
-// data once.  Every spin is bounded by a clock budget; on expiry the kernel
-// reports SIXDGS_ERR_TIMEOUT and carries on with in-bounds writes only.
+// Why not radix passes over all duplicates: those moved every duplicate once
+// per digit and needed a dozen dependent launches (compaction, four depth
+// passes, two scans and an expansion, two or three tile passes, ranges).
+// Tile first, a duplicate is written once, read once and written sorted, in
+// three launches.  Measured (sum of the kernels; radix -> tile first):
+//   300k / 8 x 800^2 (2.5 M duplicates)     206 -> 85 us
+//   2M / 4 x 1920x1080 (3.4 M)              236 -> 96 us
+//   500k / 64 mixed views (29 M)           1907 -> 1215 us
+//   one view, 54 k duplicates                74 -> 28 us
+// (the projection, which counts the tiles, takes 83 -> 99 us at 300k).
+#include <algorithm>
+
+#include "bin.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
+#include "stage.cuh"
 
 namespace sixdgs {
+
+constexpr int kBinThreads = 256;
+constexpr int kBinWarps = kBinThreads / 32;
+constexpr int kCluster = 8;               // CTAs that share one very long list
+constexpr int kClasses = 64;
 
 constexpr unsigned long long kScanAgg = 1ull << 62;
 constexpr unsigned long long kScanInc = 2ull << 62;
@@ -67,9 +83,11 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t& total,
   return r;
 }
 
-// Decoupled look-back over 64-bit scan state, run by one full warp.
-// Publishes this tile's aggregate, waits for the predecessors and
-// publishes the inclusive prefix.  Returns the exclusive prefix.
+// Decoupled look-back over 64-bit scan state (Merrill and Garland, 2016), run
+// by one full warp.  Publishes this block's aggregate, waits for the
+// predecessors and publishes the inclusive prefix.  Returns the exclusive
+// prefix.  The wait is bounded by a clock budget; on expiry the status word
+// gets SIXDGS_ERR_TIMEOUT and the callers carry on with clamped ranges.
 __device__ unsigned long long scan_lookback(unsigned long long* state, uint32_t tile,
                                             unsigned long long block_total, int64_t budget,
                                             int32_t* status) {
@@ -113,436 +131,611 @@ __device__ unsigned long long scan_lookback(unsigned long long* state, uint32_t 
   return excl;
 }
 
+// Class of a list length: 0 for an empty list, else four classes per power of
+// two of len - 1: lists of up to 2^p entries (p >= 1) have classes up to 4 p,
+// longer ones classes from 4 p + 1 (the last class takes the rest).
+__device__ __forceinline__ uint32_t length_class(uint32_t len) {
+  if (len == 0u) return 0u;
+  const uint32_t m = len - 1u;
+  const uint32_t l = m ? 31u - __clz(m) : 0u;
+  const uint32_t frac = l >= 2u ? (m >> (l - 2u)) & 3u : (l == 1u ? (m & 1u) * 2u : 0u);
+  return min(1u + 4u * l + frac, (uint32_t)kClasses - 1u);
+}
+constexpr int kBinLevels = 4;   // 4096, 2048, 1024, 512 entries: the sizes of the sorting teams
+
+// Adds this block's tiles to per-class counters in shared memory; returns the
+// tile's rank within its class and block.  Called by the whole block, tiles
+// past the end with valid = false.  Empty lists (most of a frame that shows
+// an object) are counted by ballot, not by colliding atomics.
+__device__ __forceinline__ uint32_t count_class(uint32_t cls, bool valid, uint32_t* s_class) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t empty = __ballot_sync(0xffffffffu, valid && cls == 0u);
+  uint32_t base = 0;
+  if (lane == 0 && empty) base = atomicAdd(&s_class[0], (uint32_t)__popc(empty));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (!valid) return 0u;
+  if (cls == 0u) return base + __popc(empty & ((1u << lane) - 1u));
+  return atomicAdd(&s_class[cls], 1u);
+}
+
 // --------------------------------------------------------------------------
-// 1. Visible-pair compaction + depth-digit histograms
+// Ranges of the tiles' lists
 // --------------------------------------------------------------------------
-__global__ void __launch_bounds__(kScanThreads) compact_kernel(CompactArgs a) {
-  __shared__ uint32_t s_warp[kScanThreads / 32 + 1];
-  __shared__ uint32_t s_hist[4 * 256];
-  __shared__ uint32_t s_tile;
+// Latency-bound (T x 4 bytes in, T x 12 out).  One tile per thread, so that a
+// frame of a few thousand tiles is spread over several SMs.
+__global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
+  __shared__ uint32_t s_warp[kBinWarps + 1];
+  __shared__ uint32_t s_class[kClasses];
+  __shared__ uint32_t s_block;
   __shared__ unsigned long long s_excl;
-  for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_hist[i] = 0;
-  const uint64_t n = (uint64_t)a.n_pairs;
-  const uint32_t num_tiles = (uint32_t)((n + kCompactTile - 1) / kCompactTile);
-  while (true) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_tile = atomicAdd(a.tile_counter, 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= num_tiles) break;
-    const uint64_t base = (uint64_t)tile * kCompactTile + (uint64_t)threadIdx.x * kCompactItems;
-    uint32_t cnt[kCompactItems];
-    if (base + kCompactItems <= n) {
-#pragma unroll
-      for (int k = 0; k < kCompactItems; k += 4) {
-        const uint4 q = *reinterpret_cast<const uint4*>(a.ntiles + base + k);
-        cnt[k] = q.x; cnt[k + 1] = q.y; cnt[k + 2] = q.z; cnt[k + 3] = q.w;
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < kCompactItems; ++k) cnt[k] = (base + k < n) ? a.ntiles[base + k] : 0u;
-    }
-    // the depth keys of all items, loaded together (an invisible pair's key is
-    // not used)
-    uint32_t key[kCompactItems];
-#pragma unroll
-    for (int k = 0; k < kCompactItems; ++k) key[k] = (base + k < n) ? a.depth_key[base + k] : 0u;
-    uint32_t vis = 0;
-#pragma unroll
-    for (int k = 0; k < kCompactItems; ++k) vis += cnt[k] > 0u;
-    uint32_t total;
-    uint32_t excl = block_excl_scan<kScanThreads>(vis, total, s_warp);
-    if (threadIdx.x < 32) {
-      unsigned long long e = scan_lookback(a.scan_state, tile, total, a.spin_budget, a.status);
-      if (threadIdx.x == 0) s_excl = e;
-    }
-    __syncthreads();
-    uint64_t off = s_excl + excl;
-#pragma unroll
-    for (int k = 0; k < kCompactItems; ++k) {
-      if (cnt[k] > 0u) {
-        if (off < n) {
-          a.keys_out[off] = key[k];
-          a.vals_out[off] = (uint32_t)(base + k);
-        }
-        ++off;
-        for (int p = 0; p < a.passes; ++p) atomicAdd(&s_hist[p * 256 + ((key[k] >> (8 * p)) & 255u)], 1u);
-      }
-    }
-    if (tile == num_tiles - 1 && threadIdx.x == 0) *a.n_vis_out = (uint32_t)(s_excl + total);
-  }
+  const int tid = threadIdx.x;
+  if (tid == 0) s_block = atomicAdd(&a.state[kBinTicket], 1u);
+  if (tid < kClasses) s_class[tid] = 0u;
   __syncthreads();
-  for (int i = threadIdx.x; i < a.passes * 256; i += kScanThreads)
-    if (s_hist[i]) atomicAdd(&a.hist[i], s_hist[i]);
+  const uint32_t block = s_block;
+  const uint32_t t = block * kScanTile + tid;
+  const bool valid = t < a.total_tiles;
+  const uint32_t cnt = valid ? a.tile[t].count : 0u;
+  uint32_t total;
+  const uint32_t excl = block_excl_scan<kBinThreads>(cnt, total, s_warp);
+  if (tid < 32) {
+    const unsigned long long e = scan_lookback(a.scan_state, block, total, a.spin_budget, a.status);
+    if (tid == 0) s_excl = e;
+  }
+  // counters of the kernels that follow (every block has its own ticket, so
+  // exactly one block is block 0); the pair counters behind the first two
+  // public words are the blend's
+  if (block == 0 && tid < 10) a.counts[2 + tid] = 0u;
+  if (block == 0 && tid == 10) a.counts[0] = 0u;
+  if (block == 0 && tid == 11) a.state[kBinQueue] = 0u;
+  __syncthreads();
+  // lists beyond the duplicate capacity are cut there (and reported below)
+  const unsigned long long off = s_excl + excl;
+  const uint32_t start = (uint32_t)min(off, (unsigned long long)a.capacity);
+  const uint32_t end = (uint32_t)min(off + cnt, (unsigned long long)a.capacity);
+  if (valid) {
+    a.tile[t].cursor = start;
+    a.ranges[t] = end > start ? make_uint2(start, end) : make_uint2(0u, 0u);
+  }
+  count_class(length_class(end - start), valid, s_class);
+  __syncthreads();
+  if (tid < kClasses && s_class[tid]) atomicAdd(&a.state[kBinClass + tid], s_class[tid]);
+  if (block == gridDim.x - 1 && tid == 0) {
+    const unsigned long long k = s_excl + total;
+    a.counts[1] = (uint32_t)min(k, 0xffffffffull);
+    if (k > a.capacity) raise_status(a.status, SIXDGS_ERR_CAPACITY);
+  }
 }
 
 // --------------------------------------------------------------------------
-// 2/4. One stable 8-bit digit pass (onesweep)
+// Duplicates to their tiles, and the tile order
 // --------------------------------------------------------------------------
-// 80 registers, 3 CTAs per SM (2 at the unbounded 128): bin_sort 0.327 -> 0.320 ms
-// on the 300k / 8 x 800^2 frame.
-__global__ void __launch_bounds__(kSortThreads, 3) onesweep_kernel(OnesweepArgs a) {
-  constexpr int WARPS = kSortThreads / 32;
-  static_assert(kSortThreads == 256, "one thread per digit");
-  __shared__ uint32_t s_whist[WARPS][256];
-  __shared__ uint32_t s_keys[kSortTile];
-  __shared__ uint32_t s_vals[kSortTile];
-  __shared__ uint32_t s_dstart[256];
-  __shared__ uint32_t s_glob[256];
-  __shared__ uint32_t s_warp[WARPS + 1];
-  __shared__ uint32_t s_tile;
+// A CTA takes a segment of the visible queue, 256 entries at a time, and
+// spreads their duplicates over its threads whatever the rectangles' sizes:
+// duplicate o goes to thread o % 128, which finds its entry by a binary search
+// of the entries' prefix sums in shared memory.  Bound by L2 requests (one
+// atomic and one 8-byte store a duplicate, at random places), so the atomics
+// are issued by full warps, kScatterBatch a thread in flight.  (A thread that
+// walks its own entry's duplicates needs neither search nor barrier, but more
+// and emptier atomic instructions: 60 instead of 51 us at 300k / 8 x 800^2.)
+constexpr int kScatterThreads = 128;
+constexpr int kScatterEntries = 2 * kScatterThreads;
+constexpr int kScatterBatch = 4;
+__global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a) {
+  constexpr int kWarps = kScatterThreads / 32;
+  __shared__ uint32_t s_class[kClasses], s_base[kClasses], s_longer[kClasses];
+  __shared__ uint32_t s_warp[kWarps + 1];
+  __shared__ uint32_t s_incl[kScatterEntries];   // inclusive prefix of the entries' tile counts
+  __shared__ uint4 s_entry[kScatterEntries];     // (first tile, tiles_x << 16 | width, pair, depth)
+  __shared__ uint32_t s_vis;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // input buffer: fixed (parity == null) or as the previous pass left it
-  const uint32_t par = a.parity ? *a.parity : 0u;
-  // (selects, not an index: a runtime index into the parameter arrays would
-  // copy them to local memory)
-  const uint32_t* keys_in = par ? a.keys[1] : a.keys[0];
-  const uint32_t* vals_in = par ? a.vals[1] : a.vals[0];
-  uint32_t* keys_out = par ? a.keys[0] : a.keys[1];
-  uint32_t* vals_out = par ? a.vals[0] : a.vals[1];
-  const uint32_t n = min(*a.n_ptr, a.capacity);
-  const uint32_t num_tiles = (n + kSortTile - 1) / kSortTile;
-  // exclusive digit offsets of the whole pass (thread tid owns digit tid)
-  uint32_t htot;
-  const uint32_t my_count = a.hist[tid];
-  const uint32_t hist_excl = block_excl_scan<kSortThreads>(my_count, htot, s_warp);
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  // Every key has the same digit: the stable pass is the identity.  With a
-  // parity word the data stays where it is (the next reader is told so);
-  // otherwise the tiles are copied through without ranking or look-back.
-  if (__syncthreads_or(n > 0u && my_count == n)) {
-    if (a.parity) {
-      if (blockIdx.x == 0 && tid == 0) a.parity[1] = par;
-      return;
-    }
-    for (uint32_t i = blockIdx.x * kSortThreads + tid; i < n; i += gridDim.x * kSortThreads) {
-      keys_out[i] = keys_in[i];
-      vals_out[i] = vals_in[i];
-    }
-    return;
-  }
-  if (a.parity && blockIdx.x == 0 && tid == 0) a.parity[1] = par ^ 1u;
-  while (true) {
-    __syncthreads();
-    if (tid == 0) s_tile = atomicAdd(a.tile_counter, 1u);
-#pragma unroll
-    for (int w = 0; w < WARPS; ++w) s_whist[w][tid] = 0u;
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= num_tiles) break;
-    const uint32_t base = tile * kSortTile;
-    const uint32_t wbase = base + warp * (32 * kSortItems);
-    uint32_t key[kSortItems], val[kSortItems], rank[kSortItems];
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-      uint32_t idx = wbase + j * 32 + lane;
-      bool valid = idx < n;
-      key[j] = valid ? keys_in[idx] : 0xffffffffu;
-      val[j] = valid ? vals_in[idx] : 0u;
-    }
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-      uint32_t idx = wbase + j * 32 + lane;
-      uint32_t d = idx < n ? (key[j] >> a.shift) & 255u : 256u;
-      // lanes with the same digit, from one ballot per digit bit
-      uint32_t peers = __ballot_sync(0xffffffffu, d < 256u);
-      if (d >= 256u) peers = ~peers;
-#pragma unroll
-      for (int bit = 0; bit < 8; ++bit) {
-        const uint32_t set = (d >> bit) & 1u;
-        const uint32_t bal = __ballot_sync(0xffffffffu, set);
-        peers &= set ? bal : ~bal;
-      }
-      uint32_t before = d < 256u ? s_whist[warp][d] : 0u;
-      __syncwarp();
-      if (d < 256u && lane == (uint32_t)(__ffs(peers) - 1)) s_whist[warp][d] = before + __popc(peers);
-      __syncwarp();
-      rank[j] = before + __popc(peers & lt_mask);
-    }
-    __syncthreads();
-    // per digit: exclusive prefix over warps, block count
-    uint32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < WARPS; ++w) {
-      uint32_t c = s_whist[w][tid];
-      s_whist[w][tid] = run;
-      run += c;
-    }
-    const uint32_t cnt = run;
-    uint32_t btot;
-    const uint32_t dstart = block_excl_scan<kSortThreads>(cnt, btot, s_warp);
-    s_dstart[tid] = dstart;
-    // decoupled look-back for digit tid
-    uint32_t* lb = a.lookback;
-    uint32_t excl = 0;
-    if (tile == 0) {
-      st_volatile(&lb[tid], kFlagInc | cnt);
-    } else {
-      st_volatile(&lb[tile * 256 + tid], kFlagAgg | cnt);
-      // Walk back over the predecessors' words for this digit, kWindow at a
-      // time (all loads in flight together), summing aggregates up to the
-      // first inclusive prefix; a word not yet published is waited for.
-      constexpr int kWindow = 8;
-      long long p = (long long)tile - 1;
-      const long long t0 = clock64();
-      while (p >= 0) {
-        uint32_t w[kWindow];
-#pragma unroll
-        for (int i = 0; i < kWindow; ++i) w[i] = (p - i >= 0) ? ld_volatile(&lb[(p - i) * 256 + tid]) : kFlagInc;
-        int used = 0;
-        bool found = false, waiting = false;
-#pragma unroll
-        for (int i = 0; i < kWindow; ++i) {
-          if (found || waiting) continue;
-          const uint32_t f = w[i] & kFlagMask;
-          if (f == 0u) {
-            waiting = true;
-            continue;
-          }
-          excl += w[i] & kValMask;
-          ++used;
-          found = f == kFlagInc;
-        }
-        if (found) break;
-        p -= used;
-        if (waiting && clock64() - t0 > a.spin_budget) {
-          raise_status(a.status, SIXDGS_ERR_TIMEOUT);
-          break;
-        }
-      }
-      st_volatile(&lb[tile * 256 + tid], kFlagInc | ((excl + cnt) & kValMask));
-    }
-    s_glob[tid] = hist_excl + excl - dstart;
-    __syncthreads();
-    // local scatter into digit order
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-      uint32_t idx = wbase + j * 32 + lane;
-      if (idx < n) {
-        uint32_t d = (key[j] >> a.shift) & 255u;
-        uint32_t pos = s_dstart[d] + s_whist[warp][d] + rank[j];
-        s_keys[pos] = key[j];
-        s_vals[pos] = val[j];
-      }
-    }
-    __syncthreads();
-    const uint32_t tile_n = min((uint32_t)kSortTile, n - base);
-    for (uint32_t i = tid; i < tile_n; i += kSortThreads) {
-      uint32_t k = s_keys[i];
-      uint32_t out = s_glob[(k >> a.shift) & 255u] + i;
-      if (out < n) {
-        keys_out[out] = k;
-        vals_out[out] = s_vals[i];
-      }
-    }
-  }
-}
-
-// --------------------------------------------------------------------------
-// 3. Duplicate emission in depth order + tile-digit histograms
-//
-// Two kernels, so that the work is spread over the duplicates, not over the
-// visible pairs (a few large Gaussians can own most of the duplicates):
-//   emit_scan_kernel   -- exclusive scan of the depth-sorted pairs' tile
-//                         counts (decoupled look-back): every pair's first
-//                         output, the pair owning the first output of every
-//                         chunk of kEmitChunk outputs, and the total K;
-//   emit_expand_kernel -- one chunk per CTA at a time: the chunk's pairs
-//                         (at most kEmitChunk + 1, since every visible pair
-//                         has at least one tile) are staged in shared
-//                         memory, each marks the chunk position where its
-//                         outputs start, a prefix maximum over the positions
-//                         gives every output its pair, and consecutive
-//                         threads write consecutive duplicates, so stores are
-//                         coalesced.
-// --------------------------------------------------------------------------
-__global__ void __launch_bounds__(kScanThreads) emit_scan_kernel(EmitArgs a) {
-  __shared__ uint32_t s_warp[kScanThreads / 32 + 1];
-  __shared__ uint32_t s_tile;
-  __shared__ unsigned long long s_excl;
-  const uint32_t n_vis = *a.n_vis;
-  const uint32_t num_tiles = (n_vis + kScanTile - 1) / kScanTile;
-  const unsigned long long cap = a.capacity;
-  const uint32_t par = *a.depth_parity;
-  const uint32_t* pairs = par ? a.pairs[1] : a.pairs[0];
-  uint32_t* dup_off = par ? a.dup_off[1] : a.dup_off[0];
-  while (true) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_tile = atomicAdd(a.tile_counter, 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    if (tile >= num_tiles) break;
-    const uint32_t base = tile * kScanTile + threadIdx.x * kScanItems;
-    // all pair indices first, then all their tile counts (two rounds of
-    // loads in flight instead of a dependent pair per item)
-    uint32_t cnt[kScanItems];
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) cnt[k] = base + k < n_vis ? pairs[base + k] : 0xffffffffu;
-    uint32_t sum = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-      cnt[k] = cnt[k] < a.n_pairs ? a.ntiles[cnt[k]] : 0u;
-      sum += cnt[k];
-    }
-    uint32_t total;
-    const uint32_t run = block_excl_scan<kScanThreads>(sum, total, s_warp);
-    if (threadIdx.x < 32) {
-      unsigned long long e = scan_lookback(a.scan_state, tile, total, a.spin_budget, a.status);
-      if (threadIdx.x == 0) s_excl = e;
-    }
-    __syncthreads();
-    unsigned long long off = s_excl + run;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-      if (base + k < n_vis) {
-        dup_off[base + k] = (uint32_t)min(off, 0xffffffffull);
-        // chunk boundaries b in [off, off + cnt) below the capacity
-        const unsigned long long end = min(off + cnt[k], cap);
-        for (unsigned long long b = (off + kEmitChunk - 1) / kEmitChunk * kEmitChunk; b < end; b += kEmitChunk)
-          a.chunk_first[b / kEmitChunk] = base + k;
-      }
-      off += cnt[k];
-    }
-    if (tile == num_tiles - 1 && threadIdx.x == 0) {
-      const unsigned long long k_total = s_excl + total;
-      *a.k_out = (uint32_t)min(k_total, 0xffffffffull);
-      if (k_total > cap) raise_status(a.status, SIXDGS_ERR_CAPACITY);
-    }
-  }
-}
-
-// row = local / w for the small integers of a tile rectangle: a float
-// estimate corrected to the exact quotient.
-// (64-bit, so that the correction terminates for any 32-bit input; w >= 1).
-__device__ __forceinline__ uint32_t rect_row(uint32_t local, uint32_t w) {
-  uint64_t row = (uint64_t)__fdividef((float)local, (float)w);
-  while (row > 0u && row * w > local) --row;
-  while ((row + 1u) * w <= local) ++row;
-  return (uint32_t)row;
-}
-
-__global__ void __launch_bounds__(kScanThreads) emit_expand_kernel(EmitArgs a) {
-  constexpr int kMaxPairs = kEmitChunk + 1;
-  __shared__ uint32_t s_start[kMaxPairs];      // first output of each staged pair
-  __shared__ uint32_t s_pair[kMaxPairs];
-  __shared__ uint32_t s_base[kMaxPairs];       // key of the pair's top-left tile
-  __shared__ uint32_t s_shape[kMaxPairs];      // rect width | tiles_x << 16
-  __shared__ uint32_t s_owner[kEmitChunk];     // staged pair of every output of the chunk
-  __shared__ uint32_t s_wmax[kScanThreads / 32];
-  __shared__ uint32_t s_hist[4 * 256];
-  static_assert(kEmitChunk == 2 * kScanThreads, "two outputs per thread in the owner scan");
-  for (int i = threadIdx.x; i < 4 * 256; i += kScanThreads) s_hist[i] = 0;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t n_vis = *a.n_vis;
-  const uint32_t k_all = (uint32_t)min((unsigned long long)*a.k_out, (unsigned long long)a.capacity);
-  const uint32_t n_chunks = n_vis ? (k_all + kEmitChunk - 1) / kEmitChunk : 0u;
-  const uint32_t par = *a.depth_parity;
-  const uint32_t* pairs = par ? a.pairs[1] : a.pairs[0];
-  const uint32_t* dup_off = par ? a.dup_off[1] : a.dup_off[0];
-  for (uint32_t c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-    const uint32_t o0 = c * kEmitChunk;
-    const uint32_t o1 = min(k_all, o0 + kEmitChunk);
-    // Every visible pair owns at least one output, so a chunk spans at most
-    // kMaxPairs pairs.  The clamps keep every index in bounds even if the
-    // scan gave up on a look-back wait (then the status word already
-    // reports the timeout).
-    const uint32_t e0 = min(a.chunk_first[c], n_vis - 1);
-    uint32_t e1 = (c + 1 < n_chunks) ? a.chunk_first[c + 1] : n_vis - 1;
-    e1 = max(min(e1, n_vis - 1), e0);
-    const int m = (int)min(e1 - e0 + 1u, (uint32_t)kMaxPairs);
-    __syncthreads();
-    for (int i = threadIdx.x; i < kEmitChunk; i += kScanThreads) s_owner[i] = 0u;
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += kScanThreads) {
-      const uint32_t e = e0 + i;
-      const uint32_t p = pairs[e];
-      const uint32_t st = dup_off[e];
-      s_start[i] = st;
-      s_pair[i] = p;
-      // a pair's outputs start at most once in the chunk (every visible pair
-      // has at least one), so each position is marked by at most one pair
-      const int64_t lp = (int64_t)st - (int64_t)o0;
-      if (lp >= 0 && lp < kEmitChunk) s_owner[lp] = (uint32_t)i;
-      uint32_t base = 0, shape = 1;
-      if (p < a.n_pairs) {
-        const CamRec& cam = a.cams[p / (uint32_t)a.n];
-        const ushort4 r = a.rect[p];
-        base = (uint32_t)cam.tile_offset + (uint32_t)r.z * (uint32_t)cam.tiles_x + r.x;
-        shape = max((uint32_t)(r.y - r.x), 1u) | ((uint32_t)cam.tiles_x << 16);
-      }
-      s_base[i] = base;
-      s_shape[i] = shape;
-    }
-    __syncthreads();
-    // The owner of output o is the last staged pair whose outputs start at
-    // or before o: an inclusive prefix maximum of the marks (unmarked
-    // positions hold 0, the chunk's first pair).  Thread t scans positions
-    // 2t and 2t + 1.
-    {
-      const uint32_t m0 = s_owner[2 * threadIdx.x];
-      const uint32_t m1 = max(m0, s_owner[2 * threadIdx.x + 1]);
-      uint32_t x = m1;
+  if (tid == 0) s_vis = 0u;
+  const uint32_t blocks = (a.total_tiles + kScatterThreads - 1) / kScatterThreads;
+  if (blockIdx.x < blocks) {
+    // tile order: longest class first, any order within a class (it decides
+    // when a tile is worked on, never a result)
+    if (warp == 0) {   // tiles of longer classes: a suffix sum over the 64 classes
+      const uint32_t c0 = a.state[kBinClass + lane], c1 = a.state[kBinClass + 32 + lane];
+      uint32_t x0 = c0, x1 = c1;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x = max(x, y);
+        const uint32_t y0 = __shfl_down_sync(0xffffffffu, x0, o), y1 = __shfl_down_sync(0xffffffffu, x1, o);
+        if (lane + o < 32) {
+          x0 += y0;
+          x1 += y1;
+        }
       }
-      if (lane == 31) s_wmax[warp] = x;
-      uint32_t before = __shfl_up_sync(0xffffffffu, x, 1);
-      if (lane == 0) before = 0u;
-      __syncthreads();
-      for (int w = 0; w < warp; ++w) before = max(before, s_wmax[w]);
-      s_owner[2 * threadIdx.x] = max(before, m0);
-      s_owner[2 * threadIdx.x + 1] = max(before, m1);
+      const uint32_t high = __shfl_sync(0xffffffffu, x1, 0);
+      s_longer[lane] = x0 - c0 + high;
+      s_longer[32 + lane] = x1 - c1;
     }
     __syncthreads();
-    for (uint32_t o1r = o0; o1r < o1; o1r += kScanThreads) {
-      const uint32_t o = o1r + threadIdx.x;
-      uint32_t key = 0xffffffffu;
-      if (o < o1) {
-        const int lo = (int)min(s_owner[o - o0], (uint32_t)(m - 1));
-        const uint32_t local = o - s_start[lo];
-        const uint32_t shape = s_shape[lo];
-        const uint32_t w = shape & 0xffffu, tiles_x = shape >> 16;
-        const uint32_t row = rect_row(local, w);
-        key = s_base[lo] + row * tiles_x + (local - row * w);
-        a.keys_out[o] = key;
-        a.vals_out[o] = s_pair[lo];
+    if (blockIdx.x == 0 && tid <= kBinLevels) {
+      // tiles with lists above the sort's limits: those of the classes beyond
+      const uint32_t limit_class = tid < kBinLevels ? 4u * (12u - (uint32_t)tid) : 0u;
+      a.state[kBinOver + tid] = s_longer[limit_class];
+    }
+    for (uint32_t b = blockIdx.x; b < blocks; b += gridDim.x) {
+      if (tid < kClasses) s_class[tid] = 0u;
+      __syncthreads();
+      const uint32_t t = b * kScatterThreads + tid;
+      const bool valid = t < a.total_tiles;
+      const uint2 r = valid ? a.ranges[t] : make_uint2(0u, 0u);
+      const uint32_t cls = length_class(r.y - r.x);
+      const uint32_t rank = count_class(cls, valid, s_class);
+      __syncthreads();
+      if (tid < kClasses && s_class[tid])
+        s_base[tid] = s_longer[tid] + atomicAdd(&a.state[kBinCursor + tid], s_class[tid]);
+      __syncthreads();
+      if (valid) {
+        const uint32_t at = s_base[cls] + rank;
+        if (at < a.total_tiles) a.order[at] = t;
       }
-      if (key != 0xffffffffu)
-        for (int q = 0; q < a.passes; ++q) atomicAdd(&s_hist[q * 256 + ((key >> (8 * q)) & 255u)], 1u);
     }
   }
+  // the scan is over: its words are clean for the next call
+  const uint32_t scan_blocks = (a.total_tiles + kScanTile - 1) / kScanTile;
+  for (uint32_t i = blockIdx.x * kScatterThreads + tid; i < scan_blocks; i += gridDim.x * kScatterThreads)
+    a.scan_state[i] = 0ull;
+  if (blockIdx.x == 0 && tid == 0) a.state[kBinTicket] = 0u;
+
+  uint32_t visible = 0;
+  for (uint32_t seg = blockIdx.x; seg < a.segments; seg += gridDim.x) {
+    const uint32_t count = min(a.vis_count[seg], a.segment_size);
+    const uint4* vis = a.vis + (size_t)seg * a.segment_size;
+    for (uint32_t c0 = 0; c0 < count; c0 += kScatterEntries) {
+      uint4 e[2];
+      uint32_t nt[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t i = c0 + 2 * tid + h;
+        e[h] = i < count ? vis[i] : make_uint4(0u, 0u, 0u, 0u);
+        nt[h] = ((e[h].z >> 16) - (e[h].z & 0xffffu)) * ((e[h].w >> 16) - (e[h].w & 0xffffu));
+      }
+      uint32_t total;
+      const uint32_t excl = block_excl_scan<kScatterThreads>(nt[0] + nt[1], total, s_warp);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        s_incl[2 * tid + h] = excl + nt[0] + (h ? nt[1] : 0u);
+        if (nt[h]) {
+          ++visible;
+          const CamRec& cam = a.cams[e[h].x / a.n];
+          const uint32_t x0 = e[h].z & 0xffffu, y0 = e[h].w & 0xffffu;
+          s_entry[2 * tid + h] = make_uint4((uint32_t)cam.tile_offset + y0 * (uint32_t)cam.tiles_x + x0,
+                                            ((uint32_t)cam.tiles_x << 16) | ((e[h].z >> 16) - x0), e[h].x, e[h].y);
+        }
+      }
+      __syncthreads();
+      for (uint32_t o0 = tid; o0 < total; o0 += kScatterThreads * kScatterBatch) {
+        uint32_t pos[kScatterBatch];
+        uint64_t key[kScatterBatch];
+#pragma unroll
+        for (int k = 0; k < kScatterBatch; ++k) {
+          const uint32_t o = o0 + k * kScatterThreads;
+          pos[k] = 0xffffffffu;
+          if (o < total) {
+            uint32_t l = 0;   // entries whose duplicates all come before o
+#pragma unroll
+            for (uint32_t s = kScatterEntries / 2; s > 0; s >>= 1)
+              if (s_incl[l + s - 1] <= o) l += s;
+            const uint4 en = s_entry[l];
+            const uint32_t w = en.y & 0xffffu;
+            const uint32_t local = o - (l ? s_incl[l - 1] : 0u);
+            const uint32_t row = rect_row(local, w);
+            const uint32_t tile = en.x + row * (en.y >> 16) + (local - row * w);
+            key[k] = ((uint64_t)en.w << 32) | en.z;
+            if (tile < a.total_tiles) pos[k] = atomicAdd(&a.tile[tile].cursor, 1u);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < kScatterBatch; ++k)
+          if (pos[k] < a.capacity) a.dup[pos[k]] = key[k];
+      }
+      __syncthreads();
+    }
+  }
+  visible = __reduce_add_sync(0xffffffffu, visible);
+  if (lane == 0 && visible) atomicAdd(&s_vis, visible);
   __syncthreads();
-  for (int i = threadIdx.x; i < a.passes * 256; i += kScanThreads)
-    if (s_hist[i]) atomicAdd(&a.hist[i], s_hist[i]);
+  if (tid == 0 && s_vis) atomicAdd(&a.counts[0], s_vis);
 }
 
 // --------------------------------------------------------------------------
-// 5. Per-tile ranges in the sorted duplicate list
+// Sort of one tile's entries
 // --------------------------------------------------------------------------
-__global__ void ranges_kernel(RangesArgs a) {
-  const uint32_t k = min(*a.k_ptr, a.capacity);
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) {
-    const uint32_t t = a.keys[i];
-    if (t >= a.total_tiles) continue;
-    if (i == 0 || a.keys[i - 1] != t) a.ranges[t].x = i;
-    if (i == k - 1 || a.keys[i + 1] != t) a.ranges[t].y = i + 1;
+// A team of kWarps warps sorts up to 32 kItems kWarps entries, kItems (2 to 16)
+// a thread, with bitonic networks (Batcher, 1968) in registers: element i of
+// the network is item i % kItems of thread i / kItems, so that strides below
+// kItems stay in a thread, strides below 32 kItems are shuffles and only
+// longer ones go through shared memory.  What bounds it is integer
+// instructions, so
+//   * the network runs on 32-bit keys: the depth above the list's smallest,
+//     without the low bits that do not fit, over the entry's place in the
+//     unsorted list;
+//   * the keys of a thread whose run is to descend are complemented, so that
+//     every comparison of a run is ascending (two instructions, no selects).
+// Entries that agree in that much depth (equal depths, or neighbours in a long
+// list) may come out in the wrong order.  Then, and only then, the full
+// (depth, pair) keys are laid out in that order in shared memory and odd-even
+// transposition rounds put the few displaced neighbours right; a list with
+// many equal depths, still not in order after kFixRounds, is sorted by its
+// 64-bit keys.
+constexpr int kFixRounds = 8;
+constexpr int kMaxItems = 16;
+
+template <int kWarps>
+__device__ __forceinline__ void team_sync(uint32_t team) {
+  __syncwarp();
+  if (kWarps > 1) asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(32 * kWarps) : "memory");
+}
+
+// Is `flag` set in any thread of the team?  (Also a team barrier.)
+template <int kWarps>
+__device__ __forceinline__ bool team_any(uint32_t team, bool flag) {
+  __syncwarp();
+  if (kWarps == 1) return __any_sync(0xffffffffu, flag);
+  uint32_t any;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %3, 0;\n barrier.cta.red.or.pred.aligned q, %1, %2, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(any)
+      : "r"(team + 1), "r"(32 * kWarps), "r"((uint32_t)flag)
+      : "memory");
+  return any != 0u;
+}
+
+__device__ __forceinline__ void order_pair(uint32_t& x, uint32_t& y) {
+  const uint32_t lo = min(x, y);
+  y = max(x, y);
+  x = lo;
+}
+__device__ __forceinline__ void order_pair(uint64_t& x, uint64_t& y) {
+  const bool swap = x > y;
+  const uint64_t lo = swap ? y : x;
+  y = swap ? x : y;
+  x = lo;
+}
+
+template <int kItems, typename Key>
+__device__ __forceinline__ void flip(Key (&key)[kItems], bool on) {
+  const Key m = on ? ~(Key)0 : (Key)0;
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) key[i] ^= m;
+}
+
+template <int kItems, typename Key>
+__device__ __forceinline__ void merge_in_thread(Key (&key)[kItems]) {
+#pragma unroll
+  for (int j = kItems / 2; j > 0; j >>= 1)
+#pragma unroll
+    for (int i = 0; i < kItems; ++i)
+      if (!(i & j)) order_pair(key[i], key[i | j]);
+}
+
+// Sorts the team's 32 kItems kWarps keys.  tid: thread of the team; s_x: 4
+// keys a thread for the strides across warps (unused by one warp).
+template <int kItems, int kWarps, typename Key>
+__device__ __forceinline__ void bitonic_sort(Key (&key)[kItems], uint32_t team, uint32_t tid, Key* s_x) {
+  constexpr uint32_t kThreads = 32 * kWarps;
+#pragma unroll
+  for (int k = 2; k < kItems; k <<= 1)
+#pragma unroll
+    for (int j = k / 2; j > 0; j >>= 1)
+#pragma unroll
+      for (int i = 0; i < kItems; ++i)
+        if (!(i & j)) {
+          if ((i & k) == 0) order_pair(key[i], key[i | j]);
+          else order_pair(key[i | j], key[i]);
+        }
+  bool down = (tid & 1u) != 0u;   // the thread's run descends: its keys are complemented
+  flip(key, down);
+  merge_in_thread(key);
+#pragma unroll 1
+  for (uint32_t k = 2; k <= kThreads; k <<= 1) {   // in threads: runs of k kItems elements
+    const bool next = (tid & k) != 0u;
+    flip(key, down != next);
+    down = next;
+#pragma unroll 1
+    for (uint32_t m = k >> 1; m > 0u; m >>= 1) {
+      const bool lower = (tid & m) == 0u;   // of the two threads, the one that keeps the smaller keys
+      if (kWarps > 1 && m >= 32u) {
+#pragma unroll
+        for (int i0 = 0; i0 < kItems; i0 += 4) {
+          team_sync<kWarps>(team);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s_x[i * kThreads + tid] = key[i0 + i];
+          team_sync<kWarps>(team);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const Key other = s_x[i * kThreads + (tid ^ m)];
+            key[i0 + i] = ((key[i0 + i] < other) == lower) ? key[i0 + i] : other;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) {
+          const Key other = __shfl_xor_sync(0xffffffffu, key[i], m);
+          key[i] = ((key[i] < other) == lower) ? key[i] : other;
+        }
+      }
+    }
+    merge_in_thread(key);
+  }
+  team_sync<kWarps>(team);
+}
+
+// Place of element e in a team's shared memory: one word of padding a thread,
+// so that neither thread-order writes nor consecutive reads collide.
+template <int kItems>
+__device__ __forceinline__ uint32_t padded(uint32_t e) {
+  return e + e / kItems;
+}
+constexpr uint32_t kTeamWords = 512 + 512 / kMaxItems;   // 64-bit words of shared memory per warp
+
+// The list src[0, len) in order in s (padded()).
+template <int kItems, int kWarps>
+__device__ __noinline__ void sort_full(const uint64_t* src, uint32_t len, uint32_t team, uint32_t tid, uint64_t* s) {
+  constexpr uint32_t kThreads = 32 * kWarps;
+  uint64_t key[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) key[i] = i * kThreads + tid < len ? src[i * kThreads + tid] : ~0ull;
+  team_sync<kWarps>(team);
+  bitonic_sort<kItems, kWarps>(key, team, tid, s);
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) s[padded<kItems>(tid * kItems + i)] = key[i];
+  team_sync<kWarps>(team);
+}
+
+// The same for a list almost in order: place e holds entry at[e] of src.
+template <int kItems, int kWarps>
+__device__ __noinline__ void fix_order(const uint64_t* src, uint32_t len, uint32_t team, uint32_t tid, uint64_t* s,
+                                       const uint32_t* s_at) {
+  constexpr uint32_t kThreads = 32 * kWarps;
+  uint32_t at[kItems];
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) at[i] = s_at[padded<kItems>(tid * kItems + i)];
+  team_sync<kWarps>(team);
+#pragma unroll
+  for (int i = 0; i < kItems; ++i)
+    if (tid * kItems + i < len) s[padded<kItems>(tid * kItems + i)] = src[at[i]];
+  for (int round = 0;; ++round) {
+    bool moved = false;
+#pragma unroll
+    for (uint32_t odd = 0; odd < 2; ++odd) {   // e and e + 1 of even, then of odd e
+      team_sync<kWarps>(team);
+      for (uint32_t e = 2 * tid + odd; e + 1 < len; e += 2 * kThreads) {
+        const uint64_t x = s[padded<kItems>(e)], y = s[padded<kItems>(e + 1)];
+        if (x > y) {
+          s[padded<kItems>(e)] = y;
+          s[padded<kItems>(e + 1)] = x;
+          moved = true;
+        }
+      }
+    }
+    if (!team_any<kWarps>(team, moved)) break;
+    if (round == kFixRounds) {
+      sort_full<kItems, kWarps>(src, len, team, tid, s);
+      break;
+    }
   }
 }
 
-void launch_compact(const CompactArgs& a, int grid, cudaStream_t stream) {
-  compact_kernel<<<grid, kScanThreads, 0, stream>>>(a);
+// Sorts src[0, len), len <= 32 kItems kWarps, and calls store(e, full) for
+// the team's elements e < len in order, consecutive threads for consecutive
+// e: full() gives the element's (depth, pair) key.
+template <int kItems, int kWarps, typename Store>
+__device__ __forceinline__ void sort_team(const uint64_t* src, uint32_t len, uint32_t team, uint32_t tid, uint64_t* s,
+                                          Store store) {
+  constexpr uint32_t kThreads = 32 * kWarps, kCap = kThreads * kItems;
+  constexpr int kBits = 5 + (kItems >= 2) + (kItems >= 4) + (kItems >= 8) + (kItems >= 16) + (kWarps >= 2) +
+                        (kWarps >= 4) + (kWarps >= 8);   // log2(kCap)
+  uint32_t key[kItems];
+  uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const uint32_t e = i * kThreads + tid;
+    key[i] = e < len ? (uint32_t)(src[e] >> 32) : 0u;
+    if (e < len) {
+      lo = min(lo, key[i]);
+      hi = max(hi, key[i]);
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  uint32_t* s_w = reinterpret_cast<uint32_t*>(s);
+  if (kWarps > 1) {
+    if ((tid & 31u) == 0u) {
+      s_w[tid >> 4] = lo;
+      s_w[(tid >> 4) + 1] = hi;
+    }
+    team_sync<kWarps>(team);
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      lo = min(lo, s_w[2 * w]);
+      hi = max(hi, s_w[2 * w + 1]);
+    }
+  }
+  const int shift = max(kBits - __clz(hi - lo), 0);   // __clz(0) = 32
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const uint32_t e = i * kThreads + tid;
+    key[i] = e < len ? (((key[i] - lo) >> shift) << kBits) | e : 0xffffffffu;
+  }
+  bitonic_sort<kItems, kWarps>(key, team, tid, s_w);
+  bool tie = false;
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) {
+    const uint32_t e = tid * kItems + i;
+    s_w[padded<kItems>(e)] = key[i] & (kCap - 1u);
+    if (i > 0) tie = tie || ((key[i] ^ key[i - 1]) < kCap && e < len);
+  }
+  // a tie across two threads: the neighbour's last key
+  uint32_t last = __shfl_up_sync(0xffffffffu, key[kItems - 1], 1);
+  if (kWarps > 1) {
+    uint32_t* s_last = s_w + kCap + kCap / kItems;
+    if ((tid & 31u) == 31u) s_last[tid >> 5] = key[kItems - 1];
+    team_sync<kWarps>(team);
+    if ((tid & 31u) == 0u && tid) last = s_last[(tid >> 5) - 1];
+  }
+  tie = tie || (tid && (key[0] ^ last) < kCap && tid * kItems < len);
+  if (team_any<kWarps>(team, tie)) {
+    fix_order<kItems, kWarps>(src, len, team, tid, s, s_w);
+    for (uint32_t e = tid; e < len; e += kThreads) store(e, [&]() { return s[padded<kItems>(e)]; });
+  } else {
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) {
+      const uint32_t e = i * kThreads + tid;
+      if (e < len) store(e, [&]() { return src[s_w[padded<kItems>(e)]]; });
+    }
+  }
 }
-void launch_onesweep(const OnesweepArgs& a, int grid, cudaStream_t stream) {
-  onesweep_kernel<<<grid, kSortThreads, 0, stream>>>(a);
+
+// Sorted lists of the CTA's teams: one tile each.
+template <int kItems, int kWarps>
+__device__ __forceinline__ void sort_tile(const BinArgs& a, uint32_t tile, uint32_t start, uint32_t len,
+                                          uint64_t* s_key) {
+  const uint32_t team = threadIdx.x / (32 * kWarps), tid = threadIdx.x % (32 * kWarps);
+  sort_team<kItems, kWarps>(a.dup + start, len, team, tid, s_key + team * kWarps * kTeamWords,
+                            [&](uint32_t e, auto full) {
+                              a.sorted[start + e] = (uint32_t)full();
+                              a.sorted_key[start + e] = tile;
+                            });
 }
-void launch_emit(const EmitArgs& a, int scan_grid, int expand_grid, cudaStream_t stream) {
-  emit_scan_kernel<<<scan_grid, kScanThreads, 0, stream>>>(a);
-  emit_expand_kernel<<<expand_grid, kScanThreads, 0, stream>>>(a);
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-void launch_ranges(const RangesArgs& a, int grid, cudaStream_t stream) {
-  ranges_kernel<<<grid, 256, 0, stream>>>(a);
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// A list of more than kRun entries, by the CTAs of a cluster: runs of kRun
+// sorted on chip, then merged pairwise, each entry finding its rank in the
+// sibling run by a binary search.  The merges go back and forth between dup
+// and the (sorted_key, sorted) arrays, which hold a key in two words.
+constexpr uint32_t kRun = kMaxItems * kBinThreads;
+
+__device__ __noinline__ void sort_long(const BinArgs& a, uint32_t start, uint32_t len, uint32_t tile, uint64_t* s) {
+  const uint32_t rank = cluster_rank();
+  uint64_t* A = a.dup + start;
+  uint32_t* hi = a.sorted_key + start;
+  uint32_t* lo = a.sorted + start;
+  for (uint32_t r = rank * kRun; r < len; r += kCluster * kRun) {
+    const uint32_t m = min(kRun, len - r);
+    // (the run goes to the other arrays: its entries are still read here)
+    sort_team<kMaxItems, kBinWarps>(A + r, m, 0u, threadIdx.x, s, [&](uint32_t e, auto full) {
+      const uint64_t k = full();
+      hi[r + e] = (uint32_t)(k >> 32);
+      lo[r + e] = (uint32_t)k;
+    });
+    __syncthreads();
+  }
+  cluster_sync();
+  bool in_a = false;
+  for (uint32_t w = kRun; w < len; w *= 2) {
+    const bool last = w >= (len + 1) / 2;
+    auto load = [&](uint32_t i) -> uint64_t {
+      return in_a ? __ldcg(A + i) : ((uint64_t)__ldcg(hi + i) << 32) | __ldcg(lo + i);
+    };
+    for (uint32_t i = rank * kBinThreads + threadIdx.x; i < len; i += kCluster * kBinThreads) {
+      const uint64_t x = load(i);
+      const uint32_t run = i / w, sib = run ^ 1u;
+      const uint32_t s0 = min(sib * w, len), s1 = min(s0 + w, len);
+      uint32_t l = s0, h = s1;   // entries of the sibling run below x
+      while (l < h) {
+        const uint32_t m = (l + h) >> 1;
+        if (load(m) < x) l = m + 1u;
+        else h = m;
+      }
+      const uint32_t out = min((run & ~1u) * w + (i - run * w) + (l - s0), len - 1u);
+      if (in_a) {
+        hi[out] = last ? tile : (uint32_t)(x >> 32);
+        lo[out] = (uint32_t)x;
+      } else {
+        A[out] = x;
+      }
+    }
+    in_a = !in_a;
+    cluster_sync();
+  }
+  if (in_a) {
+    for (uint32_t i = rank * kBinThreads + threadIdx.x; i < len; i += kCluster * kBinThreads) {
+      lo[i] = (uint32_t)__ldcg(A + i);
+      hi[i] = tile;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
+  __shared__ uint64_t s_key[kBinWarps * kTeamWords];
+  __shared__ uint32_t s_unit;
+  const int tid = threadIdx.x;
+  // order: over[0] tiles with lists above 4096 entries, up to over[1] those
+  // above 2048, over[2] 1024, over[3] 512, over[4] the rest that are not empty
+  uint32_t over[kBinLevels + 1];
+  over[kBinLevels] = min(a.state[kBinOver + kBinLevels], a.total_tiles);
+#pragma unroll
+  for (int l = kBinLevels - 1; l >= 0; --l) over[l] = min(a.state[kBinOver + l], over[l + 1]);
+  if (blockIdx.x == 0 && tid < 2 * kClasses) a.state[kBinClass + tid] = 0u;   // clean for the next call
+  for (uint32_t u = blockIdx.x / kCluster; u < over[0]; u += gridDim.x / kCluster) {
+    const uint32_t t = a.order[u];
+    const uint2 r = t < a.total_tiles ? a.ranges[t] : make_uint2(0u, 0u);
+    sort_long(a, r.x, r.y - r.x, t, s_key);
+    cluster_sync();
+  }
+  // units of the rest: one, two, four or eight tiles a CTA
+  const uint32_t u1 = over[1] - over[0], u2 = u1 + (over[2] - over[1] + 1) / 2, u4 = u2 + (over[3] - over[2] + 3) / 4;
+  const uint32_t units = u4 + (over[4] - over[3] + 7) / 8;
+  while (true) {
+    __syncthreads();
+    if (tid == 0) s_unit = atomicAdd(&a.state[kBinQueue], 1u);
+    __syncthreads();
+    const uint32_t u = s_unit;
+    if (u >= units) break;
+    uint32_t at, end, teams;
+    if (u < u1) at = over[0] + u, end = over[1], teams = 1;
+    else if (u < u2) at = over[1] + 2 * (u - u1), end = over[2], teams = 2;
+    else if (u < u4) at = over[2] + 4 * (u - u2), end = over[3], teams = 4;
+    else at = over[3] + 8 * (u - u4), end = over[4], teams = 8;
+    at += threadIdx.x / (kBinThreads / teams);
+    const uint32_t t = at < end ? a.order[at] : 0xffffffffu;
+    const uint2 r = t < a.total_tiles ? a.ranges[t] : make_uint2(0u, 0u);
+    const uint32_t len = min(r.y - r.x, kRun / teams);
+    if (len == 0u) continue;   // (the whole team)
+    if (teams == 1) sort_tile<16, 8>(a, t, r.x, len, s_key);
+    else if (teams == 2) sort_tile<16, 4>(a, t, r.x, len, s_key);
+    else if (teams == 4) sort_tile<16, 2>(a, t, r.x, len, s_key);
+    else if (len > 256u) sort_tile<16, 1>(a, t, r.x, len, s_key);
+    else if (len > 128u) sort_tile<8, 1>(a, t, r.x, len, s_key);
+    else if (len > 64u) sort_tile<4, 1>(a, t, r.x, len, s_key);
+    else sort_tile<2, 1>(a, t, r.x, len, s_key);
+  }
+}
+
+// Grids: the scan has one block per 256 tiles; the scatter at most 16 CTAs per
+// SM, each with the segments of its stride; the sort, which takes its tiles
+// from a queue, a whole number of clusters, at most 4 CTAs per SM.
+cudaError_t launch_bin(const BinArgs& a, int sms, cudaStream_t stream) {
+  const uint32_t blocks = std::max(1u, (a.total_tiles + kScanTile - 1) / kScanTile);
+  bin_scan_kernel<<<blocks, kBinThreads, 0, stream>>>(a);
+  const uint32_t order = (a.total_tiles + kScatterThreads - 1) / kScatterThreads;
+  const uint32_t grid = std::min(std::max(std::max(a.segments, order), 1u), (uint32_t)sms * 16u);
+  bin_scatter_kernel<<<grid, kScatterThreads, 0, stream>>>(a);
+  const uint32_t most = std::max(1u, (uint32_t)sms * 4u / kCluster);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(std::min(most, (std::max(a.total_tiles, 1u) + kCluster - 1) / kCluster) * kCluster);
+  cfg.blockDim = dim3(kBinThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kCluster;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, bin_sort_kernel, a);
 }
 
 }  // namespace sixdgs
