@@ -342,6 +342,7 @@ static BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
   a.n_pairs = (uint32_t)p->n_pairs;
   a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
   a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
+  a.order = ws_ptr<uint32_t>(ws, p, WS_ORDER);
   for (int i = 0; i < 3; ++i) a.bg[i] = p->settings.bg[i];
   const double norm = p->settings.loss_norm > 0.f ? (double)p->settings.loss_norm
                                                    : 3.0 * (double)p->total_pixels;

