@@ -3,26 +3,32 @@
 //
 // One CTA per global tile (all cameras' tiles in one grid, so cameras of
 // different resolutions share a launch); each warp owns an 8x4 sub-block of
-// the tile, one pixel per lane.  The tile's sorted list is walked in
-// batches: each batch of pair records is gathered into shared memory by the
-// whole CTA; then every warp tests 32 entries at a time against its
-// sub-block (lane-parallel box test with the entry's alpha >= 1/255 box,
-// ballot) and composites its pixels only against the entries that can reach
-// them, in list order.  An entry a warp passes over would be skipped at
-// every pixel of its sub-block (q < log2(1/255)), so the result is the same
-// as walking every entry at every pixel.  A CTA leaves as soon as
-// __syncthreads_count reports every pixel saturated; a warp leaves a batch
-// as soon as all its lanes are done.
+// the tile, each half-warp a 4x4 block of it, one pixel per lane.  The tile's
+// sorted list is walked in batches: each batch of pair records is gathered
+// into shared memory by the whole CTA, each thread testing its entries' alpha
+// >= 1/255 ellipses against all blocks of the tile (ballots: a bit per block
+// and entry); then every warp turns its two blocks' ballots into lists and
+// composites each pixel against its block's list, in list order.  An entry a
+// block passes over would be skipped at every pixel of it (q < log2(1/255)),
+// so the result is the same as walking every entry at every pixel.  A CTA
+// leaves as soon as __syncthreads_count reports every pixel saturated; a warp
+// leaves a batch as soon as all its lanes are done.
+//
+// The walks are bound by instructions, most of them spent at pixels that an
+// entry does not reach and on finding the next entry.  Hence the 4x4 blocks
+// (a Gaussian of 5 pixels radius reaches 11 of them, 174 pixels, against 230
+// pixels of 8x4 blocks; a warp's two lists are nearly equally long), and the
+// lists: a walk takes four entries' addresses with one load instead of
+// scanning a ballot bit by bit.  Against 8x4 blocks tested by their own warps
+// (fused kernel / warp instructions): 858 -> 722 us, 755 -> 618 M at 300k /
+// 8 x 800^2; 1487 -> 1244 us at 2M / 4 x 1920x1080; forward 663 -> 599 us for
+// 20 views of 183k Gaussians at 1024^2.
 //
 // Per entry and pixel:  q = qa dx^2 + qb dx dy + qc dy^2 + lo  (log2 alpha),
 // skipped when q < log2(1/255); alpha = min(0.99, 2^q); stop (excluding the
 // entry) when T (1 - alpha) < 1e-4; C += c alpha T; T *= (1 - alpha).
 // Explicit rounding intrinsics make the backward replay bit-identical.
-// The stand-alone forward culls with the alpha box only (its per-entry work
-// is too cheap for the exact test to pay off); the backward, whose
-// per-entry work is several times larger, also applies the exact quadratic
-// test, and in the fused kernel the forward applies it and records each
-// group's ballot for the backward.  Pairs of values that take the same
+// Pairs of values that take the same
 // operation (the pixel offset, T (1 - alpha) and alpha T, two colour
 // channels) use the packed two-wide FP32 instructions, with the same
 // rounding as the scalar ones.
@@ -35,6 +41,7 @@ namespace sixdgs {
 
 constexpr int kSubW = 8;   // warp sub-block: 8 x 4 pixels
 constexpr int kSubH = 4;
+constexpr int kBlkW = 4;   // half-warp block: 4 x 4 pixels
 
 __device__ __forceinline__ int find_camera(const CamRec* cams, int n_cams, uint32_t gt) {
   int lo = 0, hi = n_cams - 1;
@@ -49,7 +56,9 @@ __device__ __forceinline__ int find_camera(const CamRec* cams, int n_cams, uint3
 // Pixel of this thread and the pixel-centre box of its warp's sub-block.
 struct PixelMap {
   int px, py;
-  float x0, x1, y0, y1;   // pixel centres spanned by the warp
+  float x0, y0;   // first pixel centre of the warp
+  float tx0, ty0; // and of the tile
+  int block;      // the warp's left block in the tile
 };
 
 __device__ __forceinline__ PixelMap map_pixel(int tile_w, int tx, int ty, int tile_h) {
@@ -57,66 +66,121 @@ __device__ __forceinline__ PixelMap map_pixel(int tile_w, int tx, int ty, int ti
   const int sub_per_row = tile_w / kSubW;
   const int sx = (warp % sub_per_row) * kSubW, sy = (warp / sub_per_row) * kSubH;
   PixelMap m;
-  m.px = tx * tile_w + sx + (lane % kSubW);
-  m.py = ty * tile_h + sy + (lane / kSubW);
+  m.px = tx * tile_w + sx + (lane >> 4) * kBlkW + (lane & 3);
+  m.py = ty * tile_h + sy + ((lane >> 2) & 3);
   m.x0 = (float)(tx * tile_w + sx) + 0.5f;
-  m.x1 = m.x0 + (float)(kSubW - 1);
   m.y0 = (float)(ty * tile_h + sy) + 0.5f;
-  m.y1 = m.y0 + (float)(kSubH - 1);
+  m.tx0 = (float)(tx * tile_w) + 0.5f;
+  m.ty0 = (float)(ty * tile_h) + 0.5f;
+  m.block = sy / kSubH * (tile_w / kBlkW) + sx / kBlkW;
   return m;
 }
 
-// Can the entry have q >= log2(1/255) at some pixel centre of the warp's
-// sub-block?  First the entry's alpha box (u, v, hx, hy); with kExact also
-// the maximum of the concave quadratic q over the sub-block's pixel-centre
-// rectangle: the entry's centre if it lies inside, else the best point of
-// the four edges (vertex of q along each edge, clamped to the edge).  The
-// continuous maximum bounds every pixel centre's q, and the 1e-3 margin (in
-// log2 units) is far above FP32 rounding, so no pixel that would composite
-// the entry is ever passed over.
-template <bool kExact>
-__device__ __forceinline__ bool reaches(const PixelMap& m, float4 a, float4 b, float4 c) {
-  if (!((a.x + c.y >= m.x0) && (a.x - c.y <= m.x1) && (a.y + c.z >= m.y0) && (a.y - c.z <= m.y1)))
-    return false;
-  if (!kExact) return true;
-  const float dx0 = a.x - m.x1, dx1 = a.x - m.x0;   // dx = u - x over the sub-block
-  const float dy0 = a.y - m.y1, dy1 = a.y - m.y0;
-  if (dx0 <= 0.f && dx1 >= 0.f && dy0 <= 0.f && dy1 >= 0.f) return true;
-  const float qa = a.z, qb = a.w, qc = b.x;
-  const float kx = __fdividef(-0.5f * qb, qc), ky = __fdividef(-0.5f * qb, qa);
-  float best = -INFINITY;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const float dx = e ? dx1 : dx0;
-    const float dy = fminf(fmaxf(kx * dx, dy0), dy1);
-    best = fmaxf(best, (qa * dx + qb * dy) * dx + qc * dy * dy);
-    const float ey = e ? dy1 : dy0;
-    const float ex = fminf(fmaxf(ky * ey, dx0), dx1);
-    best = fmaxf(best, (qa * ex + qb * ey) * ex + qc * ey * ey);
+// The 4x4 blocks of a tile of tile_w x 4 nby pixels that the entry (u, v, qa,
+// qb), (qc, lo), (hx, hy) can reach, bit y * tile_w / 4 + x: those where q >=
+// log2(1/255) at some point of the block's pixel-centre rectangle.  (x0, y0):
+// the tile's first pixel centre.  For every row of blocks (a band of four
+// pixel rows) the ellipse {q >= log2(1/255) - m} meets the band in a convex
+// set, whose columns reach from the leftmost to the rightmost point: the
+// ellipse's own extreme points (+-hx) if the band holds them, else the
+// boundary at the band's row nearest to them.  The margin m (in log2 units)
+// covers the FP32 rounding of a pixel's q, at most a few ulp of S = |qa| dx^2 +
+// |qc| dy^2 at the tile's far corner, and of the boundary's square root; so no
+// pixel that would composite the entry is ever passed over.  One thread tests
+// an entry against all blocks: a tenth of the instructions of every warp
+// testing every entry against its own blocks (153 a warp and 32 entries).
+__device__ __forceinline__ uint32_t block_mask(float4 a, float4 b, float4 c, float x0, float y0, int tile_w, int nby) {
+  const float ux = a.x - x0, vy = a.y - y0, hx = c.y, hy = c.z;
+  const float fw = (float)(tile_w - 1), fh = (float)(nby * kSubH - 1);
+  if (!(ux + hx >= 0.f && ux - hx <= fw && vy + hy >= 0.f && vy - hy <= fh)) return 0u;
+  const int nbx = tile_w / kBlkW;
+  const float A = -a.z, B = -a.w, C = -b.x;   // A dx^2 + B dx dy + C dy^2 <= L
+  const float dxm = fmaxf(fabsf(ux), fabsf(ux - fw)), dym = fmaxf(fabsf(vy), fabsf(vy - fh));
+  const float S = A * dxm * dxm + C * dym * dym;
+  if (!(A > 1e-30f && C > 1e-30f && S < 1e30f)) return nbx * nby == 32 ? ~0u : (1u << (nbx * nby)) - 1u;
+  const float L = b.y - kQMin + (1e-3f + 1e-6f * S);
+  const float ia = __fdividef(1.f, A);
+  const float k = 0.5f * B * ia;                    // middle of the columns of a row: dx = -k dy
+  const float E = L * ia, F = k * k - C * ia;       // their half-length: sqrt(E + F dy^2)
+  const float dyr = -0.5f * B * __fdividef(1.f, C) * hx;   // row of the rightmost point (leftmost: -dyr)
+  const float pad = 2e-3f + 1e-6f * dxm;
+  uint32_t mask = 0u;
+#pragma unroll 4
+  for (int r = 0; r < nby; ++r) {
+    const float d1 = vy - (float)(r * kSubH), d0 = d1 - (float)(kSubH - 1);
+    const float cr = fminf(fmaxf(dyr, d0), d1), cl = fminf(fmaxf(-dyr, d0), d1);
+    const float sr = fmaf(F, cr * cr, E), sl = fmaf(F, cl * cl, E);
+    const bool in_r = cr == dyr, in_l = cl == -dyr;
+    const float dxr = in_r ? hx : fmaf(-k, cr, sqrt_approx(fmaxf(sr, 0.f)));
+    const float dxl = in_l ? -hx : fmaf(-k, cl, -sqrt_approx(fmaxf(sl, 0.f)));
+    const bool hit = in_r || in_l || sr >= 0.f || sl >= 0.f;
+    // columns ux - dxr .. ux - dxl; block x spans 4 x .. 4 x + 3
+    const int first = max(__float2int_ru((ux - dxr - pad - (float)(kBlkW - 1)) * (1.f / kBlkW)), 0);
+    const int last = min(__float2int_rd((ux - dxl + pad) * (1.f / kBlkW)), nbx - 1);
+    if (hit && first <= last) mask |= ((2u << last) - (1u << first)) << (r * nbx);
   }
-  return best + b.y >= kQMin - 1e-3f;
+  return mask;
 }
 
 // A list entry as staged in shared memory: its blend record (u, v, qa, qb),
-// (qc, lo, r, g), (b, hx, hy) and its pair index (bits of c.w).  One struct
+// (qc, lo, r, g), b and its pair index (bits of c.w).  One struct
 // per entry, so a walk addresses all three parts from one index.
 struct __align__(16) Entry {
   float4 a, b, c;
 };
 
-__device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, int cnt, Entry* s_e) {
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-    const uint32_t p = a.sorted[start + i];
-    if (p < a.n_pairs) {
-      const PairRec& r = a.rec[p];
-      s_e[i].a = r.a;
-      s_e[i].b = r.b;
-      s_e[i].c = make_float4(r.c.x, r.c.y, r.c.z, __uint_as_float(p));
-    } else {  // unreachable for a consistent sort: an entry that reaches no pixel
-      s_e[i].a = make_float4(-1e30f, -1e30f, 0.f, 0.f);
-      s_e[i].b = make_float4(0.f, -1e30f, 0.f, 0.f);
-      s_e[i].c = make_float4(0.f, 0.f, 0.f, __uint_as_float(0u));
+__device__ __forceinline__ void null_entry(Entry& e, uint32_t p) {   // reaches no pixel
+  e.a = make_float4(-1e30f, -1e30f, 0.f, 0.f);
+  e.b = make_float4(0.f, -1e30f, 0.f, 0.f);
+  e.c = make_float4(0.f, 0.f, 0.f, __uint_as_float(p));
+}
+
+// Shared memory of a CTA: the batch's entries and a null entry, which pads the
+// lists (entry a.batch), the ballots of every block over the batch (word
+// block * cull_stride(batch) + g: entries 32 g to 32 g + 31), then each warp's
+// scratch.
+__host__ __device__ constexpr int cull_stride(int batch) { return (batch / 32 + 3) & ~3; }
+__host__ __device__ constexpr int stage_bytes(int batch, int blocks) {
+  return (batch + 1) * (int)sizeof(Entry) + blocks * cull_stride(batch) * 4;
+}
+__device__ __forceinline__ int blocks_of(const BlendArgs& a) { return a.tile_w * a.tile_h / (kBlkW * kSubH); }
+__device__ __forceinline__ uint32_t* cull_of(const BlendArgs& a, Entry* s_e) {
+  return reinterpret_cast<uint32_t*>(s_e + a.batch + 1);
+}
+__device__ __forceinline__ char* scratch_of(const BlendArgs& a, void* s_mem) {
+  return reinterpret_cast<char*>(s_mem) + stage_bytes(a.batch, blocks_of(a));
+}
+
+// Stages list entries [start, start + cnt) and their blocks' ballots.
+// (x0, y0): first pixel centre of the tile.
+__device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, int cnt, float x0, float y0,
+                                           Entry* s_e) {
+  if (threadIdx.x == 0) null_entry(s_e[a.batch], 0u);
+  const int lane = threadIdx.x & 31, blocks = blocks_of(a);
+  uint32_t* cull = cull_of(a, s_e);
+  for (int i0 = threadIdx.x & ~31; i0 < cnt; i0 += blockDim.x) {
+    const int i = i0 + lane;
+    uint32_t mask = 0u;
+    if (i < cnt) {
+      const uint32_t p = a.sorted[start + i];
+      if (p < a.n_pairs) {
+        const PairRec& r = a.rec[p];
+        const float4 ra = r.a, rb = r.b, rc = r.c;
+        s_e[i].a = ra;
+        s_e[i].b = rb;
+        s_e[i].c = make_float4(rc.x, rc.y, rc.z, __uint_as_float(p));
+        mask = block_mask(ra, rb, rc, x0, y0, a.tile_w, a.tile_h / kSubH);
+      } else {  // unreachable for a consistent sort
+        null_entry(s_e[i], 0u);
+      }
     }
+    uint32_t word = 0u;   // of block `lane`
+#pragma unroll 4
+    for (int b = 0; b < blocks; ++b) {
+      const uint32_t w = __ballot_sync(0xffffffffu, (mask >> b) & 1u);
+      if (lane == b) word = w;
+    }
+    if (lane < blocks) cull[lane * cull_stride(a.batch) + (i0 >> 5)] = word;
   }
 }
 
@@ -125,35 +189,79 @@ __device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, i
 //  1. pixel-parallel (lane = pixel), front to back like the forward: the
 //     transmittance T and the running dL/dC . (colour prefix) Q are carried
 //     per pixel, and each pixel's dL/dq and blend weight w for the entry are
-//     written to the warp's shared-memory slots (kSlots = 8 entries at a
-//     time);
+//     written to the warp's shared-memory slots (kSlots = 8 entries of each
+//     half-warp at a time);
 //  2. entry-parallel, once the slots are full (or the batch ends): lane
-//     8 r + s takes slot s over row r of the 8 x 4 sub-block and sums, over
-//     the row's 8 pixels, dq, c dq, c^2 dq and dL/dC . w (c the column
-//     relative to the sub-block's centre); the four rows are added with
-//     shuffles, and lane s turns the sums into the entry's nine record
-//     gradients (moments of dq in dx = u - px, dy = v - py) and adds them to
-//     the record gradients in global memory.
+//     16 h + 8 r + s takes slot s of half h over two rows of its 4 x 4 block
+//     and sums, over their 8 pixels, dq, c dq, c^2 dq and dL/dC . w (c the
+//     column relative to the block's centre); the two halves of the block are
+//     added with a shuffle, and lane 16 h + s turns the sums into the entry's
+//     nine record gradients (moments of dq in dx = u - px, dy = v - py) and
+//     adds them to the record gradients in global memory.
 // A slot's 32 pixel values are stored with a stride of 33 (one float2 of
 // padding per slot), so the row writes of pass 1 and the column reads of
 // pass 2 are both free of shared-memory bank conflicts.
 constexpr int kSlots = 8;
-constexpr int kCullGroups = 64;   // 2,048 list entries
+constexpr int kChunk = 128;   // list entries whose ballots are turned into lists at a time
+constexpr int kStep = 4;      // entries walked between two looks at the lists
+
+// A block's list: byte offsets of its entries in the staging area (at most
+// 1,024 x 48), padded with the null entry to a multiple of kStep.
+struct __align__(16) WalkLists {
+  uint16_t off[2][kChunk + 8];
+};
 struct __align__(16) WarpScratch {
+  WalkLists lists;
   float2 dqw[kSlots][33];   // (dL/dq / ln 2, w) of slot s at pixel p, at [s][p]
   float4 pix[35];           // dL/dC of pixel p at p + (p >> 3) (rows in other banks)
-  int slot_j[kSlots];       // batch index of the entry in slot s
-  // fused kernel: the forward walk's culling ballot of list entries
-  // [32 g, 32 g + 32) of the tile's list (first kCullGroups groups)
-  uint32_t cull[kCullGroups];
+  uint2 slot[2][kSlots / kStep];   // offsets of the entries in the slots, four to a word pair
 };
 
-__host__ __device__ constexpr int bwd_scratch_bytes(int threads) {
-  return (threads / 32) * (int)sizeof(WarpScratch);
+// Fills a warp's lists with the batch's entries [c0, c0 + kChunk) (cnt in the
+// batch); returns the number of steps of the longer one, a multiple of kStep.
+// cull: the ballots of the warp's left block (its right one's follow).
+__device__ __forceinline__ int fill_lists(const uint32_t* cull, int batch, int c0, int cnt, WalkLists& lists,
+                                          uint32_t* n_warp = nullptr) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t n0 = 0u, n1 = 0u;
+  __syncwarp();   // the lists are no longer read
+  cull += c0 >> 5;
+#pragma unroll
+  for (int g = 0; g < kChunk / 32; ++g) {
+    const int base = c0 + 32 * g;
+    if (base < cnt) {
+      const uint32_t m0 = cull[g], m1 = cull[cull_stride(batch) + g];
+      const uint16_t off = (uint16_t)((base + lane) * (int)sizeof(Entry));
+      if ((m0 >> lane) & 1u) lists.off[0][n0 + __popc(m0 & below)] = off;
+      if ((m1 >> lane) & 1u) lists.off[1][n1 + __popc(m1 & below)] = off;
+      n0 += __popc(m0);
+      n1 += __popc(m1);
+      if (n_warp) *n_warp += __popc(m0 | m1);
+    }
+  }
+  const int steps = (int)(max(n0, n1) + (kStep - 1)) & ~(kStep - 1);
+  const int h = lane >> 4;
+  for (int i = (int)(h ? n1 : n0) + (lane & 15); i < steps; i += 16)
+    lists.off[h][i] = (uint16_t)(batch * (int)sizeof(Entry));
+  __syncwarp();
+  return steps;
+}
+
+// Offsets of four consecutive list entries (i a multiple of kStep).
+__device__ __forceinline__ uint2 list_quad(const WalkLists& lists, int i) {
+  return *reinterpret_cast<const uint2*>(&lists.off[(threadIdx.x >> 4) & 1][i]);
+}
+__device__ __forceinline__ uint32_t quad_off(uint2 q, int k) {
+  const uint32_t w = k < 2 ? q.x : q.y;
+  return (k & 1) ? w >> 16 : w & 0xffffu;
+}
+__device__ __forceinline__ const Entry& entry_at(const Entry* s_e, uint32_t off) {
+  return *reinterpret_cast<const Entry*>(reinterpret_cast<const char*>(s_e) + off);
 }
 
 // Per-pixel front-to-back walk of a tile's list (the forward blend): T and
-// C accumulate over the entries that reach the warp's sub-block; walked is
+// C accumulate over the entries that reach the pixel's block; walked is
 // the number of list entries before the stop (the list length if none).
 struct FwdPixel {
   float T, C0, C1, C2;
@@ -161,15 +269,12 @@ struct FwdPixel {
   bool staged;   // the whole list was loaded as one batch (CTA-uniform)
 };
 
-// cull (fused kernel, else null): the exact sub-block test is used and each
-// group's ballot is recorded there for the backward walk.
 template <bool kCount>
 __device__ __forceinline__ FwdPixel fwd_walk(const BlendArgs& a, const PixelMap& pm, float pxc, float pyc,
-                                             uint2 range, bool inside, Entry* s_e,
-                                             uint32_t& n_eval, uint32_t& n_comp, uint32_t& n_warp,
-                                             uint32_t* cull = nullptr) {
+                                             uint2 range, bool inside, Entry* s_e, WalkLists& lists,
+                                             uint32_t& n_eval, uint32_t& n_comp, uint32_t& n_warp) {
   const int B = a.batch;
-  const int lane = threadIdx.x & 31;
+  const uint32_t* cull = cull_of(a, s_e) + pm.block * cull_stride(B);
   float T = 1.f, C2 = 0.f;
   float2 C01 = make_float2(0.f, 0.f);
   const float2 npix = make_float2(-pxc, -pyc);
@@ -179,55 +284,66 @@ __device__ __forceinline__ FwdPixel fwd_walk(const BlendArgs& a, const PixelMap&
   for (uint32_t start = range.x; start < range.y; start += B) {
     if (__syncthreads_count(done) == (int)blockDim.x) break;
     const int cnt = (int)min((uint32_t)B, range.y - start);
-    load_batch(a, start, cnt, s_e);
+    load_batch(a, start, cnt, pm.tx0, pm.ty0, s_e);
     staged = start == range.x && start + cnt == range.y;
     __syncthreads();
     if (__all_sync(0xffffffffu, done)) continue;
-    for (int base = 0; base < cnt; base += 32) {
-      const int jl = base + lane;
-      const bool rel = jl < cnt && (cull ? reaches<true>(pm, s_e[jl].a, s_e[jl].b, s_e[jl].c)
-                                         : reaches<false>(pm, s_e[jl].a, s_e[jl].b, s_e[jl].c));
-      uint32_t mask = __ballot_sync(0xffffffffu, rel);
-      if (cull) {
-        const uint32_t g = (start - range.x + base) >> 5;
-        if (lane == 0 && g < kCullGroups) cull[g] = mask;
-      }
-      if (kCount) n_warp += __popc(mask);
-      while (mask) {
-        const int j = base + __ffs(mask) - 1;
-        mask &= mask - 1;
-        // Branch-free: a skipped (or finished) pixel takes alpha = 0, which
-        // leaves T and C bit-for-bit unchanged.
-        const float4 ra = s_e[j].a, rb = s_e[j].b;
-        const float blue = s_e[j].c.x;
-        float2 d;
-        const float q = entry_q(ra, rb, npix, d);
-        const bool vis = !done && q >= kQMin;
-        const float alpha = vis ? fminf(kAlphaMax, ex2_approx(q)) : 0.f;
-        // (T (1 - alpha), alpha T) in one packed multiply
-        const float2 tw = __fmul2_rn(make_float2(T, T), make_float2(__fsub_rn(1.f, alpha), alpha));
-        const bool stop = tw.x < kTMin;
-        const float w = stop ? 0.f : tw.y;
-        C01 = __ffma2_rn(make_float2(rb.z, rb.w), make_float2(w, w), C01);
-        C2 = __fmaf_rn(blue, w, C2);
-        T = stop ? T : tw.x;
-        if (stop) walked = start - range.x + j;
-        if (kCount) {
-          n_eval += done ? 0u : 1u;
-          n_comp += (vis && !stop) ? 1u : 0u;
+    uint32_t stop_off = 0xffffffffu;   // of the entry this pixel stopped at in this batch
+    for (int c0 = 0; c0 < cnt; c0 += kChunk) {
+      const int steps = fill_lists(cull, B, c0, cnt, lists, kCount ? &n_warp : nullptr);
+      bool all = false;
+#pragma unroll 1
+      for (int i = 0; i < steps && !all; i += kStep) {
+        const uint2 quad = list_quad(lists, i);
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) {
+          // Branch-free: a skipped (or finished) pixel takes alpha = 0, which
+          // leaves T and C bit-for-bit unchanged.
+          const uint32_t off = quad_off(quad, k);
+          const Entry& en = entry_at(s_e, off);
+          const float4 ra = en.a, rb = en.b;
+          const float blue = en.c.x;
+          float2 d;
+          const float q = entry_q(ra, rb, npix, d);
+          const bool vis = !done && q >= kQMin;
+          const float alpha = vis ? fminf(kAlphaMax, ex2_approx(q)) : 0.f;
+          // (T (1 - alpha), alpha T) in one packed multiply
+          const float2 tw = __fmul2_rn(make_float2(T, T), make_float2(__fsub_rn(1.f, alpha), alpha));
+          const bool stop = tw.x < kTMin;   // (never for alpha = 0: T is not below kTMin)
+          const float w = stop ? 0.f : tw.y;
+          C01 = __ffma2_rn(make_float2(rb.z, rb.w), make_float2(w, w), C01);
+          C2 = __fmaf_rn(blue, w, C2);
+          T = stop ? T : tw.x;
+          stop_off = stop ? off : stop_off;
+          if (kCount) {
+            n_eval += (done || off == (uint32_t)(B * (int)sizeof(Entry))) ? 0u : 1u;
+            n_comp += (vis && !stop) ? 1u : 0u;
+          }
+          done = done || stop;
         }
-        done = done || stop;
+        all = __all_sync(0xffffffffu, done);
       }
-      if (__all_sync(0xffffffffu, done)) break;
+      if (all) break;
     }
+    if (stop_off != 0xffffffffu) walked = start - range.x + stop_off / (uint32_t)sizeof(Entry);
   }
   return FwdPixel{T, C01.x, C01.y, C2, walked, staged};
+}
+
+// Sum over the 32 pixels of a sub-block, rows first, then columns from the
+// outermost bit in (an order that does not depend on how the pixels are dealt
+// to the lanes; lane bits: half, row, row, column, column).
+__device__ __forceinline__ float sub_block_sum(float v) {
+#pragma unroll
+  for (int o : {8, 4, 16, 2, 1}) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // Forward blend of global tile gt by the calling CTA.
 template <bool kCount, bool kStore>
 __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint32_t gt, float4* s_mem) {
   Entry* s_e = reinterpret_cast<Entry*>(s_mem);
+  WalkLists* lists = reinterpret_cast<WalkLists*>(scratch_of(a, s_mem));
   __shared__ float s_red[16];
 
   const CamRec& cam = a.cams[find_camera(a.cams, a.n_cams, gt)];
@@ -239,7 +355,8 @@ __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint32_t gt, 
   const int lane = threadIdx.x & 31;
 
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
-  const FwdPixel fp = fwd_walk<kCount>(a, pm, pxc, pyc, range, inside, s_e, n_eval, n_comp, n_warp);
+  const FwdPixel fp =
+      fwd_walk<kCount>(a, pm, pxc, pyc, range, inside, s_e, lists[threadIdx.x >> 5], n_eval, n_comp, n_warp);
   float T = fp.T, C0 = fp.C0, C1 = fp.C1, C2 = fp.C2;
   const uint32_t walked = fp.walked;
 
@@ -279,7 +396,7 @@ __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint32_t gt, 
     }
   }
   if (a.targets) {
-    l1 = warp_sum(l1);
+    l1 = sub_block_sum(l1);
     if (lane == 0) s_red[threadIdx.x >> 5] = l1;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -300,40 +417,50 @@ __device__ __forceinline__ void red_add4(float* addr, float x, float y, float z,
                : "memory");
 }
 
-// Pass 2 over slots [0, k).  xc, yc: centre of the 8 x 4 sub-block.
+// Pass 2 over slots [0, k) of both halves.  null_off: offset of the null entry.
 __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws, int k, const Entry* s_e,
-                                            float xc, float yc) {
-  static_assert(kSlots == kSubW && kSubH == 4, "one row of the sub-block per slot group");
+                                            const PixelMap& pm, uint32_t null_off) {
+  static_assert(kSlots == 8 && kBlkW == 4 && kSubH == 4, "two rows of a block per lane");
   __syncwarp();
   const int lane = threadIdx.x & 31;
   const int s = lane & (kSlots - 1);
-  const int r = lane >> 3;                 // row of the sub-block
-  const float2* row = ws.dqw[s];
-  float R1 = 0.f, R2 = 0.f;
-  float2 RG = make_float2(0.f, 0.f);    // (sum dq, sum dC2 w)
-  float2 G01 = make_float2(0.f, 0.f);   // (sum dC0 w, sum dC1 w)
+  const int r = (lane >> 3) & 1;           // rows 2 r and 2 r + 1 of the block
+  const int h = lane >> 4;
+  const float2* row = ws.dqw[s] + (lane & ~7);
+  const float4* pix = ws.pix + (lane & ~7) + (lane >> 3);
+  float R1[2] = {0.f, 0.f}, R2[2] = {0.f, 0.f};
+  float2 RG[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // (sum dq, sum dC2 w)
+  float2 G01 = make_float2(0.f, 0.f);                              // (sum dC0 w, sum dC1 w)
 #pragma unroll
-  for (int c = 0; c < kSubW; ++c) {
-    const int p = r * kSubW + c;
+  for (int p = 0; p < 2 * kBlkW; ++p) {
+    const int y = p / kBlkW;
     const float2 v = row[p];
-    const float4 dc = ws.pix[p + (p >> 3)];   // (dC0, dC1, 1, dC2)
-    const float cc = (float)c - 0.5f * (float)(kSubW - 1);   // column about the centre
-    R1 = fmaf(cc, v.x, R1);
-    R2 = fmaf(cc * cc, v.x, R2);
-    RG = __ffma2_rn(make_float2(dc.z, dc.w), v, RG);
+    const float4 dc = pix[p];   // (dC0, dC1, 1, dC2)
+    const float cc = (float)(p % kBlkW) - 0.5f * (float)(kBlkW - 1);   // column about the centre
+    R1[y] = fmaf(cc, v.x, R1[y]);
+    R2[y] = fmaf(cc * cc, v.x, R2[y]);
+    RG[y] = __ffma2_rn(make_float2(dc.z, dc.w), v, RG[y]);
     G01 = __ffma2_rn(make_float2(dc.x, dc.y), make_float2(v.y, v.y), G01);
   }
-  const float R0 = RG.x, G0 = G01.x, G1 = G01.y, G2 = RG.y;
-  const float rr = (float)r - 0.5f * (float)(kSubH - 1);      // row about the centre
+  const float ra = 2.f * (float)r - 0.5f * (float)(kSubH - 1), rb = ra + 1.f;   // rows about the centre
   // moments of dq in (c, r) about the centre: 1, c, r, c^2, c r, r^2; then dL/dC . w
-  float m[9] = {R0, R1, rr * R0, R2, rr * R1, rr * rr * R0, G0, G1, G2};
+  float m[9] = {RG[0].x + RG[1].x,
+                R1[0] + R1[1],
+                fmaf(ra, RG[0].x, rb * RG[1].x),
+                R2[0] + R2[1],
+                fmaf(ra, R1[0], rb * R1[1]),
+                fmaf(ra * ra, RG[0].x, rb * rb * RG[1].x),
+                G01.x,
+                G01.y,
+                RG[0].y + RG[1].y};
 #pragma unroll
-  for (int o = kSlots; o < 32; o <<= 1)
-#pragma unroll
-    for (int q = 0; q < 9; ++q) m[q] += __shfl_xor_sync(0xffffffffu, m[q], o);
-  if (lane < k) {
-    const int j = ws.slot_j[lane];
-    const float U = s_e[j].a.x - xc, V = s_e[j].a.y - yc;   // dx = U - c, dy = V - r
+  for (int q = 0; q < 9; ++q) m[q] += __shfl_xor_sync(0xffffffffu, m[q], kSlots);
+  const uint32_t off = reinterpret_cast<const uint16_t*>(ws.slot[h])[s];
+  if (r == 0 && s < k && off != null_off) {
+    const Entry& en = entry_at(s_e, off);
+    // dx = U - c, dy = V - r
+    const float U = en.a.x - (pm.x0 + (float)(h * kBlkW) + 0.5f * (float)(kBlkW - 1));
+    const float V = en.a.y - (pm.y0 + 0.5f * (float)(kSubH - 1));
     float g[9];
     g[0] = fmaf(U, m[0], -m[1]);                          // sum dq dx
     g[1] = fmaf(V, m[0], -m[2]);                          // sum dq dy
@@ -344,7 +471,7 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
     g[6] = m[6];
     g[7] = m[7];
     g[8] = m[8];
-    float* dst = a.grad_rec + (size_t)__float_as_uint(s_e[j].c.w) * 12;
+    float* dst = a.grad_rec + (size_t)__float_as_uint(en.c.w) * 12;
     // a record is 48 bytes, 16-byte aligned: floats 0-3 and 4-7 as vectors
     red_add4(dst, g[0], g[1], g[2], g[3]);
     red_add4(dst + 4, g[4], g[5], g[6], g[7]);
@@ -361,10 +488,11 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
 template <bool kRecompute>
 __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm, float pxc, float pyc,
                                          uint2 range, bool inside, const float* Cf, const float* dC,
-                                         uint32_t bound, bool staged, Entry* s_e, WarpScratch& ws,
-                                         bool recorded = false) {
+                                         uint32_t bound, bool staged, Entry* s_e, WarpScratch& ws) {
   const int B = a.batch;
+  const uint32_t* cull = cull_of(a, s_e) + pm.block * cull_stride(B);
   const int lane = threadIdx.x & 31;
+  const uint32_t null_off = (uint32_t)(B * (int)sizeof(Entry));
   // dL/dalpha_i = sum_c dC_c (c_i T_i - S_c / (1 - alpha_i)) with S the colour
   // behind entry i, S_c = C_c - P_c (P the running front-to-back sum), so
   // sum_c dC_c S_c = D0 - Q with D0 = dC . C and Q = dC . P kept as a scalar.
@@ -375,72 +503,74 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm,
   if (kRecompute || !inside) bound = inside ? 0xffffffffu : 0u;   // outside the image: an empty walk
   // (dC0, dC1, 1, dC2): pass 2 pairs the 1 with dq and dC2 with w
   ws.pix[lane + (lane >> 3)] = make_float4(dC[0], dC[1], 1.f, dC[2]);
-  int k = 0;          // slots filled (warp-uniform)
+  int k0 = 0;         // slots filled (warp-uniform, a multiple of kStep)
 
   for (uint32_t start = range.x; start < range.y; start += B) {
     // a staged list is already in shared memory (read-only): no CTA barrier
     if (!staged && __syncthreads_count(done) == (int)blockDim.x) break;
     const int cnt = (int)min((uint32_t)B, range.y - start);
     if (!staged) {
-      load_batch(a, start, cnt, s_e);
+      load_batch(a, start, cnt, pm.tx0, pm.ty0, s_e);
       __syncthreads();
     }
     if (__all_sync(0xffffffffu, done)) continue;
-    // entries j < lim of this batch lie within the pixel's walk
-    const int lim = (int)min((uint32_t)cnt, bound - min(bound, start - range.x));
-    for (int base = 0; base < cnt; base += 32) {
-      // the sub-block test of these 32 entries: recorded by the fused
-      // kernel's forward walk (the list is the same), else evaluated here
-      const uint32_t g = (start - range.x + base) >> 5;
-      uint32_t mask;
-      if (recorded && g < kCullGroups) {
-        mask = ws.cull[g];
-      } else {
-        const int jl = base + lane;
-        const bool rel = jl < cnt && reaches<true>(pm, s_e[jl].a, s_e[jl].b, s_e[jl].c);
-        mask = __ballot_sync(0xffffffffu, rel);
-      }
-      while (mask) {
-        const int j = base + __ffs(mask) - 1;
-        mask &= mask - 1;
-        // Branch-free, as in the forward: alpha = 0 for a pixel that skips
-        // the entry or is finished, which leaves T and Q unchanged and gives
-        // zero dq and w.
-        const float4 ra = s_e[j].a, rb = s_e[j].b;
-        const float blue = s_e[j].c.x;
-        float2 d;
-        const float q = entry_q(ra, rb, npix, d);
-        const bool vis = (kRecompute ? !done : j < lim) && q >= kQMin;
-        const float e = ex2_approx(q);
-        const float alpha = vis ? fminf(kAlphaMax, e) : 0.f;
-        const float om = __fsub_rn(1.f, alpha);
-        const float2 tw = __fmul2_rn(make_float2(T, T), make_float2(om, alpha));   // (T (1 - alpha), alpha T)
-        const float test_T = tw.x;
-        // stored walk: never a stop inside it, and alpha = 0 past it
-        const bool stop = kRecompute && test_T < kTMin;
-        const float w = stop ? 0.f : tw.y;
-        const float G = dC[0] * rb.z + dC[1] * rb.w + dC[2] * blue;
-        Q = fmaf(w, G, Q);   // now includes this entry: D0 - Q is behind it
-        const float dLda = T * G - (D0 - Q) * __fdividef(1.f, om);
-        // dL/dq / ln 2 (the factor ln 2 of d 2^q / dq is applied by the
-        // per-Gaussian backward); no gradient through the 0.99 clamp; alpha = 0
-        // (skipped, off the walk) gives dq = 0
-        const float dq = (!stop && e <= kAlphaMax) ? dLda * alpha : 0.f;
-        T = stop ? T : test_T;
-        if (kRecompute) done = done || stop;
-        ws.dqw[k][lane] = make_float2(dq, w);
-        if (lane == 0) ws.slot_j[k] = j;
-        if (++k == kSlots) {
-          flush_slots(a, ws, k, s_e, 0.5f * (pm.x0 + pm.x1), 0.5f * (pm.y0 + pm.y1));
-          k = 0;
+    // entries at offsets below lim of this batch lie within the pixel's walk
+    const uint32_t lim = min((uint32_t)cnt, bound - min(bound, start - range.x)) * (uint32_t)sizeof(Entry);
+    for (int c0 = 0; c0 < cnt; c0 += kChunk) {
+      const int steps = fill_lists(cull, B, c0, cnt, ws.lists);
+      bool all = false;
+#pragma unroll 1
+      for (int i = 0; i < steps && !all; i += kStep) {
+        const uint2 quad = list_quad(ws.lists, i);
+        if ((lane & 15) == 0) ws.slot[lane >> 4][k0 / kStep] = quad;
+        float2* slot = &ws.dqw[k0][lane];
+        uint32_t off = 0;
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) {
+          // Branch-free, as in the forward: alpha = 0 for a pixel that skips
+          // the entry or is finished, which leaves T and Q unchanged and gives
+          // zero dq and w.
+          off = quad_off(quad, k);
+          const Entry& en = entry_at(s_e, off);
+          const float4 ra = en.a, rb = en.b;
+          const float blue = en.c.x;
+          float2 d;
+          const float q = entry_q(ra, rb, npix, d);
+          const bool vis = (kRecompute ? !done : off < lim) && q >= kQMin;
+          const float e = ex2_approx(q);
+          const float alpha = vis ? fminf(kAlphaMax, e) : 0.f;
+          const float om = __fsub_rn(1.f, alpha);
+          const float2 tw = __fmul2_rn(make_float2(T, T), make_float2(om, alpha));   // (T (1 - alpha), alpha T)
+          const float test_T = tw.x;
+          // stored walk: never a stop inside it, and alpha = 0 past it
+          const bool stop = kRecompute && test_T < kTMin;
+          const float w = stop ? 0.f : tw.y;
+          const float G = dC[0] * rb.z + dC[1] * rb.w + dC[2] * blue;
+          Q = fmaf(w, G, Q);   // now includes this entry: D0 - Q is behind it
+          const float dLda = T * G - (D0 - Q) * rcp_approx(om);
+          // dL/dq / ln 2 (the factor ln 2 of d 2^q / dq is applied by the
+          // per-Gaussian backward); no gradient through the 0.99 clamp; alpha = 0
+          // (skipped, off the walk) gives dq = 0
+          const float dq = (!stop && e <= kAlphaMax) ? dLda * alpha : 0.f;
+          T = stop ? T : test_T;
+          if (kRecompute) done = done || stop;
+          slot[k * 33] = make_float2(dq, w);
         }
+        k0 += kStep;
+        if (k0 == kSlots) {
+          flush_slots(a, ws, kSlots, s_e, pm, null_off);
+          k0 = 0;
+        }
+        // (a padded list says nothing about the walk's end)
+        all = __all_sync(0xffffffffu, kRecompute ? done : off >= lim && off != null_off);
       }
-      if (__all_sync(0xffffffffu, kRecompute ? done : base + 32 >= lim)) break;
+      if (all || __all_sync(0xffffffffu, kRecompute ? done : (uint32_t)(c0 + kChunk) * (uint32_t)sizeof(Entry) >= lim))
+        break;
     }
     if (!kRecompute) done = done || start - range.x + cnt >= bound;
-    if (k) {   // the slots refer to this batch's shared-memory records
-      flush_slots(a, ws, k, s_e, 0.5f * (pm.x0 + pm.x1), 0.5f * (pm.y0 + pm.y1));
-      k = 0;
+    if (k0) {   // the slots refer to this batch's shared-memory records
+      flush_slots(a, ws, k0, s_e, pm, null_off);
+      k0 = 0;
     }
   }
 }
@@ -450,8 +580,6 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm,
 // pixel's stored number of entries.
 template <bool kRecompute>
 __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint32_t gt, float4* s_mem) {
-  const int B = a.batch;
-
   const CamRec& cam = a.cams[find_camera(a.cams, a.n_cams, gt)];
   const uint32_t local = gt - (uint32_t)cam.tile_offset;
   const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h);
@@ -473,7 +601,7 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint32_t gt, 
     }
     if (!kRecompute) bound = a.nwalk[cam.pixel_base + pix];
   }
-  WarpScratch* ws = reinterpret_cast<WarpScratch*>(s_mem + 3 * B);
+  WarpScratch* ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem));
   bwd_walk<kRecompute>(a, pm, pxc, pyc, range, inside, Cf, dC, bound, false, reinterpret_cast<Entry*>(s_mem),
                        ws[threadIdx.x >> 5]);
 }
@@ -491,7 +619,6 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint32_t gt, 
 // blend_bwd in stored-walk mode, bit for bit up to the order of the atomic
 // additions.
 __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint32_t gt, float4* s_mem) {
-  const int B = a.batch;
   Entry* s_e = reinterpret_cast<Entry*>(s_mem);
   __shared__ float s_red[16];
 
@@ -503,10 +630,10 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint32_t gt
   const uint2 range = a.ranges[gt];
   const int lane = threadIdx.x & 31;
 
-  WarpScratch& ws = reinterpret_cast<WarpScratch*>(s_mem + 3 * B)[threadIdx.x >> 5];
+  WarpScratch& ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem))[threadIdx.x >> 5];
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
   const FwdPixel fp =
-      fwd_walk<false>(a, pm, pxc, pyc, range, inside, s_e, n_eval, n_comp, n_warp, ws.cull);
+      fwd_walk<false>(a, pm, pxc, pyc, range, inside, s_e, ws.lists, n_eval, n_comp, n_warp);
   float Cf[3] = {0.f, 0.f, 0.f}, dC[3] = {0.f, 0.f, 0.f};
   float l1 = 0.f;
   if (inside) {
@@ -531,10 +658,10 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint32_t gt
     }
     if (a.nwalk) a.nwalk[cam.pixel_base + pix] = fp.walked;
   }
-  l1 = warp_sum(l1);
+  l1 = sub_block_sum(l1);
   if (lane == 0) s_red[threadIdx.x >> 5] = l1;
   __syncwarp();
-  bwd_walk<false>(a, pm, pxc, pyc, range, inside, Cf, dC, fp.walked, fp.staged, s_e, ws, true);
+  bwd_walk<false>(a, pm, pxc, pyc, range, inside, Cf, dC, fp.walked, fp.staged, s_e, ws);
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
@@ -583,7 +710,12 @@ __global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a
 // fit on the GPU at once, each taking tiles from a device counter until all
 // cameras' tiles are done.
 template <bool kCount, bool kStore>
-__global__ void __launch_bounds__(512) blend_fwd_kernel(BlendArgs a) {
+// (the forward's registers: 64 / 48 / 40 give 617 / 599 / 606 us for 20 views of
+// 183k Gaussians at 1024^2)
+#ifndef SIXDGS_FWD_MAXNREG
+#define SIXDGS_FWD_MAXNREG 48
+#endif
+__global__ void __maxnreg__(SIXDGS_FWD_MAXNREG) blend_fwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
   for_each_blend_tile(a, [&](uint32_t gt) { blend_fwd_tile<kCount, kStore>(a, gt, s_mem); });
 }
@@ -593,8 +725,6 @@ __global__ void __maxnreg__(SIXDGS_BWD_MAXNREG) blend_bwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
   for_each_blend_tile(a, [&](uint32_t gt) { blend_bwd_tile<kRecompute>(a, gt, s_mem); });
 }
-
-static int blend_smem(int batch) { return batch * 3 * (int)sizeof(float4); }
 
 // Batches near or above 48 KB of shared memory (with the kernels' static
 // shared memory) need the opt-in limit.
@@ -612,11 +742,11 @@ static int resident_grid(const void* fn, int threads, int smem, int64_t tiles) {
   return (int)std::min<int64_t>(g, tiles);
 }
 
-// scratch: the backward walk's per-warp shared memory (0 for the forward)
+// scratch: the backward walk's per-warp shared memory (the forward: lists only)
 template <typename K>
 static void launch_blend(K kernel, const BlendArgs& a, int64_t total_tiles, bool scratch, cudaStream_t stream) {
   const int threads = a.tile_w * a.tile_h;
-  const int smem = blend_smem(a.batch) + (scratch ? bwd_scratch_bytes(threads) : 0);
+  const int smem = stage_bytes(a.batch, threads / (kBlkW * kSubH)) + threads / 32 * (int)(scratch ? sizeof(WarpScratch) : sizeof(WalkLists));
   allow_smem((const void*)kernel, smem);
   if (a.tile_queue) {
     cudaMemsetAsync(a.tile_queue, 0, sizeof(uint32_t), stream);
