@@ -19,7 +19,7 @@ enum {
   WS_TILE = 14,        // counters of every tile
   WS_ZERO_END = 15,
   WS_COUNTERS = 16,    // word 32: persistent blend queue
-  WS_ORDER = 18,       // tiles, longest lists first
+  WS_ORDER = 18,       // TileWork of every tile, longest lists first
   WS_VIS = 19,         // visible queue of the projection (16 bytes an entry)
   WS_DUP = 20,         // (depth, pair) of every duplicate, grouped by tile
   WS_SORT_K = 21,      // SIXDGS_WS_SORTEDKEY
@@ -224,7 +224,7 @@ sixdgs_status sixdgs_plan_init(int64_t n, int32_t sh_degree, const sixdgs_camera
   take(WS_SCAN, (tiles + kScanTile - 1) / kScanTile * 8);
   take(WS_TILE, tiles * (int64_t)sizeof(TileCounters));
   plan->off[WS_ZERO_END] = o;
-  take(WS_ORDER, tiles * 4);
+  take(WS_ORDER, tiles * 16);
   take(WS_VIS, n_pairs * 16);
   take(WS_VIS_COUNT, (n + kStageTile - 1) / kStageTile * 4);
   take(WS_DUP, dup_capacity * 8);
@@ -308,6 +308,7 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   BinArgs a;
   a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
+  a.n_cams = p->n_cams;
   a.n = (uint32_t)p->n;
   a.total_tiles = (uint32_t)p->total_tiles;
   a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
@@ -317,7 +318,7 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
   a.segment_size = (uint32_t)(kStageTile * p->n_cams);
   a.state = ws_ptr<uint32_t>(ws, p, WS_STATE);
   a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN);
-  a.order = ws_ptr<uint32_t>(ws, p, WS_ORDER);
+  a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
   a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
   a.capacity = (uint64_t)p->dup_capacity;
   a.dup = ws_ptr<uint64_t>(ws, p, WS_DUP);
@@ -342,7 +343,8 @@ static BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
   a.n_pairs = (uint32_t)p->n_pairs;
   a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
   a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
-  a.order = ws_ptr<uint32_t>(ws, p, WS_ORDER);
+  a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
+  a.n_busy = ws_ptr<uint32_t>(ws, p, WS_STATE) + kBinOver + kBinLevels;
   for (int i = 0; i < 3; ++i) a.bg[i] = p->settings.bg[i];
   const double norm = p->settings.loss_norm > 0.f ? (double)p->settings.loss_norm
                                                    : 3.0 * (double)p->total_pixels;

@@ -50,6 +50,23 @@ struct __align__(16) PairRec {
   float4 a, b, c;
 };
 
+// What the sort and the blend need to know of a tile, in one 16-byte load:
+// (global tile id, list start, list end, camera).
+__device__ __forceinline__ uint4 tile_work(uint32_t tile, uint2 range, uint32_t cam) {
+  return make_uint4(tile, range.x, range.y, cam);
+}
+
+// Camera of global tile gt.
+__device__ __forceinline__ int find_camera(const CamRec* cams, int n_cams, uint32_t gt) {
+  int lo = 0, hi = n_cams - 1;
+  while (lo < hi) {
+    int mid = (lo + hi + 1) >> 1;
+    if ((uint32_t)cams[mid].tile_offset <= gt) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 __device__ __forceinline__ void raise_status(int32_t* status, int code) {
   if (status) atomicOr(status, 1 << code);
 }

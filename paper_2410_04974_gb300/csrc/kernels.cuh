@@ -51,10 +51,12 @@ enum BinWord {
   kBinOver = 130,        // tiles with lists above 4096, 2048, 1024, 512 and 0 entries
   kBinWords = 192
 };
+constexpr int kBinLevels = 4;   // 4096, 2048, 1024, 512 entries: the sizes of the sorting teams
 
 // Per-tile lists from the projection's tile counts and visible queue.
 struct BinArgs {
   const CamRec* cams;
+  int32_t n_cams;
   uint32_t n;                      // Gaussians per camera
   uint32_t total_tiles;
   TileCounters* tile;
@@ -62,9 +64,10 @@ struct BinArgs {
   const uint32_t* vis_count;
   uint32_t segments;               // of the queue
   uint32_t segment_size;
+  uint32_t scatter_grid;           // CTAs that share the segments (set by the launch)
   uint32_t* state;                 // kBinWords words
   unsigned long long* scan_state;  // one word per scan block
-  uint32_t* order;                 // tiles, longest list class first
+  uint4* order;                    // TileWork of every tile, longest list class first
   uint2* ranges;
   uint64_t capacity;
   uint64_t* dup;                   // (depth, pair) of every duplicate, grouped by tile
@@ -83,7 +86,8 @@ struct BlendArgs {
   uint32_t n_pairs;
   const uint32_t* sorted;   // pair index per list entry
   const uint2* ranges;
-  const uint32_t* order;    // tiles, longest lists first
+  const uint4* order;       // TileWork of every tile, longest lists first
+  const uint32_t* n_busy;   // tiles with a list (the others come last)
   float bg[3];
   float* images;
   const float* targets;
@@ -152,7 +156,7 @@ void launch_project_fwd(const ProjectArgs& a, cudaStream_t stream);
 void launch_scale_rotation(const ScaleRotationArgs& a, cudaStream_t stream);
 void launch_cond_cache(const CondCacheArgs& a, cudaStream_t stream);
 void launch_peak_probe(int kind, int64_t iters, float* out, int blocks, cudaStream_t stream);
-cudaError_t launch_bin(const BinArgs& a, int sms, cudaStream_t stream);
+cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream);
 void launch_blend_fwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_blend_fused(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_blend_bwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);

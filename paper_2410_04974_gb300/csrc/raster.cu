@@ -43,16 +43,6 @@ constexpr int kSubW = 8;   // warp sub-block: 8 x 4 pixels
 constexpr int kSubH = 4;
 constexpr int kBlkW = 4;   // half-warp block: 4 x 4 pixels
 
-__device__ __forceinline__ int find_camera(const CamRec* cams, int n_cams, uint32_t gt) {
-  int lo = 0, hi = n_cams - 1;
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if ((uint32_t)cams[mid].tile_offset <= gt) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 // Pixel of this thread and the pixel-centre box of its warp's sub-block.
 struct PixelMap {
   int px, py;
@@ -61,8 +51,9 @@ struct PixelMap {
   int block;      // the warp's left block in the tile
 };
 
-__device__ __forceinline__ PixelMap map_pixel(int tile_w, int tx, int ty, int tile_h) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// warp: sub-block of the tile (row-major).
+__device__ __forceinline__ PixelMap map_pixel(int tile_w, int tx, int ty, int tile_h, int warp) {
+  const int lane = threadIdx.x & 31;
   const int sub_per_row = tile_w / kSubW;
   const int sx = (warp % sub_per_row) * kSubW, sy = (warp / sub_per_row) * kSubH;
   PixelMap m;
@@ -151,6 +142,14 @@ __device__ __forceinline__ char* scratch_of(const BlendArgs& a, void* s_mem) {
   return reinterpret_cast<char*>(s_mem) + stage_bytes(a.batch, blocks_of(a));
 }
 
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Stages list entries [start, start + cnt) and their blocks' ballots.
 // (x0, y0): first pixel centre of the tile.
 __device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, int cnt, float x0, float y0,
@@ -158,20 +157,37 @@ __device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, i
   if (threadIdx.x == 0) null_entry(s_e[a.batch], 0u);
   const int lane = threadIdx.x & 31, blocks = blocks_of(a);
   uint32_t* cull = cull_of(a, s_e);
+  // the records go to shared memory by asynchronous copies, which hold no
+  // registers, all of a thread's in flight together
+  for (int i0 = threadIdx.x; i0 < cnt; i0 += 2 * blockDim.x) {
+    uint32_t p[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int i = i0 + u * blockDim.x;
+      p[u] = i < cnt ? a.sorted[start + i] : 0xffffffffu;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (p[u] < a.n_pairs) {
+        Entry* e = s_e + i0 + u * blockDim.x;
+        const PairRec* r = a.rec + p[u];
+        copy_async16(&e->a, &r->a);
+        copy_async16(&e->b, &r->b);
+        copy_async16(&e->c, &r->c);
+      }
+  }
+  copy_async_wait();
   for (int i0 = threadIdx.x & ~31; i0 < cnt; i0 += blockDim.x) {
     const int i = i0 + lane;
     uint32_t mask = 0u;
     if (i < cnt) {
       const uint32_t p = a.sorted[start + i];
+      Entry& e = s_e[i];
       if (p < a.n_pairs) {
-        const PairRec& r = a.rec[p];
-        const float4 ra = r.a, rb = r.b, rc = r.c;
-        s_e[i].a = ra;
-        s_e[i].b = rb;
-        s_e[i].c = make_float4(rc.x, rc.y, rc.z, __uint_as_float(p));
-        mask = block_mask(ra, rb, rc, x0, y0, a.tile_w, a.tile_h / kSubH);
+        mask = block_mask(e.a, e.b, e.c, x0, y0, a.tile_w, a.tile_h / kSubH);
+        e.c.w = __uint_as_float(p);
       } else {  // unreachable for a consistent sort
-        null_entry(s_e[i], 0u);
+        null_entry(e, 0u);
       }
     }
     uint32_t word = 0u;   // of block `lane`
@@ -339,19 +355,19 @@ __device__ __forceinline__ float sub_block_sum(float v) {
   return v;
 }
 
-// Forward blend of global tile gt by the calling CTA.
+// Forward blend of tile tw (tile_work) by the calling CTA.
 template <bool kCount, bool kStore>
-__device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint32_t gt, float4* s_mem) {
+__device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
   Entry* s_e = reinterpret_cast<Entry*>(s_mem);
   WalkLists* lists = reinterpret_cast<WalkLists*>(scratch_of(a, s_mem));
   __shared__ float s_red[16];
 
-  const CamRec& cam = a.cams[find_camera(a.cams, a.n_cams, gt)];
-  const uint32_t local = gt - (uint32_t)cam.tile_offset;
-  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h);
+  const CamRec& cam = a.cams[tw.w];
+  const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
+  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h, threadIdx.x >> 5);
   const bool inside = pm.px < cam.width && pm.py < cam.height;
   const float pxc = (float)pm.px + 0.5f, pyc = (float)pm.py + 0.5f;
-  const uint2 range = a.ranges[gt];
+  const uint2 range = make_uint2(tw.y, tw.z);
   const int lane = threadIdx.x & 31;
 
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
@@ -575,17 +591,17 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm,
   }
 }
 
-// Backward blend of global tile gt by the calling CTA.  kRecompute: re-derive
+// Backward blend of tile tw by the calling CTA.  kRecompute: re-derive
 // the stop from the transmittance (no per-pixel state); otherwise walk each
 // pixel's stored number of entries.
 template <bool kRecompute>
-__device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint32_t gt, float4* s_mem) {
-  const CamRec& cam = a.cams[find_camera(a.cams, a.n_cams, gt)];
-  const uint32_t local = gt - (uint32_t)cam.tile_offset;
-  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h);
+__device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
+  const CamRec& cam = a.cams[tw.w];
+  const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
+  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h, threadIdx.x >> 5);
   const bool inside = pm.px < cam.width && pm.py < cam.height;
   const float pxc = (float)pm.px + 0.5f, pyc = (float)pm.py + 0.5f;
-  const uint2 range = a.ranges[gt];
+  const uint2 range = make_uint2(tw.y, tw.z);
 
   float Cf[3] = {0.f, 0.f, 0.f}, dC[3] = {0.f, 0.f, 0.f};
   uint32_t bound = range.y - range.x;
@@ -606,8 +622,8 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint32_t gt, 
                        ws[threadIdx.x >> 5]);
 }
 
-// Forward blend, fused L1 loss and backward blend of global tile gt by the
-// calling CTA, for the training step whose loss is the L1 term (section
+// Forward blend, fused L1 loss and backward blend of tile tw by the calling
+// CTA, for the training step whose loss is the L1 term (section
 // 4.4): each pixel's dL/dC = sign(C - target) / M is known as soon as its
 // forward walk ends, so the backward replay follows in the same CTA with C,
 // dL/dC and the walk length in registers, and a list that fitted in one
@@ -618,16 +634,16 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint32_t gt, 
 // dL/dC, loss and record gradients equal those of raster_fwd followed by
 // blend_bwd in stored-walk mode, bit for bit up to the order of the atomic
 // additions.
-__device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint32_t gt, float4* s_mem) {
+__device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
   Entry* s_e = reinterpret_cast<Entry*>(s_mem);
   __shared__ float s_red[16];
 
-  const CamRec& cam = a.cams[find_camera(a.cams, a.n_cams, gt)];
-  const uint32_t local = gt - (uint32_t)cam.tile_offset;
-  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h);
+  const CamRec& cam = a.cams[tw.w];
+  const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
+  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h, threadIdx.x >> 5);
   const bool inside = pm.px < cam.width && pm.py < cam.height;
   const float pxc = (float)pm.px + 0.5f, pyc = (float)pm.py + 0.5f;
-  const uint2 range = a.ranges[gt];
+  const uint2 range = make_uint2(tw.y, tw.z);
   const int lane = threadIdx.x & 31;
 
   WarpScratch& ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem))[threadIdx.x >> 5];
@@ -678,15 +694,79 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint32_t gt
 #ifndef SIXDGS_BWD_MAXNREG
 #define SIXDGS_BWD_MAXNREG 64
 #endif
-// Tiles are taken in the binning's order, longest lists first, so that the
-// launch does not end on a few CTAs that started a long list late: 917 -> 858 us
-// (fused kernel, 300k / 8 x 800^2), 68 -> 52 us (forward, one 1408^2 view of
-// 175k Gaussians).
-template <typename Tile>
-__device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile tile) {
+// Tiles without a list, one per warp from order[first] on: the background, and
+// with targets its loss and dL/dC (the same sums as the blends' own).
+template <bool kStore>
+__device__ __forceinline__ void blend_empty(const BlendArgs& a, uint32_t first) {
+  __shared__ double s_loss[16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double loss = 0.0;
+  if (first + warp < a.total_tiles) {
+    const uint4 tw = a.order[first + warp];
+    const CamRec& cam = a.cams[tw.w];
+    const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
+    const int tx = local % cam.tiles_x, ty = local / cam.tiles_x;
+    const int64_t hw = (int64_t)cam.width * cam.height;
+    float* img = a.images + 3 * cam.pixel_base;
+#pragma unroll 4
+    for (int b = 0; b < (int)blockDim.x / 32; ++b) {
+      const PixelMap pm = map_pixel(a.tile_w, tx, ty, a.tile_h, b);
+      const int64_t pix = (int64_t)pm.py * cam.width + pm.px;
+      float l1 = 0.f;
+      if (pm.px < cam.width && pm.py < cam.height) {
+        if (kStore) a.nwalk[cam.pixel_base + pix] = 0u;
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+          img[ch * hw + pix] = a.bg[ch];
+          if (a.targets) {
+            const float d = a.bg[ch] - a.targets[3 * cam.pixel_base + ch * hw + pix];
+            if (a.grad_images)
+              a.grad_images[3 * cam.pixel_base + ch * hw + pix] =
+                  d > 0.f ? a.inv_count : (d < 0.f ? -a.inv_count : 0.f);
+            l1 += fabsf(d);
+          }
+        }
+      }
+      if (a.targets) loss += sub_block_sum(l1);
+    }
+  }
+  if (!a.targets) return;
+  if (lane == 0) s_loss[warp] = loss * (double)a.inv_count;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) sum += s_loss[w];
+    atomicAdd(a.loss, sum);
+  }
+}
+
+// Work unit u of a blend launch.  Tiles are taken in the binning's order,
+// longest lists first, so that the launch does not end on a few CTAs that
+// started a long list late (917 -> 858 us for the fused kernel at 300k / 8 x
+// 800^2, 68 -> 52 us for the forward of one 1408^2 view of 175k Gaussians).
+// The tiles without a list, 70% of that frame's, come last, one per warp of a
+// CTA: a CTA each spent most of its time waiting for a handful of loads.  With
+// that, the one-load tile record and the asynchronous staging of a batch
+// (load_batch): fused kernel 722 -> 663 us at 300k / 8 x 800^2, forward 600 ->
+// 536 us for 20 views of 183k Gaussians at 1024^2.
+template <typename Tile, typename Empty>
+__device__ __forceinline__ bool blend_unit(const BlendArgs& a, uint32_t u, Tile tile, Empty empty) {
+  const uint4 tw = a.order[min(u, a.total_tiles - 1)];
+  const uint32_t busy = min(*a.n_busy, a.total_tiles);
+  if (u < busy) {
+    if (tw.x < a.total_tiles) tile(tw);
+    return true;
+  }
+  const uint32_t first = busy + (u - busy) * (blockDim.x / 32);
+  if (first >= a.total_tiles) return false;
+  empty(first);
+  return true;
+}
+
+template <typename Tile, typename Empty>
+__device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile tile, Empty empty) {
   if (!a.tile_queue) {
-    const uint32_t gt = a.order[blockIdx.x];
-    if (gt < a.total_tiles) tile(gt);
+    blend_unit(a, blockIdx.x, tile, empty);
     return;
   }
   __shared__ uint32_t s_next;
@@ -694,16 +774,19 @@ __device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile til
     if (threadIdx.x == 0) s_next = atomicAdd(a.tile_queue, 1u);
     __syncthreads();
     const uint32_t next = s_next;
-    if (next >= a.total_tiles) break;
-    const uint32_t gt = a.order[next];
-    if (gt < a.total_tiles) tile(gt);
+    if (!blend_unit(a, next, tile, empty)) break;
     __syncthreads();
   }
 }
 
 __global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  for_each_blend_tile(a, [&](uint32_t gt) { blend_fused_tile(a, gt, s_mem); });
+  for_each_blend_tile(
+      a, [&](uint4 tw) { blend_fused_tile(a, tw, s_mem); },
+      [&](uint32_t first) {
+        if (a.nwalk) blend_empty<true>(a, first);
+        else blend_empty<false>(a, first);
+      });
 }
 
 // One CTA per tile (grid = tiles), or persistent: a grid of as many CTAs as
@@ -717,13 +800,16 @@ template <bool kCount, bool kStore>
 #endif
 __global__ void __maxnreg__(SIXDGS_FWD_MAXNREG) blend_fwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  for_each_blend_tile(a, [&](uint32_t gt) { blend_fwd_tile<kCount, kStore>(a, gt, s_mem); });
+  for_each_blend_tile(
+      a, [&](uint4 tw) { blend_fwd_tile<kCount, kStore>(a, tw, s_mem); },
+      [&](uint32_t first) { blend_empty<kStore>(a, first); });
 }
 
 template <bool kRecompute>
 __global__ void __maxnreg__(SIXDGS_BWD_MAXNREG) blend_bwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  for_each_blend_tile(a, [&](uint32_t gt) { blend_bwd_tile<kRecompute>(a, gt, s_mem); });
+  for_each_blend_tile(
+      a, [&](uint4 tw) { blend_bwd_tile<kRecompute>(a, tw, s_mem); }, [](uint32_t) {});
 }
 
 // Batches near or above 48 KB of shared memory (with the kernels' static

@@ -141,7 +141,6 @@ __device__ __forceinline__ uint32_t length_class(uint32_t len) {
   const uint32_t frac = l >= 2u ? (m >> (l - 2u)) & 3u : (l == 1u ? (m & 1u) * 2u : 0u);
   return min(1u + 4u * l + frac, (uint32_t)kClasses - 1u);
 }
-constexpr int kBinLevels = 4;   // 4096, 2048, 1024, 512 entries: the sizes of the sorting teams
 
 // Adds this block's tiles to per-class counters in shared memory; returns the
 // tile's rank within its class and block.  Called by the whole block, tiles
@@ -230,10 +229,9 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
   __shared__ uint32_t s_vis;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) s_vis = 0u;
-  const uint32_t blocks = (a.total_tiles + kScatterThreads - 1) / kScatterThreads;
-  if (blockIdx.x < blocks) {
-    // tile order: longest class first, any order within a class (it decides
-    // when a tile is worked on, never a result)
+  if (blockIdx.x >= a.scatter_grid) {
+    // these CTAs build the tile order: longest class first, any order within a
+    // class (it decides when a tile is worked on, never a result)
     if (warp == 0) {   // tiles of longer classes: a suffix sum over the 64 classes
       const uint32_t c0 = a.state[kBinClass + lane], c1 = a.state[kBinClass + 32 + lane];
       uint32_t x0 = c0, x1 = c1;
@@ -249,38 +247,34 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
       s_longer[lane] = x0 - c0 + high;
       s_longer[32 + lane] = x1 - c1;
     }
+    if (tid < kClasses) s_class[tid] = 0u;
+    const uint32_t t = (blockIdx.x - a.scatter_grid) * kScatterThreads + tid;
+    const bool valid = t < a.total_tiles;
+    const uint2 r = valid ? a.ranges[t] : make_uint2(0u, 0u);
+    const uint32_t cam = valid ? (uint32_t)find_camera(a.cams, a.n_cams, t) : 0u;
     __syncthreads();
-    if (blockIdx.x == 0 && tid <= kBinLevels) {
+    const uint32_t cls = length_class(r.y - r.x);
+    const uint32_t rank = count_class(cls, valid, s_class);
+    __syncthreads();
+    if (tid < kClasses && s_class[tid])
+      s_base[tid] = s_longer[tid] + atomicAdd(&a.state[kBinCursor + tid], s_class[tid]);
+    __syncthreads();
+    if (valid) {
+      const uint32_t at = s_base[cls] + rank;
+      if (at < a.total_tiles) a.order[at] = tile_work(t, r, cam);
+    }
+    if (blockIdx.x == a.scatter_grid) {
       // tiles with lists above the sort's limits: those of the classes beyond
-      const uint32_t limit_class = tid < kBinLevels ? 4u * (12u - (uint32_t)tid) : 0u;
-      a.state[kBinOver + tid] = s_longer[limit_class];
+      if (tid <= kBinLevels) a.state[kBinOver + tid] = s_longer[tid < kBinLevels ? 4 * (12 - tid) : 0];
+      if (tid == 32) a.state[kBinTicket] = 0u;
     }
-    for (uint32_t b = blockIdx.x; b < blocks; b += gridDim.x) {
-      if (tid < kClasses) s_class[tid] = 0u;
-      __syncthreads();
-      const uint32_t t = b * kScatterThreads + tid;
-      const bool valid = t < a.total_tiles;
-      const uint2 r = valid ? a.ranges[t] : make_uint2(0u, 0u);
-      const uint32_t cls = length_class(r.y - r.x);
-      const uint32_t rank = count_class(cls, valid, s_class);
-      __syncthreads();
-      if (tid < kClasses && s_class[tid])
-        s_base[tid] = s_longer[tid] + atomicAdd(&a.state[kBinCursor + tid], s_class[tid]);
-      __syncthreads();
-      if (valid) {
-        const uint32_t at = s_base[cls] + rank;
-        if (at < a.total_tiles) a.order[at] = t;
-      }
-    }
+    // the scan is over: its words are clean for the next call
+    if (tid == 0 && t % kScanTile == 0) a.scan_state[t / kScanTile] = 0ull;
+    return;
   }
-  // the scan is over: its words are clean for the next call
-  const uint32_t scan_blocks = (a.total_tiles + kScanTile - 1) / kScanTile;
-  for (uint32_t i = blockIdx.x * kScatterThreads + tid; i < scan_blocks; i += gridDim.x * kScatterThreads)
-    a.scan_state[i] = 0ull;
-  if (blockIdx.x == 0 && tid == 0) a.state[kBinTicket] = 0u;
 
   uint32_t visible = 0;
-  for (uint32_t seg = blockIdx.x; seg < a.segments; seg += gridDim.x) {
+  for (uint32_t seg = blockIdx.x; seg < a.segments; seg += a.scatter_grid) {
     const uint32_t count = min(a.vis_count[seg], a.segment_size);
     const uint4* vis = a.vis + (size_t)seg * a.segment_size;
     for (uint32_t c0 = 0; c0 < count; c0 += kScatterEntries) {
@@ -681,9 +675,8 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
   for (int l = kBinLevels - 1; l >= 0; --l) over[l] = min(a.state[kBinOver + l], over[l + 1]);
   if (blockIdx.x == 0 && tid < 2 * kClasses) a.state[kBinClass + tid] = 0u;   // clean for the next call
   for (uint32_t u = blockIdx.x / kCluster; u < over[0]; u += gridDim.x / kCluster) {
-    const uint32_t t = a.order[u];
-    const uint2 r = t < a.total_tiles ? a.ranges[t] : make_uint2(0u, 0u);
-    sort_long(a, r.x, r.y - r.x, t, s_key);
+    const uint4 w = a.order[u];
+    sort_long(a, w.y, w.z - w.y, w.x, s_key);
     cluster_sync();
   }
   // units of the rest: one, two, four or eight tiles a CTA
@@ -701,29 +694,28 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
     else if (u < u4) at = over[2] + 4 * (u - u2), end = over[3], teams = 4;
     else at = over[3] + 8 * (u - u4), end = over[4], teams = 8;
     at += threadIdx.x / (kBinThreads / teams);
-    const uint32_t t = at < end ? a.order[at] : 0xffffffffu;
-    const uint2 r = t < a.total_tiles ? a.ranges[t] : make_uint2(0u, 0u);
-    const uint32_t len = min(r.y - r.x, kRun / teams);
+    const uint4 w = at < end ? a.order[at] : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t len = min(w.z - w.y, kRun / teams);
     if (len == 0u) continue;   // (the whole team)
-    if (teams == 1) sort_tile<16, 8>(a, t, r.x, len, s_key);
-    else if (teams == 2) sort_tile<16, 4>(a, t, r.x, len, s_key);
-    else if (teams == 4) sort_tile<16, 2>(a, t, r.x, len, s_key);
-    else if (len > 256u) sort_tile<16, 1>(a, t, r.x, len, s_key);
-    else if (len > 128u) sort_tile<8, 1>(a, t, r.x, len, s_key);
-    else if (len > 64u) sort_tile<4, 1>(a, t, r.x, len, s_key);
-    else sort_tile<2, 1>(a, t, r.x, len, s_key);
+    if (teams == 1) sort_tile<16, 8>(a, w.x, w.y, len, s_key);
+    else if (teams == 2) sort_tile<16, 4>(a, w.x, w.y, len, s_key);
+    else if (teams == 4) sort_tile<16, 2>(a, w.x, w.y, len, s_key);
+    else if (len > 256u) sort_tile<16, 1>(a, w.x, w.y, len, s_key);
+    else if (len > 128u) sort_tile<8, 1>(a, w.x, w.y, len, s_key);
+    else if (len > 64u) sort_tile<4, 1>(a, w.x, w.y, len, s_key);
+    else sort_tile<2, 1>(a, w.x, w.y, len, s_key);
   }
 }
 
 // Grids: the scan has one block per 256 tiles; the scatter at most 16 CTAs per
-// SM, each with the segments of its stride; the sort, which takes its tiles
+// SM, each with the segments of its stride, and one per 128 tiles for the order; the sort, which takes its tiles
 // from a queue, a whole number of clusters, at most 4 CTAs per SM.
-cudaError_t launch_bin(const BinArgs& a, int sms, cudaStream_t stream) {
+cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream) {
   const uint32_t blocks = std::max(1u, (a.total_tiles + kScanTile - 1) / kScanTile);
   bin_scan_kernel<<<blocks, kBinThreads, 0, stream>>>(a);
-  const uint32_t order = (a.total_tiles + kScatterThreads - 1) / kScatterThreads;
-  const uint32_t grid = std::min(std::max(std::max(a.segments, order), 1u), (uint32_t)sms * 16u);
-  bin_scatter_kernel<<<grid, kScatterThreads, 0, stream>>>(a);
+  a.scatter_grid = std::min(a.segments, (uint32_t)sms * 16u);
+  const uint32_t order = std::max(1u, (a.total_tiles + kScatterThreads - 1) / kScatterThreads);
+  bin_scatter_kernel<<<a.scatter_grid + order, kScatterThreads, 0, stream>>>(a);
   const uint32_t most = std::max(1u, (uint32_t)sms * 4u / kCluster);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(most, (std::max(a.total_tiles, 1u) + kCluster - 1) / kCluster) * kCluster);
