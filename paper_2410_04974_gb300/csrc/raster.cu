@@ -43,29 +43,15 @@ constexpr int kSubW = 8;   // warp sub-block: 8 x 4 pixels
 constexpr int kSubH = 4;
 constexpr int kBlkW = 4;   // half-warp block: 4 x 4 pixels
 
-// Pixel of this thread and the pixel-centre box of its warp's sub-block.
-struct PixelMap {
-  int px, py;
-  float x0, y0;   // first pixel centre of the warp
-  float tx0, ty0; // and of the tile
-  int block;      // the warp's left block in the tile
-};
-
-// warp: sub-block of the tile (row-major).
-__device__ __forceinline__ PixelMap map_pixel(int tile_w, int tx, int ty, int tile_h, int warp) {
+// Pixel of this thread in sub-block `warp` (row-major) of tile (tx, ty).
+__device__ __forceinline__ int2 map_pixel(const BlendArgs& a, int tx, int ty, int warp) {
   const int lane = threadIdx.x & 31;
-  const int sub_per_row = tile_w / kSubW;
+  const int sub_per_row = a.tile_w / kSubW;
   const int sx = (warp % sub_per_row) * kSubW, sy = (warp / sub_per_row) * kSubH;
-  PixelMap m;
-  m.px = tx * tile_w + sx + (lane >> 4) * kBlkW + (lane & 3);
-  m.py = ty * tile_h + sy + ((lane >> 2) & 3);
-  m.x0 = (float)(tx * tile_w + sx) + 0.5f;
-  m.y0 = (float)(ty * tile_h + sy) + 0.5f;
-  m.tx0 = (float)(tx * tile_w) + 0.5f;
-  m.ty0 = (float)(ty * tile_h) + 0.5f;
-  m.block = sy / kSubH * (tile_w / kBlkW) + sx / kBlkW;
-  return m;
+  return make_int2(tx * a.tile_w + sx + (lane >> 4) * kBlkW + (lane & 3), ty * a.tile_h + sy + ((lane >> 2) & 3));
 }
+// The negated centre of a pixel, which is what the walks carry.
+__device__ __forceinline__ float2 neg_centre(int2 p) { return make_float2(-((float)p.x + 0.5f), -((float)p.y + 0.5f)); }
 
 // The 4x4 blocks of a tile of tile_w x 4 nby pixels that the entry (u, v, qa,
 // qb), (qc, lo), (hx, hy) can reach, bit y * tile_w / 4 + x: those where q >=
@@ -138,6 +124,11 @@ __device__ __forceinline__ int blocks_of(const BlendArgs& a) { return a.tile_w *
 __device__ __forceinline__ uint32_t* cull_of(const BlendArgs& a, Entry* s_e) {
   return reinterpret_cast<uint32_t*>(s_e + a.batch + 1);
 }
+// The ballots of the warp's left block (its sub-blocks and their blocks are
+// both row-major; its right block's follow).
+__device__ __forceinline__ const uint32_t* warp_cull(const BlendArgs& a, Entry* s_e) {
+  return cull_of(a, s_e) + 2 * (threadIdx.x >> 5) * cull_stride(a.batch);
+}
 __device__ __forceinline__ char* scratch_of(const BlendArgs& a, void* s_mem) {
   return reinterpret_cast<char*>(s_mem) + stage_bytes(a.batch, blocks_of(a));
 }
@@ -151,9 +142,8 @@ __device__ __forceinline__ void copy_async16(void* dst, const void* src) {
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Stages list entries [start, start + cnt) and their blocks' ballots.
-// (x0, y0): first pixel centre of the tile.
-__device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, int cnt, float x0, float y0,
-                                           Entry* s_e) {
+// npix: neg_centre of a pixel of the tile (whose sides are powers of two).
+__device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, int cnt, float2 npix, Entry* s_e) {
   if (threadIdx.x == 0) null_entry(s_e[a.batch], 0u);
   const int lane = threadIdx.x & 31, blocks = blocks_of(a);
   uint32_t* cull = cull_of(a, s_e);
@@ -176,6 +166,8 @@ __device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, i
         copy_async16(&e->c, &r->c);
       }
   }
+  const float x0 = (float)((int)-npix.x & ~(a.tile_w - 1)) + 0.5f;   // first pixel centre of the tile
+  const float y0 = (float)((int)-npix.y & ~(a.tile_h - 1)) + 0.5f;
   copy_async_wait();
   for (int i0 = threadIdx.x & ~31; i0 < cnt; i0 += blockDim.x) {
     const int i = i0 + lane;
@@ -286,27 +278,25 @@ struct FwdPixel {
 };
 
 template <bool kCount>
-__device__ __forceinline__ FwdPixel fwd_walk(const BlendArgs& a, const PixelMap& pm, float pxc, float pyc,
-                                             uint2 range, bool inside, Entry* s_e, WalkLists& lists,
-                                             uint32_t& n_eval, uint32_t& n_comp, uint32_t& n_warp) {
+__device__ __forceinline__ FwdPixel fwd_walk(const BlendArgs& a, float2 npix, uint2 range, bool inside, Entry* s_e,
+                                             WalkLists& lists, uint32_t& n_eval, uint32_t& n_comp,
+                                             uint32_t& n_warp) {
   const int B = a.batch;
-  const uint32_t* cull = cull_of(a, s_e) + pm.block * cull_stride(B);
   float T = 1.f, C2 = 0.f;
   float2 C01 = make_float2(0.f, 0.f);
-  const float2 npix = make_float2(-pxc, -pyc);
   bool done = !inside;
   uint32_t walked = range.y - range.x;
   bool staged = false;
   for (uint32_t start = range.x; start < range.y; start += B) {
     if (__syncthreads_count(done) == (int)blockDim.x) break;
     const int cnt = (int)min((uint32_t)B, range.y - start);
-    load_batch(a, start, cnt, pm.tx0, pm.ty0, s_e);
+    load_batch(a, start, cnt, npix, s_e);
     staged = start == range.x && start + cnt == range.y;
     __syncthreads();
     if (__all_sync(0xffffffffu, done)) continue;
     uint32_t stop_off = 0xffffffffu;   // of the entry this pixel stopped at in this batch
     for (int c0 = 0; c0 < cnt; c0 += kChunk) {
-      const int steps = fill_lists(cull, B, c0, cnt, lists, kCount ? &n_warp : nullptr);
+      const int steps = fill_lists(warp_cull(a, s_e), B, c0, cnt, lists, kCount ? &n_warp : nullptr);
       bool all = false;
 #pragma unroll 1
       for (int i = 0; i < steps && !all; i += kStep) {
@@ -364,15 +354,15 @@ __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint4 tw, flo
 
   const CamRec& cam = a.cams[tw.w];
   const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
-  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h, threadIdx.x >> 5);
-  const bool inside = pm.px < cam.width && pm.py < cam.height;
-  const float pxc = (float)pm.px + 0.5f, pyc = (float)pm.py + 0.5f;
+  const int2 pm = map_pixel(a, local % cam.tiles_x, local / cam.tiles_x, threadIdx.x >> 5);
+  const bool inside = pm.x < cam.width && pm.y < cam.height;
+  const float2 npix = neg_centre(pm);
   const uint2 range = make_uint2(tw.y, tw.z);
   const int lane = threadIdx.x & 31;
 
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
   const FwdPixel fp =
-      fwd_walk<kCount>(a, pm, pxc, pyc, range, inside, s_e, lists[threadIdx.x >> 5], n_eval, n_comp, n_warp);
+      fwd_walk<kCount>(a, npix, range, inside, s_e, lists[threadIdx.x >> 5], n_eval, n_comp, n_warp);
   float T = fp.T, C0 = fp.C0, C1 = fp.C1, C2 = fp.C2;
   const uint32_t walked = fp.walked;
 
@@ -382,7 +372,7 @@ __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint4 tw, flo
     C1 = __fmaf_rn(T, a.bg[1], C1);
     C2 = __fmaf_rn(T, a.bg[2], C2);
     const int64_t hw = (int64_t)cam.width * cam.height;
-    const int64_t pix = (int64_t)pm.py * cam.width + pm.px;
+    const int64_t pix = (int64_t)pm.y * cam.width + pm.x;
     float* img = a.images + 3 * cam.pixel_base;
     img[pix] = C0;
     img[hw + pix] = C1;
@@ -434,8 +424,8 @@ __device__ __forceinline__ void red_add4(float* addr, float x, float y, float z,
 }
 
 // Pass 2 over slots [0, k) of both halves.  null_off: offset of the null entry.
-__device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws, int k, const Entry* s_e,
-                                            const PixelMap& pm, uint32_t null_off) {
+__device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws, int k, const Entry* s_e, float2 npix,
+                                            uint32_t null_off) {
   static_assert(kSlots == 8 && kBlkW == 4 && kSubH == 4, "two rows of a block per lane");
   __syncwarp();
   const int lane = threadIdx.x & 31;
@@ -474,9 +464,9 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
   const uint32_t off = reinterpret_cast<const uint16_t*>(ws.slot[h])[s];
   if (r == 0 && s < k && off != null_off) {
     const Entry& en = entry_at(s_e, off);
-    // dx = U - c, dy = V - r
-    const float U = en.a.x - (pm.x0 + (float)(h * kBlkW) + 0.5f * (float)(kBlkW - 1));
-    const float V = en.a.y - (pm.y0 + 0.5f * (float)(kSubH - 1));
+    // dx = U - c, dy = V - r; the block's centre from this lane's pixel
+    const float U = en.a.x + (npix.x + ((float)(lane & 3) - 0.5f * (float)(kBlkW - 1)));
+    const float V = en.a.y + (npix.y + ((float)((lane >> 2) & 3) - 0.5f * (float)(kSubH - 1)));
     float g[9];
     g[0] = fmaf(U, m[0], -m[1]);                          // sum dq dx
     g[1] = fmaf(V, m[0], -m[2]);                          // sum dq dy
@@ -502,19 +492,18 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
 // walks `bound` entries.  staged (CTA-uniform): the whole list is already in
 // shared memory (a single batch that the forward of the same CTA staged).
 template <bool kRecompute>
-__device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm, float pxc, float pyc,
-                                         uint2 range, bool inside, const float* Cf, const float* dC,
-                                         uint32_t bound, bool staged, Entry* s_e, WarpScratch& ws) {
+__device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 range, bool inside, const float* Cf,
+                                         const float* dC, uint32_t bound, bool staged, Entry* s_e, WarpScratch& ws) {
   const int B = a.batch;
-  const uint32_t* cull = cull_of(a, s_e) + pm.block * cull_stride(B);
   const int lane = threadIdx.x & 31;
   const uint32_t null_off = (uint32_t)(B * (int)sizeof(Entry));
   // dL/dalpha_i = sum_c dC_c (c_i T_i - S_c / (1 - alpha_i)) with S the colour
   // behind entry i, S_c = C_c - P_c (P the running front-to-back sum), so
   // sum_c dC_c S_c = D0 - Q with D0 = dC . C and Q = dC . P kept as a scalar.
+  // (Carrying D0 - Q itself saves an instruction and a register, but its error
+  // is larger: Q rounds much as C did, and the difference cancels that.)
   const float D0 = dC[0] * Cf[0] + dC[1] * Cf[1] + dC[2] * Cf[2];
   float T = 1.f, Q = 0.f;
-  const float2 npix = make_float2(-pxc, -pyc);
   bool done = !inside;
   if (kRecompute || !inside) bound = inside ? 0xffffffffu : 0u;   // outside the image: an empty walk
   // (dC0, dC1, 1, dC2): pass 2 pairs the 1 with dq and dC2 with w
@@ -526,20 +515,24 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm,
     if (!staged && __syncthreads_count(done) == (int)blockDim.x) break;
     const int cnt = (int)min((uint32_t)B, range.y - start);
     if (!staged) {
-      load_batch(a, start, cnt, pm.tx0, pm.ty0, s_e);
+      load_batch(a, start, cnt, npix, s_e);
       __syncthreads();
     }
     if (__all_sync(0xffffffffu, done)) continue;
     // entries at offsets below lim of this batch lie within the pixel's walk
     const uint32_t lim = min((uint32_t)cnt, bound - min(bound, start - range.x)) * (uint32_t)sizeof(Entry);
     for (int c0 = 0; c0 < cnt; c0 += kChunk) {
-      const int steps = fill_lists(cull, B, c0, cnt, ws.lists);
+      const int steps = fill_lists(warp_cull(a, s_e), B, c0, cnt, ws.lists);
       bool all = false;
 #pragma unroll 1
       for (int i = 0; i < steps && !all; i += kStep) {
         const uint2 quad = list_quad(ws.lists, i);
         if ((lane & 15) == 0) ws.slot[lane >> 4][k0 / kStep] = quad;
         float2* slot = &ws.dqw[k0][lane];
+        // the results wait in registers until all four are there: a store would
+        // keep the next entry's loads from starting (668 -> 651 us at 300k / 8 x
+        // 800^2)
+        float2 res[kStep];
         uint32_t off = 0;
 #pragma unroll
         for (int k = 0; k < kStep; ++k) {
@@ -570,11 +563,13 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm,
           const float dq = (!stop && e <= kAlphaMax) ? dLda * alpha : 0.f;
           T = stop ? T : test_T;
           if (kRecompute) done = done || stop;
-          slot[k * 33] = make_float2(dq, w);
+          res[k] = make_float2(dq, w);
         }
+#pragma unroll
+        for (int k = 0; k < kStep; ++k) slot[k * 33] = res[k];
         k0 += kStep;
         if (k0 == kSlots) {
-          flush_slots(a, ws, kSlots, s_e, pm, null_off);
+          flush_slots(a, ws, kSlots, s_e, npix, null_off);
           k0 = 0;
         }
         // (a padded list says nothing about the walk's end)
@@ -585,7 +580,7 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, const PixelMap& pm,
     }
     if (!kRecompute) done = done || start - range.x + cnt >= bound;
     if (k0) {   // the slots refer to this batch's shared-memory records
-      flush_slots(a, ws, k0, s_e, pm, null_off);
+      flush_slots(a, ws, k0, s_e, npix, null_off);
       k0 = 0;
     }
   }
@@ -598,16 +593,16 @@ template <bool kRecompute>
 __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
   const CamRec& cam = a.cams[tw.w];
   const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
-  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h, threadIdx.x >> 5);
-  const bool inside = pm.px < cam.width && pm.py < cam.height;
-  const float pxc = (float)pm.px + 0.5f, pyc = (float)pm.py + 0.5f;
+  const int2 pm = map_pixel(a, local % cam.tiles_x, local / cam.tiles_x, threadIdx.x >> 5);
+  const bool inside = pm.x < cam.width && pm.y < cam.height;
+  const float2 npix = neg_centre(pm);
   const uint2 range = make_uint2(tw.y, tw.z);
 
   float Cf[3] = {0.f, 0.f, 0.f}, dC[3] = {0.f, 0.f, 0.f};
   uint32_t bound = range.y - range.x;
   if (inside) {
     const int64_t hw = (int64_t)cam.width * cam.height;
-    const int64_t pix = (int64_t)pm.py * cam.width + pm.px;
+    const int64_t pix = (int64_t)pm.y * cam.width + pm.x;
     const float* img = a.images_in + 3 * cam.pixel_base;
     const float* gi = a.grad_in + 3 * cam.pixel_base;
 #pragma unroll
@@ -618,7 +613,7 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint4 tw, flo
     if (!kRecompute) bound = a.nwalk[cam.pixel_base + pix];
   }
   WarpScratch* ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem));
-  bwd_walk<kRecompute>(a, pm, pxc, pyc, range, inside, Cf, dC, bound, false, reinterpret_cast<Entry*>(s_mem),
+  bwd_walk<kRecompute>(a, npix, range, inside, Cf, dC, bound, false, reinterpret_cast<Entry*>(s_mem),
                        ws[threadIdx.x >> 5]);
 }
 
@@ -640,16 +635,16 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, f
 
   const CamRec& cam = a.cams[tw.w];
   const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
-  const PixelMap pm = map_pixel(a.tile_w, local % cam.tiles_x, local / cam.tiles_x, a.tile_h, threadIdx.x >> 5);
-  const bool inside = pm.px < cam.width && pm.py < cam.height;
-  const float pxc = (float)pm.px + 0.5f, pyc = (float)pm.py + 0.5f;
+  const int2 pm = map_pixel(a, local % cam.tiles_x, local / cam.tiles_x, threadIdx.x >> 5);
+  const bool inside = pm.x < cam.width && pm.y < cam.height;
+  const float2 npix = neg_centre(pm);
   const uint2 range = make_uint2(tw.y, tw.z);
   const int lane = threadIdx.x & 31;
 
   WarpScratch& ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem))[threadIdx.x >> 5];
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
   const FwdPixel fp =
-      fwd_walk<false>(a, pm, pxc, pyc, range, inside, s_e, ws.lists, n_eval, n_comp, n_warp);
+      fwd_walk<false>(a, npix, range, inside, s_e, ws.lists, n_eval, n_comp, n_warp);
   float Cf[3] = {0.f, 0.f, 0.f}, dC[3] = {0.f, 0.f, 0.f};
   float l1 = 0.f;
   if (inside) {
@@ -657,7 +652,7 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, f
     Cf[1] = __fmaf_rn(fp.T, a.bg[1], fp.C1);
     Cf[2] = __fmaf_rn(fp.T, a.bg[2], fp.C2);
     const int64_t hw = (int64_t)cam.width * cam.height;
-    const int64_t pix = (int64_t)pm.py * cam.width + pm.px;
+    const int64_t pix = (int64_t)pm.y * cam.width + pm.x;
     float* img = a.images + 3 * cam.pixel_base;
     const float* tg = a.targets + 3 * cam.pixel_base + pix;
 #pragma unroll
@@ -677,7 +672,7 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, f
   l1 = sub_block_sum(l1);
   if (lane == 0) s_red[threadIdx.x >> 5] = l1;
   __syncwarp();
-  bwd_walk<false>(a, pm, pxc, pyc, range, inside, Cf, dC, fp.walked, fp.staged, s_e, ws);
+  bwd_walk<false>(a, npix, range, inside, Cf, dC, fp.walked, fp.staged, s_e, ws);
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
@@ -710,10 +705,10 @@ __device__ __forceinline__ void blend_empty(const BlendArgs& a, uint32_t first) 
     float* img = a.images + 3 * cam.pixel_base;
 #pragma unroll 4
     for (int b = 0; b < (int)blockDim.x / 32; ++b) {
-      const PixelMap pm = map_pixel(a.tile_w, tx, ty, a.tile_h, b);
-      const int64_t pix = (int64_t)pm.py * cam.width + pm.px;
+      const int2 pm = map_pixel(a, tx, ty, b);
+      const int64_t pix = (int64_t)pm.y * cam.width + pm.x;
       float l1 = 0.f;
-      if (pm.px < cam.width && pm.py < cam.height) {
+      if (pm.x < cam.width && pm.y < cam.height) {
         if (kStore) a.nwalk[cam.pixel_base + pix] = 0u;
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) {
