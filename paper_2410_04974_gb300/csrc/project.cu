@@ -265,7 +265,7 @@ __device__ __forceinline__ void project_pair(const ProjectArgs& a, Beta beta, co
 __device__ __forceinline__ void count_big(const ProjectArgs& a, const CamRec* cams, const BigRects& big) {
   __syncthreads();
   const uint32_t nb = min(big.count, (uint32_t)BigRects::kMax);
-  for (uint32_t i = threadIdx.x >> 5; i < nb; i += kStageTile / 32) {
+  for (uint32_t i = threadIdx.x >> 5; i < nb; i += blockDim.x / 32) {
     const uint4 e = *big.at[i];
     const CamRec& cam = cams[e.x / (uint32_t)a.n];
     const uint32_t x0 = e.z & 0xffffu, y0 = e.w & 0xffffu, w = max((e.z >> 16) - x0, 1u);
@@ -278,26 +278,67 @@ __device__ __forceinline__ void count_big(const ProjectArgs& a, const CamRec* ca
   }
 }
 
-// kStageTile Gaussians per CTA in two phases:
+// Queues the pairs of Gaussian g0 + gl that are visible to cameras v0, v0 +
+// step, ...
+__device__ __forceinline__ void queue_visible(const ProjectArgs& a, const CamRec* cams, int v0, int step, int64_t g0,
+                                              int gl, bool ok, const float* mp, const float* md, const M3& A,
+                                              const M3& Sdi, float alpha, float lam, uint32_t& s_count,
+                                              uint16_t* s_queue) {
+  const int lane = threadIdx.x & 31;
+  for (int v = v0; v < a.n_cams; v += step) {
+    bool vis = false;
+    if (ok) {
+      const SliceView sv = slice_view(mp, md, A, Sdi, alpha, lam, cams[v]);
+      vis = (sv.alpha_cond >= kAlphaMin) && (sv.t[2] > cams[v].znear);
+    }
+    if (!vis) a.ntiles[(int64_t)v * a.n + g0 + gl] = 0u;
+    // warp-aggregated append to the queue
+    const uint32_t active = __activemask();
+    const uint32_t bal = __ballot_sync(active, vis);
+    uint32_t base = 0;
+    const int leader = __ffs(active) - 1;
+    if (lane == leader && bal) base = atomicAdd(&s_count, (uint32_t)__popc(bal));
+    base = __shfl_sync(active, base, leader);
+    if (vis) s_queue[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(gl | (v << 7));
+  }
+}
+
+// kStageTile Gaussians per CTA in three phases:
 //  A. one thread per Gaussian: the tile's parameter planes are staged in
 //     shared memory (stage.cuh), the view-independent state is computed (or
-//     read from the cache) and kept in shared memory, and every camera's
-//     slice decides visibility (alpha_cond >= 1/255, in front of the near
+//     read from the cache) and kept in shared memory;
+//  B. the same thread, or two threads per Gaussian with half of the cameras
+//     each: a camera's slice decides visibility (alpha_cond >= 1/255, in front of the near
 //     plane); visible (Gaussian, camera) pairs are queued in shared memory;
-//  B. the CTA's threads take the queued pairs densely, one pair each, for
+//  C. the CTA's threads take the queued pairs densely, one pair each, for
 //     the EWA projection, colour and tile rectangle, so that the expensive
 //     part runs on full warps however many pairs a Gaussian has visible.
+// The kernel waits more than it computes (loads, the barriers between the
+// phases), and the staged planes, 42 KB a CTA at degree 3, bound the CTAs per
+// SM: with kProjThreads = 256 threads sharing them there are 32 warps per SM
+// instead of 20, but four tiles in flight instead of five.  The former counts
+// with many views (phases B and C), the latter when the planes come from
+// memory: 101 -> 93 us at 300k / 8 views, 129 -> 113 us at 183k / 20 views,
+// but 205 -> 251 us at 2M / 4 views; so frames of fewer than kProjWideViews
+// views keep 128 threads.
 // kStaged (frames of several cameras, where each Gaussian's parameters serve
 // several pairs): as above.  Otherwise (one camera: little work to overlap
 // with an up-front load, at most one pair per Gaussian) each thread reads its
 // Gaussian's planes from global memory where it uses them and projects its
 // visible pair itself, with the same arithmetic.
-template <bool kCached, bool kStaged>
-__global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kernel(ProjectArgs a) {
+constexpr int kProjThreads = 256;
+constexpr int kProjWideViews = 8;
+
+// kThreads: threads of a staged CTA, 0: not staged.
+template <bool kCached, int kThreads>
+__global__ void __launch_bounds__(kThreads ? kThreads : kStageTile, kThreads == kStageTile ? 5 : 4)
+    project_fwd_kernel(ProjectArgs a) {
+  constexpr bool kStaged = kThreads != 0;
   extern __shared__ float4 s_dyn[];
   __shared__ uint64_t s_bars[2];
   __shared__ uint32_t s_count;   // the CTA's visible pairs
   __shared__ BigRects s_big;
+  __shared__ uint32_t s_ok[kStageTile / 32];   // Gaussians with a finite state
   CamRec* s_cams = reinterpret_cast<CamRec*>(s_dyn);
   float* tile = reinterpret_cast<float*>(s_cams + a.n_cams);
   const int64_t n = a.n;
@@ -308,6 +349,7 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
   uint16_t* s_queue = reinterpret_cast<uint16_t*>(tile + pp.count * kStageTile);
   for (int i = threadIdx.x; i < a.n_cams; i += blockDim.x) s_cams[i] = a.cams[i];
   if (threadIdx.x == 0) s_count = s_big.count = 0;
+  if (threadIdx.x < kStageTile / 32) s_ok[threadIdx.x] = 0;
   const int64_t g0 = (int64_t)blockIdx.x * kStageTile;
   uint4* vis_seg = a.vis + g0 * a.n_cams;   // this CTA's segment of the visible queue
   const int m = (int)min((int64_t)kStageTile, n - g0);
@@ -400,23 +442,10 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
       store_sym(cp, 15, cs.Sc);
       cp[21 * kStageTile] = cs.alpha;
       cp[22 * kStageTile] = lam;
-      const int lane = tid & 31;
-      const M3 Sdi = sym_upper(cs.Sdi);   // as phase B reads it back
-      for (int v = 0; v < a.n_cams; ++v) {
-        bool vis = false;
-        if (ok) {
-          const SliceView sv = slice_view(mp, md, cs.A, Sdi, cs.alpha, lam, s_cams[v]);
-          vis = (sv.alpha_cond >= kAlphaMin) && (sv.t[2] > s_cams[v].znear);
-        }
-        if (!vis) a.ntiles[(int64_t)v * n + g] = 0u;
-        // warp-aggregated append to the queue
-        const uint32_t active = __activemask();
-        const uint32_t bal = __ballot_sync(active, vis);
-        uint32_t base = 0;
-        const int leader = __ffs(active) - 1;
-        if (lane == leader && bal) base = atomicAdd(&s_count, (uint32_t)__popc(bal));
-        base = __shfl_sync(active, base, leader);
-        if (vis) s_queue[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(tid | (v << 7));
+      if constexpr (kThreads > kStageTile) {
+        if (ok) atomicOr(&s_ok[tid >> 5], 1u << (tid & 31));
+      } else {
+        queue_visible(a, s_cams, 0, 1, g0, tid, ok, mp, md, cs.A, sym_upper(cs.Sdi), cs.alpha, lam, s_count, s_queue);
       }
     }
   }
@@ -425,14 +454,34 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
     if (tid == 0) a.vis_count[blockIdx.x] = s_count;
     return;
   }
+
+  // ---- phase B: visibility ----
+  if constexpr (kThreads > kStageTile) {
+    __syncthreads();
+    const int gv = tid % kStageTile;
+    if (gv < m) {
+      const float* sp = tile + gv;
+      const float* cp = s_cs + gv;
+      const bool ok = (s_ok[gv >> 5] >> (gv & 31)) & 1u;
+      const float mp[3] = {sp[pp.mu_p * kStageTile], sp[(pp.mu_p + 1) * kStageTile], sp[(pp.mu_p + 2) * kStageTile]};
+      const float md[3] = {sp[pp.mu_d * kStageTile], sp[(pp.mu_d + 1) * kStageTile], sp[(pp.mu_d + 2) * kStageTile]};
+      M3 A;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) A.m[k] = cp[k * kStageTile];
+      const M3 Sdi = load_sym(cp, 9);
+      const float alpha = cp[21 * kStageTile], lam = cp[22 * kStageTile];
+      queue_visible(a, s_cams, tid / kStageTile, kThreads / kStageTile, g0, gv, ok, mp, md, A, Sdi, alpha, lam, s_count,
+                    s_queue);
+    }
+  }
   if (!stage_wait(s_bars, 1, bulk, a.spin_budget)) raise_status(a.status, SIXDGS_ERR_TIMEOUT);
   __syncthreads();
 
-  // ---- phase B: one visible pair per thread ----
+  // ---- phase C: one visible pair per thread ----
   const uint32_t count = s_count;
   if (tid == 0) a.vis_count[blockIdx.x] = count;
   const int K = (a.sh_degree + 1) * (a.sh_degree + 1);
-  for (uint32_t qi = tid; qi < count; qi += kStageTile) {
+  for (uint32_t qi = tid; qi < count; qi += kThreads) {
     const uint32_t e = s_queue[qi];
     const int gl = (int)(e & 127u);
     const int v = (int)(e >> 7);
@@ -453,29 +502,30 @@ __global__ void __launch_bounds__(kStageTile, kStaged ? 5 : 4) project_fwd_kerne
   count_big(a, s_cams, s_big);
 }
 
-template <bool kCached, bool kStaged>
+template <bool kCached, int kThreads>
 static void launch_project(const ProjectArgs& a, cudaStream_t stream) {
   const int64_t blocks = (a.n + kStageTile - 1) / kStageTile;
   const ProjPlanes pp = proj_planes(kCached, a.sh_degree, a.lambda_raw != nullptr);
   const size_t smem = sizeof(CamRec) * (size_t)a.n_cams +
-                      (kStaged ? (size_t)pp.count * kStageTile * sizeof(float) +
-                                     (size_t)kStageTile * a.n_cams * sizeof(uint16_t)
-                               : 0);
+                      (kThreads ? (size_t)pp.count * kStageTile * sizeof(float) +
+                                      (size_t)kStageTile * a.n_cams * sizeof(uint16_t)
+                                : 0);
   if (smem > 40 * 1024)   // the static shared memory counts towards the 48 KB as well
-    cudaFuncSetAttribute(project_fwd_kernel<kCached, kStaged>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  project_fwd_kernel<kCached, kStaged><<<(unsigned)blocks, kStageTile, smem, stream>>>(a);
+    cudaFuncSetAttribute(project_fwd_kernel<kCached, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  project_fwd_kernel<kCached, kThreads><<<(unsigned)blocks, kThreads ? kThreads : kStageTile, smem, stream>>>(a);
+}
+
+template <bool kCached>
+static void launch_project_views(const ProjectArgs& a, cudaStream_t stream) {
+  if (a.n_cams == 1) launch_project<kCached, 0>(a, stream);
+  else if (a.n_cams < kProjWideViews) launch_project<kCached, kStageTile>(a, stream);
+  else launch_project<kCached, kProjThreads>(a, stream);
 }
 
 void launch_project_fwd(const ProjectArgs& a, cudaStream_t stream) {
   if (a.n == 0) return;
-  const bool staged = a.n_cams > 1;
-  if (a.cond_cache) {
-    if (staged) launch_project<true, true>(a, stream);
-    else launch_project<true, false>(a, stream);
-  } else {
-    if (staged) launch_project<false, true>(a, stream);
-    else launch_project<false, false>(a, stream);
-  }
+  if (a.cond_cache) launch_project_views<true>(a, stream);
+  else launch_project_views<false>(a, stream);
 }
 
 void launch_cond_cache(const CondCacheArgs& a, cudaStream_t stream) {

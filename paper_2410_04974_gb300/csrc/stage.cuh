@@ -108,7 +108,9 @@ __device__ __forceinline__ void stage_issue(float* tile, int np, int split, Src 
 __device__ __forceinline__ bool stage_wait(uint64_t* bars, int grp, bool bulk, int64_t budget) {
   if (!bulk) return true;
   bool ok = mbar_wait(&bars[grp], 0, budget);
-  if (!ok) ok = mbar_wait(&bars[grp], 0, budget);   // the copies land in this CTA's memory: let them finish
+  // the copies land in this CTA's memory: let them finish, for at least 2^24
+  // cycles (about 8 ms) however short the budget
+  if (!ok) ok = mbar_wait(&bars[grp], 0, budget > (1 << 24) ? budget : (1 << 24));
   return ok;
 }
 
