@@ -74,8 +74,7 @@ KERNEL_SOURCES = {
     "project_fwd_kernel": ["project.cu", "bin.cuh", "cond.cuh", "sh.cuh", "mat3.cuh", "stage.cuh"],
     "bin_scan_kernel": ["sort.cu", "bin.cuh"], "bin_scatter_kernel": ["sort.cu", "bin.cuh"],
     "bin_sort_kernel": ["sort.cu", "bin.cuh"],
-    "geom_bwd_kernel": ["project_bwd.cu", "cond.cuh", "mat3.cuh"],
-    "sh_bwd_kernel": ["project_bwd.cu", "cond.cuh", "mat3.cuh", "sh.cuh"],
+    "param_bwd_kernel": ["project_bwd.cu", "cond.cuh", "mat3.cuh", "sh.cuh", "stage.cuh"],
     "scale_rotation_kernel": ["scale_rotation.cu", "cond.cuh", "mat3.cuh"],
 }
 
@@ -445,8 +444,8 @@ def launches_per_frame(plan, n_cams):
 def step_launches(n_cams):
     """Kernels of ours one fwd+bwd frame launches: camera upload (one per 48
     cameras), projection, list scan, scatter and sort, fused blend forward + L1
-    + blend backward, SH backward, geometry backward."""
-    return (n_cams + 47) // 48 + 1 + 3 + 1 + 1 + 1
+    + blend backward, per-Gaussian backward."""
+    return (n_cams + 47) // 48 + 1 + 3 + 1 + 1
 
 
 def build_inputs(args):

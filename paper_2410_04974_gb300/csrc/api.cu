@@ -447,8 +447,7 @@ sixdgs_status sixdgs_project_bwd(const sixdgs_plan* p, const sixdgs_scene* scene
   b.bulk = bulk_planes(p->n, {b.mu_p, b.mu_d, b.l_raw, b.opacity_logit, b.sh, b.lambda_raw});
   b.spin_budget = spin_budget(p);
   b.status = status_dev;
-  launch_sh_bwd(b, stream);
-  launch_geom_bwd(b, stream);
+  launch_param_bwd(b, stream);
   return launch_status();
 }
 

@@ -160,8 +160,7 @@ cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream);
 void launch_blend_fwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_blend_fused(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
 void launch_blend_bwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream);
-void launch_sh_bwd(const ProjectBwdArgs& a, cudaStream_t stream);
-void launch_geom_bwd(const ProjectBwdArgs& a, cudaStream_t stream);
+void launch_param_bwd(const ProjectBwdArgs& a, cudaStream_t stream);
 
 // Tiles per block of the list scan.
 constexpr int kScanTile = 256;
