@@ -46,7 +46,6 @@ struct ProjectArgs {
 enum BinWord {
   kBinClass = 0,         // tiles of every list-length class
   kBinCursor = 64,       // next place of every class in the tile order
-  kBinTicket = 128,      // scan tile counter
   kBinQueue = 129,       // sort work counter
   kBinOver = 130,        // tiles with lists above 4096, 2048, 1024, 512 and 0 entries
   kBinWords = 192

@@ -141,17 +141,17 @@ struct BigRects {
   static constexpr int kMax = 128;
   static constexpr uint32_t kTiles = 16;   // above: a warp counts them together
   uint32_t count;
-  const uint4* at[kMax];
+  uint4 entry[kMax];
 };
 
 // Adds one pair's duplicates to the counts of its view's tiles (no result is
 // waited for).
-__device__ __forceinline__ void count_tiles(TileCounters* c, int32_t tiles_x, uint4 e, uint32_t ntiles, const uint4* vis,
+__device__ __forceinline__ void count_tiles(TileCounters* c, int32_t tiles_x, uint4 e, uint32_t ntiles,
                                             BigRects& big) {
   if (ntiles > BigRects::kTiles) {
     const uint32_t k = atomicAdd(&big.count, 1u);
     if (k < BigRects::kMax) {
-      big.at[k] = vis;
+      big.entry[k] = e;
       return;
     }
   }
@@ -253,7 +253,7 @@ __device__ __forceinline__ void project_pair(const ProjectArgs& a, Beta beta, co
       a.rect[pair] =
           make_ushort4((unsigned short)x0, (unsigned short)x1, (unsigned short)y0, (unsigned short)y1);
       entry = vis_entry((uint32_t)pair, __float_as_uint(t[2]), (uint32_t)x0, (uint32_t)x1, (uint32_t)y0, (uint32_t)y1);
-      count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, vis, big);
+      count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, big);
     }
   }
   a.ntiles[pair] = ntiles;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void count_big(const ProjectArgs& a, const CamRec* ca
   __syncthreads();
   const uint32_t nb = min(big.count, (uint32_t)BigRects::kMax);
   for (uint32_t i = threadIdx.x >> 5; i < nb; i += blockDim.x / 32) {
-    const uint4 e = *big.at[i];
+    const uint4 e = big.entry[i];
     const CamRec& cam = cams[e.x / (uint32_t)a.n];
     const uint32_t x0 = e.z & 0xffffu, y0 = e.w & 0xffffu, w = max((e.z >> 16) - x0, 1u);
     const uint32_t nt = w * ((e.w >> 16) - y0);

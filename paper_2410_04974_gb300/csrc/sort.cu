@@ -165,13 +165,12 @@ __device__ __forceinline__ uint32_t count_class(uint32_t cls, bool valid, uint32
 __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   __shared__ uint32_t s_warp[kBinWarps + 1];
   __shared__ uint32_t s_class[kClasses];
-  __shared__ uint32_t s_block;
   __shared__ unsigned long long s_excl;
   const int tid = threadIdx.x;
-  if (tid == 0) s_block = atomicAdd(&a.state[kBinTicket], 1u);
   if (tid < kClasses) s_class[tid] = 0u;
-  __syncthreads();
-  const uint32_t block = s_block;
+  // blocks are started in the order of their index, so a block's predecessors
+  // are running or done when it waits for them (and the wait is bounded)
+  const uint32_t block = blockIdx.x;
   const uint32_t t = block * kScanTile + tid;
   const bool valid = t < a.total_tiles;
   const uint32_t cnt = valid ? a.tile[t].count : 0u;
@@ -181,8 +180,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
     const unsigned long long e = scan_lookback(a.scan_state, block, total, a.spin_budget, a.status);
     if (tid == 0) s_excl = e;
   }
-  // counters of the kernels that follow (every block has its own ticket, so
-  // exactly one block is block 0); the pair counters behind the first two
+  // counters of the kernels that follow; the pair counters behind the first two
   // public words are the blend's
   if (block == 0 && tid < 10) a.counts[2 + tid] = 0u;
   if (block == 0 && tid == 10) a.counts[0] = 0u;
@@ -266,7 +264,6 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
     if (blockIdx.x == a.scatter_grid) {
       // tiles with lists above the sort's limits: those of the classes beyond
       if (tid <= kBinLevels) a.state[kBinOver + tid] = s_longer[tid < kBinLevels ? 4 * (12 - tid) : 0];
-      if (tid == 32) a.state[kBinTicket] = 0u;
     }
     // the scan is over: its words are clean for the next call
     if (tid == 0 && t % kScanTile == 0) a.scan_state[t / kScanTile] = 0ull;
