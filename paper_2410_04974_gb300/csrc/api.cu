@@ -51,18 +51,21 @@ struct CamUpload {
 
 // Camera records from the kernel parameters, and the words that the
 // projection and the binning count in set to zero (zero_quads 16-byte words;
-// grid-stride).
+// grid-stride), and *loss unless it is null.
 template <int kCams>
 __global__ void upload_cams_kernel(const __grid_constant__ CamUpload<kCams> up, CamRec* dst, uint4* zero,
-                                   int64_t zero_quads) {
+                                   int64_t zero_quads, double* loss) {
+  after_previous();
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i0 < up.count) dst[up.first + i0] = up.cams[i0];
+  if (i0 == 0 && loss) *loss = 0.0;
   for (int64_t i = i0; i < zero_quads; i += (int64_t)gridDim.x * blockDim.x) zero[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // One launch per kCams cameras; the first also clears.
 template <int kCams, typename Make>
-void upload_cams(int n_cams, Make make, CamRec* dst, void* zero, int64_t zero_bytes, int sms, cudaStream_t stream) {
+void upload_cams(int n_cams, Make make, CamRec* dst, void* zero, int64_t zero_bytes, double* loss, int sms,
+                 cudaStream_t stream) {
   for (int first = 0; first < n_cams; first += kCams) {
     CamUpload<kCams> up;
     std::memset(&up, 0, sizeof(up));
@@ -71,7 +74,8 @@ void upload_cams(int n_cams, Make make, CamRec* dst, void* zero, int64_t zero_by
     for (int i = 0; i < up.count; ++i) up.cams[i] = make(first + i);
     const int64_t quads = first == 0 ? zero_bytes / 16 : 0;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((quads + 1023) / 1024, 2 * sms));
-    upload_cams_kernel<kCams><<<grid, 256, 0, stream>>>(up, dst, static_cast<uint4*>(zero), quads);
+    launch_after(upload_cams_kernel<kCams>, grid, 256, 0, 1, stream, up, dst, static_cast<uint4*>(zero), quads,
+                 first == 0 ? loss : nullptr);
   }
 }
 
@@ -139,6 +143,69 @@ bool valid_scene(const sixdgs_plan* p, const sixdgs_scene* s) {
 bool valid_fwd_scene(const sixdgs_plan* p, const sixdgs_scene* s) {
   return s && s->n == p->n && s->sh_degree == p->sh_degree &&
          (p->n == 0 || (s->mu_p && s->mu_d && s->sh && (s->cond_cache || (s->l_raw && s->opacity_logit))));
+}
+
+// sixdgs_condition_project; loss (may be null) is set to zero on the way.
+sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, const sixdgs_camera* cams, void* ws,
+                            size_t ws_bytes, double* loss, int32_t* status_dev, sixdgs_stream_t stream_) {
+  sixdgs_status e = check_ws(p, ws, ws_bytes);
+  if (e != SIXDGS_OK) return e;
+  if (!valid_fwd_scene(p, scene) || !cams) return SIXDGS_ERR_INVALID_ARG;
+  cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
+  CamRec* dcams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
+  int32_t tile_offset = 0;
+  int64_t pixel_base = 0;
+  for (int i = 0; i < p->n_cams; ++i) {
+    const CamRec r = make_cam_rec(cams[i], p->settings, 0, 0);
+    tile_offset += r.tiles_x * r.tiles_y;
+    pixel_base += (int64_t)r.width * r.height;
+  }
+  if (tile_offset != p->total_tiles || pixel_base != p->total_pixels) return SIXDGS_ERR_INVALID_ARG;
+  tile_offset = 0;
+  pixel_base = 0;
+  auto next_cam = [&](int i) {
+    const CamRec r = make_cam_rec(cams[i], p->settings, tile_offset, pixel_base);
+    tile_offset += r.tiles_x * r.tiles_y;
+    pixel_base += (int64_t)r.width * r.height;
+    return r;
+  };
+  char* zero = static_cast<char*>(ws) + p->off[WS_ZERO];
+  const int64_t zero_bytes = p->off[WS_ZERO_END] - p->off[WS_ZERO];
+  // kernel parameters of 128 bytes a camera: the launch copies no more of
+  // them than the frame needs
+  if (p->n_cams == 1) upload_cams<1>(1, next_cam, dcams, zero, zero_bytes, loss, sm_count(), stream);
+  else if (p->n_cams <= 8) upload_cams<8>(p->n_cams, next_cam, dcams, zero, zero_bytes, loss, sm_count(), stream);
+  else upload_cams<48>(p->n_cams, next_cam, dcams, zero, zero_bytes, loss, sm_count(), stream);
+  ProjectArgs a;
+  a.cams = dcams;
+  a.n_cams = p->n_cams;
+  a.n = p->n;
+  a.sh_degree = p->sh_degree;
+  a.lambda_opa = p->settings.lambda_opa;
+  a.inv_tile_w = 1.f / (float)p->settings.tile_w;
+  a.inv_tile_h = 1.f / (float)p->settings.tile_h;
+  a.alpha_footprint = p->settings.alpha_footprint;
+  a.mu_p = scene->mu_p;
+  a.mu_d = scene->mu_d;
+  a.l_raw = scene->l_raw;
+  a.opacity_logit = scene->opacity_logit;
+  a.sh = scene->sh;
+  a.lambda_raw = scene->lambda_raw;
+  a.cond_cache = scene->cond_cache;
+  a.rec = ws_ptr<PairRec>(ws, p, SIXDGS_WS_REC);
+  a.ntiles = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NTILES);
+  a.rect = ws_ptr<ushort4>(ws, p, SIXDGS_WS_RECT);
+  a.depth_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_DEPTHKEY);
+  a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
+  a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
+  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
+  a.grad_rec = p->settings.inference ? nullptr : ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
+  a.bulk = bulk_planes(p->n, {a.mu_p, a.mu_d, a.sh, a.lambda_raw, a.cond_cache,
+                              a.cond_cache ? nullptr : a.l_raw, a.cond_cache ? nullptr : a.opacity_logit});
+  a.spin_budget = spin_budget(p);
+  a.status = status_dev;
+  launch_project_fwd(a, stream);
+  return launch_status();
 }
 
 }  // namespace
@@ -240,65 +307,8 @@ size_t sixdgs_workspace_size(const sixdgs_plan* plan) { return plan ? (size_t)pl
 
 sixdgs_status sixdgs_condition_project(const sixdgs_plan* p, const sixdgs_scene* scene,
                                        const sixdgs_camera* cams, void* ws, size_t ws_bytes,
-                                       int32_t* status_dev, sixdgs_stream_t stream_) {
-  sixdgs_status e = check_ws(p, ws, ws_bytes);
-  if (e != SIXDGS_OK) return e;
-  if (!valid_fwd_scene(p, scene) || !cams) return SIXDGS_ERR_INVALID_ARG;
-  cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  CamRec* dcams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
-  int32_t tile_offset = 0;
-  int64_t pixel_base = 0;
-  for (int i = 0; i < p->n_cams; ++i) {
-    const CamRec r = make_cam_rec(cams[i], p->settings, 0, 0);
-    tile_offset += r.tiles_x * r.tiles_y;
-    pixel_base += (int64_t)r.width * r.height;
-  }
-  if (tile_offset != p->total_tiles || pixel_base != p->total_pixels) return SIXDGS_ERR_INVALID_ARG;
-  tile_offset = 0;
-  pixel_base = 0;
-  auto next_cam = [&](int i) {
-    const CamRec r = make_cam_rec(cams[i], p->settings, tile_offset, pixel_base);
-    tile_offset += r.tiles_x * r.tiles_y;
-    pixel_base += (int64_t)r.width * r.height;
-    return r;
-  };
-  char* zero = static_cast<char*>(ws) + p->off[WS_ZERO];
-  const int64_t zero_bytes = p->off[WS_ZERO_END] - p->off[WS_ZERO];
-  // kernel parameters of 128 bytes a camera: the launch copies no more of
-  // them than the frame needs
-  if (p->n_cams == 1) upload_cams<1>(1, next_cam, dcams, zero, zero_bytes, sm_count(), stream);
-  else if (p->n_cams <= 8) upload_cams<8>(p->n_cams, next_cam, dcams, zero, zero_bytes, sm_count(), stream);
-  else upload_cams<48>(p->n_cams, next_cam, dcams, zero, zero_bytes, sm_count(), stream);
-  ProjectArgs a;
-  a.cams = dcams;
-  a.n_cams = p->n_cams;
-  a.n = p->n;
-  a.sh_degree = p->sh_degree;
-  a.lambda_opa = p->settings.lambda_opa;
-  a.inv_tile_w = 1.f / (float)p->settings.tile_w;
-  a.inv_tile_h = 1.f / (float)p->settings.tile_h;
-  a.alpha_footprint = p->settings.alpha_footprint;
-  a.mu_p = scene->mu_p;
-  a.mu_d = scene->mu_d;
-  a.l_raw = scene->l_raw;
-  a.opacity_logit = scene->opacity_logit;
-  a.sh = scene->sh;
-  a.lambda_raw = scene->lambda_raw;
-  a.cond_cache = scene->cond_cache;
-  a.rec = ws_ptr<PairRec>(ws, p, SIXDGS_WS_REC);
-  a.ntiles = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NTILES);
-  a.rect = ws_ptr<ushort4>(ws, p, SIXDGS_WS_RECT);
-  a.depth_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_DEPTHKEY);
-  a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
-  a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
-  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
-  a.grad_rec = p->settings.inference ? nullptr : ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
-  a.bulk = bulk_planes(p->n, {a.mu_p, a.mu_d, a.sh, a.lambda_raw, a.cond_cache,
-                              a.cond_cache ? nullptr : a.l_raw, a.cond_cache ? nullptr : a.opacity_logit});
-  a.spin_budget = spin_budget(p);
-  a.status = status_dev;
-  launch_project_fwd(a, stream);
-  return launch_status();
+                                       int32_t* status_dev, sixdgs_stream_t stream) {
+  return project_frame(p, scene, cams, ws, ws_bytes, nullptr, status_dev, stream);
 }
 
 sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, int32_t* status_dev,
@@ -482,10 +492,8 @@ sixdgs_status sixdgs_render_batched(const sixdgs_plan* p, const sixdgs_scene* sc
     if (p->settings.inference || !loss_dev || !valid_scene(p, scene)) return SIXDGS_ERR_INVALID_ARG;
     if (p->n > 0 && (!grad_mu_p || !grad_mu_d || !grad_l_raw || !grad_opacity_logit || !grad_sh))
       return SIXDGS_ERR_INVALID_ARG;
-    if (cudaMemsetAsync(loss_dev, 0, sizeof(double), reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
-      return SIXDGS_ERR_CUDA;
   }
-  e = sixdgs_condition_project(p, scene, cams_host, ws, ws_bytes, status_dev, stream);
+  e = project_frame(p, scene, cams_host, ws, ws_bytes, train ? loss_dev : nullptr, status_dev, stream);
   if (e != SIXDGS_OK) return e;
   e = sixdgs_bin_sort(p, ws, ws_bytes, status_dev, stream);
   if (e != SIXDGS_OK) return e;

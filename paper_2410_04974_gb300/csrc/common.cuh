@@ -67,6 +67,13 @@ __device__ __forceinline__ int find_camera(const CamRec* cams, int n_cams, uint3
   return lo;
 }
 
+// First statement of every kernel of a frame: waits until the kernel before it
+// in the stream is done and its writes are visible.  A no-op for a plain
+// launch.  (No kernel lets its successor start earlier than at its own end:
+// waiting CTAs beside a running kernel slowed large frames, 764 -> 822 us for 20
+// views of 183k Gaussians at 1024^2, and gained nothing for small ones.)
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void raise_status(int32_t* status, int code) {
   if (status) atomicOr(status, 1 << code);
 }

@@ -333,6 +333,7 @@ constexpr int kProjWideViews = 8;
 template <bool kCached, int kThreads>
 __global__ void __launch_bounds__(kThreads ? kThreads : kStageTile, kThreads == kStageTile ? 5 : 4)
     project_fwd_kernel(ProjectArgs a) {
+  after_previous();
   constexpr bool kStaged = kThreads != 0;
   extern __shared__ float4 s_dyn[];
   __shared__ uint64_t s_bars[2];
@@ -512,7 +513,8 @@ static void launch_project(const ProjectArgs& a, cudaStream_t stream) {
                                 : 0);
   if (smem > 40 * 1024)   // the static shared memory counts towards the 48 KB as well
     cudaFuncSetAttribute(project_fwd_kernel<kCached, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  project_fwd_kernel<kCached, kThreads><<<(unsigned)blocks, kThreads ? kThreads : kStageTile, smem, stream>>>(a);
+  launch_after(project_fwd_kernel<kCached, kThreads>, (unsigned)blocks, kThreads ? kThreads : kStageTile, smem, 1,
+               stream, a);
 }
 
 template <bool kCached>

@@ -402,6 +402,7 @@ constexpr int kBins = 288;   // numbers of views, 0 to 256, and some
 
 // 4 CTAs per SM (128 registers; 5 at 102 registers spill: 204 instead of 131 us).
 __global__ void __launch_bounds__(kStageTile, 4) param_bwd_kernel(ProjectBwdArgs a) {
+  after_previous();
   extern __shared__ float4 s_dyn[];
   __shared__ uint64_t s_bars[2];
   __shared__ uint32_t s_bin[kBins];   // Gaussians of every number of views
@@ -504,7 +505,7 @@ void launch_param_bwd(const ProjectBwdArgs& a, cudaStream_t stream) {
                       sizeof(CamView) * (size_t)a.n_cams;
   if (smem > 40 * 1024)
     cudaFuncSetAttribute(param_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  param_bwd_kernel<<<(unsigned)((a.n + kStageTile - 1) / kStageTile), kStageTile, smem, stream>>>(a);
+  launch_after(param_bwd_kernel, (unsigned)((a.n + kStageTile - 1) / kStageTile), kStageTile, smem, 1, stream, a);
 }
 
 }  // namespace sixdgs

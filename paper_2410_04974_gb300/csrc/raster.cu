@@ -771,6 +771,7 @@ __device__ __forceinline__ bool blend_unit(const BlendArgs& a, uint32_t u, Tile 
 
 template <typename Tile, typename Empty>
 __device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile tile, Empty empty) {
+  after_previous();
   if (!a.tile_queue) {
     blend_unit(a, blockIdx.x, tile, empty);
     return;
@@ -843,9 +844,9 @@ static void launch_blend(K kernel, const BlendArgs& a, int64_t total_tiles, bool
   if (a.tile_queue) {
     cudaMemsetAsync(a.tile_queue, 0, sizeof(uint32_t), stream);
     const int grid = resident_grid((const void*)kernel, threads, smem, total_tiles);
-    kernel<<<grid, threads, smem, stream>>>(a);
+    launch_after(kernel, grid, threads, smem, 1, stream, a);
   } else {
-    kernel<<<(unsigned)total_tiles, threads, smem, stream>>>(a);
+    launch_after(kernel, (unsigned)total_tiles, threads, smem, 1, stream, a);
   }
 }
 

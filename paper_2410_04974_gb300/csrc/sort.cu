@@ -163,6 +163,7 @@ __device__ __forceinline__ uint32_t count_class(uint32_t cls, bool valid, uint32
 // Latency-bound (T x 4 bytes in, T x 12 out).  One tile per thread, so that a
 // frame of a few thousand tiles is spread over several SMs.
 __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
+  after_previous();
   __shared__ uint32_t s_warp[kBinWarps + 1];
   __shared__ uint32_t s_class[kClasses];
   __shared__ unsigned long long s_excl;
@@ -219,6 +220,7 @@ constexpr int kScatterThreads = 128;
 constexpr int kScatterEntries = 2 * kScatterThreads;
 constexpr int kScatterBatch = 4;
 __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a) {
+  after_previous();
   constexpr int kWarps = kScatterThreads / 32;
   __shared__ uint32_t s_class[kClasses], s_base[kClasses], s_longer[kClasses];
   __shared__ uint32_t s_warp[kWarps + 1];
@@ -661,6 +663,7 @@ __device__ __noinline__ void sort_long(const BinArgs& a, uint32_t start, uint32_
 }
 
 __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
+  after_previous();
   __shared__ uint64_t s_key[kBinWarps * kTeamWords];
   __shared__ uint32_t s_unit;
   const int tid = threadIdx.x;
@@ -709,22 +712,15 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
 // from a queue, a whole number of clusters, at most 4 CTAs per SM.
 cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream) {
   const uint32_t blocks = std::max(1u, (a.total_tiles + kScanTile - 1) / kScanTile);
-  bin_scan_kernel<<<blocks, kBinThreads, 0, stream>>>(a);
+  cudaError_t e = launch_after(bin_scan_kernel, blocks, kBinThreads, 0, 1, stream, a);
+  if (e != cudaSuccess) return e;
   a.scatter_grid = std::min(a.segments, (uint32_t)sms * 16u);
   const uint32_t order = std::max(1u, (a.total_tiles + kScatterThreads - 1) / kScatterThreads);
-  bin_scatter_kernel<<<a.scatter_grid + order, kScatterThreads, 0, stream>>>(a);
+  e = launch_after(bin_scatter_kernel, a.scatter_grid + order, kScatterThreads, 0, 1, stream, a);
+  if (e != cudaSuccess) return e;
   const uint32_t most = std::max(1u, (uint32_t)sms * 4u / kCluster);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(std::min(most, (std::max(a.total_tiles, 1u) + kCluster - 1) / kCluster) * kCluster);
-  cfg.blockDim = dim3(kBinThreads);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kCluster;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, bin_sort_kernel, a);
+  const uint32_t clusters = std::min(most, (std::max(a.total_tiles, 1u) + kCluster - 1) / kCluster);
+  return launch_after(bin_sort_kernel, clusters * kCluster, kBinThreads, 0, kCluster, stream, a);
 }
 
 }  // namespace sixdgs
