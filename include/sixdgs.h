@@ -240,8 +240,8 @@ sixdgs_status sixdgs_condition_project(const sixdgs_plan* plan, const sixdgs_sce
  * pair is duplicated once per touched tile, and each tile's list is sorted by
  * (depth, Gaussian id): the ranges from a scan of the tile counts that
  * condition_project left, the duplicates scattered to their tiles, then every
- * list sorted on chip (lists above 4,096 entries in runs that a cluster of
- * CTAs merges).  May be called again on the same projection.
+ * list sorted on chip (lists above 4,096 entries in runs that are then
+ * merged).  May be called again on the same projection.
  * Writes SORTED, SORTEDKEY, RANGES and COUNTS.  Device: CAPACITY (lists beyond
  * the capacity are cut), TIMEOUT (a look-back wait of the scan). */
 sixdgs_status sixdgs_bin_sort(const sixdgs_plan* plan, void* ws_dev, size_t ws_bytes,

@@ -78,10 +78,10 @@ enum BinWord {
   kBinClass = 0,         // tiles of every list-length class
   kBinCursor = 64,       // next place of every class in the tile order
   kBinQueue = 129,       // sort work counter
-  kBinOver = 130,        // tiles with lists above 4096, 2048, 1024, 512 and 0 entries
+  kBinOver = 130,        // tiles with lists above 16384, 4096, 2048, 1024, 512 and 0 entries
   kBinWords = 192
 };
-constexpr int kBinLevels = 4;   // 4096, 2048, 1024, 512 entries: the sizes of the sorting teams
+constexpr int kBinLevels = 5;   // 16384, 4096, 2048, 1024, 512 entries: what a CTA and its teams sort
 
 // Per-tile lists from the projection's tile counts and visible queue.
 struct BinArgs {

@@ -23,7 +23,7 @@
 // three launches.  Measured (sum of the kernels; radix -> tile first):
 //   300k / 8 x 800^2 (2.5 M duplicates)     206 -> 85 us
 //   2M / 4 x 1920x1080 (3.4 M)              236 -> 96 us
-//   500k / 64 mixed views (29 M)           1907 -> 1215 us
+//   500k / 64 mixed views (29 M)           1907 -> 900 us
 //   one view, 54 k duplicates                74 -> 28 us
 // (the projection, which counts the tiles, takes 83 -> 99 us at 300k).
 #include <algorithm>
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
     }
     if (blockIdx.x == a.scatter_grid) {
       // tiles with lists above the sort's limits: those of the classes beyond
-      if (tid <= kBinLevels) a.state[kBinOver + tid] = s_longer[tid < kBinLevels ? 4 * (12 - tid) : 0];
+      if (tid <= kBinLevels) a.state[kBinOver + tid] = s_longer[tid == 0 ? 4 * 14 : tid < kBinLevels ? 4 * (13 - tid) : 0];
     }
     // the scan is over: its words are clean for the next call
     if (tid == 0 && t % kScanTile == 0) a.scan_state[t / kScanTile] = 0ull;
@@ -605,18 +605,31 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   return r;
 }
 
-// A list of more than kRun entries, by the CTAs of a cluster: runs of kRun
-// sorted on chip, then merged pairwise, each entry finding its rank in the
-// sibling run by a binary search.  The merges go back and forth between dup
-// and the (sorted_key, sorted) arrays, which hold a key in two words.
+// A list of more than kRun entries: runs of kRun sorted on chip, then merged
+// pairwise, each entry finding its rank in the sibling run by a binary search
+// (kMergeBatch of them in flight per thread).  The merges go back and forth
+// between dup and the (sorted_key, sorted) arrays, which hold a key in two
+// words.  By one CTA for up to kAlone entries, so that as many lists are worked
+// on as CTAs fit; above, where few lists hold a frame up, by a cluster.  (All
+// of them by clusters, of whose eight CTAs two had a run to sort: the kernel
+// took 775 instead of 458 us at 500k / 64 mixed views.)
 constexpr uint32_t kRun = kMaxItems * kBinThreads;
+constexpr uint32_t kAlone = 4 * kRun;
+constexpr int kMergeBatch = 4;
 
+template <bool kByCluster>
 __device__ __noinline__ void sort_long(const BinArgs& a, uint32_t start, uint32_t len, uint32_t tile, uint64_t* s) {
-  const uint32_t rank = cluster_rank();
+  const uint32_t rank = kByCluster ? cluster_rank() : 0u;
+  constexpr uint32_t kRanks = kByCluster ? kCluster : 1;
+  constexpr uint32_t kStride = kRanks * kBinThreads;
+  auto sync = [&]() {
+    if (kByCluster) cluster_sync();
+    else __syncthreads();
+  };
   uint64_t* A = a.dup + start;
   uint32_t* hi = a.sorted_key + start;
   uint32_t* lo = a.sorted + start;
-  for (uint32_t r = rank * kRun; r < len; r += kCluster * kRun) {
+  for (uint32_t r = rank * kRun; r < len; r += kRanks * kRun) {
     const uint32_t m = min(kRun, len - r);
     // (the run goes to the other arrays: its entries are still read here)
     sort_team<kMaxItems, kBinWarps>(A + r, m, 0u, threadIdx.x, s, [&](uint32_t e, auto full) {
@@ -626,36 +639,49 @@ __device__ __noinline__ void sort_long(const BinArgs& a, uint32_t start, uint32_
     });
     __syncthreads();
   }
-  cluster_sync();
+  sync();
   bool in_a = false;
   for (uint32_t w = kRun; w < len; w *= 2) {
     const bool last = w >= (len + 1) / 2;
     auto load = [&](uint32_t i) -> uint64_t {
       return in_a ? __ldcg(A + i) : ((uint64_t)__ldcg(hi + i) << 32) | __ldcg(lo + i);
     };
-    for (uint32_t i = rank * kBinThreads + threadIdx.x; i < len; i += kCluster * kBinThreads) {
-      const uint64_t x = load(i);
-      const uint32_t run = i / w, sib = run ^ 1u;
-      const uint32_t s0 = min(sib * w, len), s1 = min(s0 + w, len);
-      uint32_t l = s0, h = s1;   // entries of the sibling run below x
-      while (l < h) {
-        const uint32_t m = (l + h) >> 1;
-        if (load(m) < x) l = m + 1u;
-        else h = m;
+    for (uint32_t i0 = rank * kBinThreads + threadIdx.x; i0 < len; i0 += kMergeBatch * kStride) {
+      uint64_t x[kMergeBatch];
+      uint32_t s0[kMergeBatch], n[kMergeBatch], l[kMergeBatch];   // sibling run, entries of it below x
+#pragma unroll
+      for (int k = 0; k < kMergeBatch; ++k) {
+        const uint32_t i = min(i0 + k * kStride, len - 1u);
+        x[k] = load(i);
+        s0[k] = min((i / w ^ 1u) * w, len);
+        n[k] = min(w, len - s0[k]);
+        l[k] = 0u;
       }
-      const uint32_t out = min((run & ~1u) * w + (i - run * w) + (l - s0), len - 1u);
-      if (in_a) {
-        hi[out] = last ? tile : (uint32_t)(x >> 32);
-        lo[out] = (uint32_t)x;
-      } else {
-        A[out] = x;
+      for (uint32_t step = w; step > 0u; step >>= 1) {
+#pragma unroll
+        for (int k = 0; k < kMergeBatch; ++k)
+          if (l[k] + step <= n[k] && load(s0[k] + l[k] + step - 1u) < x[k]) l[k] += step;
+      }
+#pragma unroll
+      for (int k = 0; k < kMergeBatch; ++k) {
+        const uint32_t i = i0 + k * kStride;
+        if (i < len) {
+          const uint32_t run = i / w;
+          const uint32_t out = min((run & ~1u) * w + (i - run * w) + l[k], len - 1u);
+          if (in_a) {
+            hi[out] = last ? tile : (uint32_t)(x[k] >> 32);
+            lo[out] = (uint32_t)x[k];
+          } else {
+            A[out] = x[k];
+          }
+        }
       }
     }
     in_a = !in_a;
-    cluster_sync();
+    sync();
   }
   if (in_a) {
-    for (uint32_t i = rank * kBinThreads + threadIdx.x; i < len; i += kCluster * kBinThreads) {
+    for (uint32_t i = rank * kBinThreads + threadIdx.x; i < len; i += kStride) {
       lo[i] = (uint32_t)__ldcg(A + i);
       hi[i] = tile;
     }
@@ -667,8 +693,9 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
   __shared__ uint64_t s_key[kBinWarps * kTeamWords];
   __shared__ uint32_t s_unit;
   const int tid = threadIdx.x;
-  // order: over[0] tiles with lists above 4096 entries, up to over[1] those
-  // above 2048, over[2] 1024, over[3] 512, over[4] the rest that are not empty
+  // order: over[0] tiles with lists above kAlone entries, up to over[1] those
+  // above 4096, over[2] 2048, over[3] 1024, over[4] 512, over[5] the rest that
+  // are not empty
   uint32_t over[kBinLevels + 1];
   over[kBinLevels] = min(a.state[kBinOver + kBinLevels], a.total_tiles);
 #pragma unroll
@@ -676,12 +703,12 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
   if (blockIdx.x == 0 && tid < 2 * kClasses) a.state[kBinClass + tid] = 0u;   // clean for the next call
   for (uint32_t u = blockIdx.x / kCluster; u < over[0]; u += gridDim.x / kCluster) {
     const uint4 w = a.order[u];
-    sort_long(a, w.y, w.z - w.y, w.x, s_key);
+    sort_long<true>(a, w.y, w.z - w.y, w.x, s_key);
     cluster_sync();
   }
   // units of the rest: one, two, four or eight tiles a CTA
-  const uint32_t u1 = over[1] - over[0], u2 = u1 + (over[2] - over[1] + 1) / 2, u4 = u2 + (over[3] - over[2] + 3) / 4;
-  const uint32_t units = u4 + (over[4] - over[3] + 7) / 8;
+  const uint32_t u1 = over[2] - over[0], u2 = u1 + (over[3] - over[2] + 1) / 2, u4 = u2 + (over[4] - over[3] + 3) / 4;
+  const uint32_t units = u4 + (over[5] - over[4] + 7) / 8;
   while (true) {
     __syncthreads();
     if (tid == 0) s_unit = atomicAdd(&a.state[kBinQueue], 1u);
@@ -689,15 +716,16 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
     const uint32_t u = s_unit;
     if (u >= units) break;
     uint32_t at, end, teams;
-    if (u < u1) at = over[0] + u, end = over[1], teams = 1;
-    else if (u < u2) at = over[1] + 2 * (u - u1), end = over[2], teams = 2;
-    else if (u < u4) at = over[2] + 4 * (u - u2), end = over[3], teams = 4;
-    else at = over[3] + 8 * (u - u4), end = over[4], teams = 8;
+    if (u < u1) at = over[0] + u, end = over[2], teams = 1;
+    else if (u < u2) at = over[2] + 2 * (u - u1), end = over[3], teams = 2;
+    else if (u < u4) at = over[3] + 4 * (u - u2), end = over[4], teams = 4;
+    else at = over[4] + 8 * (u - u4), end = over[5], teams = 8;
     at += threadIdx.x / (kBinThreads / teams);
     const uint4 w = at < end ? a.order[at] : make_uint4(0u, 0u, 0u, 0u);
-    const uint32_t len = min(w.z - w.y, kRun / teams);
+    const uint32_t len = teams == 1 ? min(w.z - w.y, kAlone) : min(w.z - w.y, kRun / teams);
     if (len == 0u) continue;   // (the whole team)
-    if (teams == 1) sort_tile<16, 8>(a, w.x, w.y, len, s_key);
+    if (len > kRun) sort_long<false>(a, w.y, len, w.x, s_key);
+    else if (teams == 1) sort_tile<16, 8>(a, w.x, w.y, len, s_key);
     else if (teams == 2) sort_tile<16, 4>(a, w.x, w.y, len, s_key);
     else if (teams == 4) sort_tile<16, 2>(a, w.x, w.y, len, s_key);
     else if (len > 256u) sort_tile<16, 1>(a, w.x, w.y, len, s_key);

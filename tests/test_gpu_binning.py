@@ -1,7 +1,7 @@
 """The per-tile lists against a NumPy sort of the same frame's rectangles and
 depths, at the sizes where the binning takes another path: lists of one entry,
 at the limits of the sorting teams (64 to 4,096 entries), above them (runs
-merged by a cluster of CTAs), rectangles of one tile and of hundreds, and
+merged by one CTA, then by a cluster of them), rectangles of one tile and of hundreds, and
 equal depths (a few, and whole lists of them)."""
 
 import numpy as np
@@ -48,6 +48,7 @@ def _expected(r):
     ("shell", 30_000, 1, (128, 128), 1.0),    # lists of several hundred
     ("shell", 9_000, 2, (48, 32), 1.0),       # lists of one to four thousand
     ("shell", 60_000, 1, (24, 24), 1.0),      # lists beyond 4,096: merged runs
+    ("shell", 300_000, 1, (24, 24), 1.0),     # beyond 16,384: merged by a cluster
     ("cube", 20_000, 1, (64, 64), 0.0),       # every depth equal: lists sorted by id alone
     ("cube", 20_000, 1, (64, 64), 1e-6),      # a handful of depths
 ])
@@ -70,7 +71,8 @@ def test_lists_equal_a_numpy_sort(kind, n, views, size, spread):
         key = r._section(_lib.WS_SORTEDKEY, torch.int32, int(counts[1]))
         np.testing.assert_array_equal(key.cpu().numpy(), tiles)
         if kind == "shell" and size == (24, 24):
-            assert (ranges[:, 1] - ranges[:, 0]).max() > 4096
+            longest = (ranges[:, 1] - ranges[:, 0]).max()
+            assert longest > 16384 if n == 300_000 else 4096 < longest <= 16384
         r.bin_sort()
         torch.cuda.synchronize()
     assert int(r.status.item()) == 0
