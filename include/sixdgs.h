@@ -384,17 +384,18 @@ sixdgs_status sixdgs_scale_rotation(int64_t n, const float* l_raw_dev, float* ro
  * with a fixed budget), or loops that must never call cudaMalloc.  It runs
  * the same work as sixdgs_condition_project + sixdgs_bin_sort +
  * sixdgs_raster_fwd (no loss) and writes the same images, but keeps the
- * frame's workspace in one array of SIXDGS_STATIC_WS_BYTES (32 MiB) that
- * lives in the library's device memory.  Every GPU that loads the library
+ * frame's workspace in one array (256 MiB) that lives in the library's device
+ * memory.  Every GPU that loads the library
  * holds that array until the process exits.  The call allocates nothing
  * (no cudaMalloc, cudaFree or allocating library routine).
  *
  * Limits: the frame is planned forward-only whatever the caller's settings
  * say (as with settings.inference = 1 and store_aux = 0: no gradient
  * records, no per-pixel walk lengths) with the default duplicate capacity,
- * and that plan must need at most SIXDGS_STATIC_WS_BYTES of workspace, about
- * 225,000 (camera, Gaussian) pairs (e.g. 225,925 Gaussians seen by one
- * 800x800 camera, or 56,504 Gaussians by four 256x256 cameras); larger
+ * and its size, a fixed function of its pairs, duplicates and tiles (about 148
+ * bytes a (camera, Gaussian) pair and 8 a tile), must be at most
+ * SIXDGS_STATIC_WS_BYTES, about 225,000 pairs (e.g. 225,925 Gaussians seen by
+ * one 800x800 camera, or 56,504 Gaussians by four 256x256 cameras); larger
  * frames are refused with SIXDGS_ERR_WORKSPACE before anything is launched.  The array is
  * shared by all calls on a device and keeps the last call's contents (each
  * call clears what it needs); calls that overlap on the GPU (different

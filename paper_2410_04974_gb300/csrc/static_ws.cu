@@ -6,8 +6,8 @@
 // Meant for callers that cannot allocate device memory themselves: code
 // running inside a host application whose allocator owns all device memory
 // (plugins, engines with a fixed memory budget), or latency-critical loops
-// that must not call cudaMalloc.  The array is SIXDGS_STATIC_WS_BYTES long
-// and every device that loads the library keeps it until the process exits.
+// that must not call cudaMalloc.  Every device that loads the library keeps
+// the array until the process exits.
 #include <mutex>
 
 #include "common.cuh"
@@ -15,8 +15,41 @@
 
 namespace {
 
-// Workspace shared by every call of sixdgs_render_fwd_static on a device.
-static __device__ __align__(256) unsigned char g_static_ws[SIXDGS_STATIC_WS_BYTES];
+// Workspace shared by every call of sixdgs_render_fwd_static on a device.  The
+// call's limit counts 8 bytes a tile, the stages keep 56 (range, counters and
+// order record): a frame of the smallest scene and the most tiles that the limit
+// takes (4.19 million) needs 7 times the limit, and one more covers alignment
+// and the scan's words.
+constexpr size_t kArrayBytes = 8 * (size_t)SIXDGS_STATIC_WS_BYTES;
+static __device__ __align__(256) unsigned char g_static_ws[kArrayBytes];
+
+// The size that is held against SIXDGS_STATIC_WS_BYTES: a fixed function of a
+// frame's pairs, duplicates and tiles (about 148.5 bytes a pair and 8 a tile), so
+// that the frames the call takes do not change with what the stages happen to
+// need inside the workspace.
+int64_t limit_bytes(const sixdgs_plan& p) {
+  int64_t o = 0;
+  auto take = [&](int64_t bytes) { o = (o + bytes + 255) / 256 * 256; };
+  const int64_t n = p.n_pairs, d = p.dup_capacity, t = p.total_tiles;
+  const int64_t sort_n = (n + 3071) / 3072 + 1, sort_d = (d + 3071) / 3072 + 1, scan = (n + 1023) / 1024 + 1;
+  take(p.n_cams * (int64_t)sizeof(sixdgs::CamRec));
+  take(n * 48);                       // records
+  take((n + 3) / 4 * 16);             // tile counts
+  take(n * 8);                        // rectangles
+  take(n * 4);                        // depth keys
+  take(t * 8);                        // ranges
+  take(48);
+  take(256);
+  take(scan * 8);
+  take(scan * 8);
+  take((int64_t)(p.depth_passes + p.tile_passes) * 1024);
+  take(p.depth_passes * sort_n * 1024);
+  take(p.tile_passes * sort_d * 1024);
+  for (int i = 0; i < 4; ++i) take(n * 4);
+  for (int i = 0; i < 4; ++i) take(d * 4);
+  take((d / 512 + 2) * 4);
+  return o;
+}
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
@@ -52,11 +85,12 @@ extern "C" sixdgs_status sixdgs_render_fwd_static(int64_t n, int32_t sh_degree, 
   sixdgs_plan plan;
   sixdgs_status e = sixdgs_plan_init(n, sh_degree, cams, n_cams, &fwd, 0, &plan);
   if (e != SIXDGS_OK) return e;
-  if (plan.ws_bytes > (int64_t)SIXDGS_STATIC_WS_BYTES) return SIXDGS_ERR_WORKSPACE;
+  if (limit_bytes(plan) > (int64_t)SIXDGS_STATIC_WS_BYTES || plan.ws_bytes > (int64_t)kArrayBytes)
+    return SIXDGS_ERR_WORKSPACE;
   void* ws = nullptr;
   e = static_ws_address(&ws);
   if (e != SIXDGS_OK) return e;
-  const size_t bytes = SIXDGS_STATIC_WS_BYTES;
+  const size_t bytes = kArrayBytes;
   e = sixdgs_condition_project(&plan, scene, cams, ws, bytes, status_dev, stream);
   if (e != SIXDGS_OK) return e;
   e = sixdgs_bin_sort(&plan, ws, bytes, status_dev, stream);
