@@ -3,6 +3,7 @@
 #include <cstring>
 #include <initializer_list>
 
+#include "bin.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 #include "stage.cuh"
@@ -293,7 +294,7 @@ sixdgs_status sixdgs_plan_init(int64_t n, int32_t sh_degree, const sixdgs_camera
   plan->off[WS_ZERO_END] = o;
   take(WS_ORDER, tiles * 16);
   take(WS_VIS, n_pairs * 16);
-  take(WS_VIS_COUNT, (n + kStageTile - 1) / kStageTile * 4);
+  take(WS_VIS_COUNT, vis_segments_max(n) * 4);
   take(WS_DUP, dup_capacity * 8);
   take(WS_SORT_K, dup_capacity * 4);
   take(WS_SORT_V, dup_capacity * 4);
@@ -324,8 +325,9 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
   a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
   a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
   a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
-  a.segments = (uint32_t)((p->n + kStageTile - 1) / kStageTile);
-  a.segment_size = (uint32_t)(kStageTile * p->n_cams);
+  a.views = view_parts(p->n, p->n_cams);
+  a.segments = (uint32_t)((p->n + kStageTile - 1) / kStageTile) * a.views.parts;
+  a.segment_size = (uint32_t)kStageTile * a.views.views;
   a.state = ws_ptr<uint32_t>(ws, p, WS_STATE);
   a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN);
   a.order = ws_ptr<uint4>(ws, p, WS_ORDER);

@@ -45,6 +45,11 @@ struct __align__(32) TileCounters {
   uint32_t pad[6];
 };
 
+// Division of a frame's views among the projection's CTAs (bin.cuh).
+struct ViewParts {
+  uint32_t parts, views;
+};
+
 struct ProjectArgs {
   const CamRec* cams;
   int32_t n_cams;
@@ -66,6 +71,7 @@ struct ProjectArgs {
   uint32_t* depth_key;
   uint4* vis;             // visible queue of the binning (bin.cuh)
   uint32_t* vis_count;
+  ViewParts views;        // set by the launch
   TileCounters* tile;     // their counts are added to
   float* grad_rec;   // zeroed for every visible pair (read by the backward); null: inference plan
   int32_t bulk;      // 1: every parameter plane segment can be staged with bulk copies
@@ -93,8 +99,10 @@ struct BinArgs {
   const uint4* vis;                // visible queue (bin.cuh)
   const uint32_t* vis_count;
   uint32_t segments;               // of the queue
-  uint32_t segment_size;
-  uint32_t scatter_grid;           // CTAs that share the segments (set by the launch)
+  uint32_t segment_size;           // entries that one can hold
+  ViewParts views;
+  // set by the launch: CTAs that share the segments, CTAs of one segment, entries of a step
+  uint32_t scatter_grid, scatter_split, scatter_step;
   uint32_t* state;                 // kBinWords words
   unsigned long long* scan_state;  // one word per scan block
   uint4* order;                    // TileWork of every tile, longest list class first
@@ -182,7 +190,7 @@ struct ScaleRotationArgs {
   int32_t* status;
 };
 
-void launch_project_fwd(const ProjectArgs& a, cudaStream_t stream);
+void launch_project_fwd(ProjectArgs a, cudaStream_t stream);
 void launch_scale_rotation(const ScaleRotationArgs& a, cudaStream_t stream);
 void launch_cond_cache(const CondCacheArgs& a, cudaStream_t stream);
 void launch_peak_probe(int kind, int64_t iters, float* out, int blocks, cudaStream_t stream);

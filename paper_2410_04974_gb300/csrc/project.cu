@@ -279,13 +279,13 @@ __device__ __forceinline__ void count_big(const ProjectArgs& a, const CamRec* ca
 }
 
 // Queues the pairs of Gaussian g0 + gl that are visible to cameras v0, v0 +
-// step, ...
-__device__ __forceinline__ void queue_visible(const ProjectArgs& a, const CamRec* cams, int v0, int step, int64_t g0,
-                                              int gl, bool ok, const float* mp, const float* md, const M3& A,
+// step, ... below v_end.
+__device__ __forceinline__ void queue_visible(const ProjectArgs& a, const CamRec* cams, int v0, int v_end, int step,
+                                              int64_t g0, int gl, bool ok, const float* mp, const float* md, const M3& A,
                                               const M3& Sdi, float alpha, float lam, uint32_t& s_count,
                                               uint16_t* s_queue) {
   const int lane = threadIdx.x & 31;
-  for (int v = v0; v < a.n_cams; v += step) {
+  for (int v = v0; v < v_end; v += step) {
     bool vis = false;
     if (ok) {
       const SliceView sv = slice_view(mp, md, A, Sdi, alpha, lam, cams[v]);
@@ -351,8 +351,11 @@ __global__ void __launch_bounds__(kThreads ? kThreads : kStageTile, kThreads == 
   for (int i = threadIdx.x; i < a.n_cams; i += blockDim.x) s_cams[i] = a.cams[i];
   if (threadIdx.x == 0) s_count = s_big.count = 0;
   if (threadIdx.x < kStageTile / 32) s_ok[threadIdx.x] = 0;
-  const int64_t g0 = (int64_t)blockIdx.x * kStageTile;
-  uint4* vis_seg = a.vis + g0 * a.n_cams;   // this CTA's segment of the visible queue
+  // the CTA's Gaussians and (staged path) views, and its segment of the visible queue
+  const ViewParts vp = kStaged ? a.views : ViewParts{1u, 1u};
+  const int64_t g0 = (int64_t)(blockIdx.x / vp.parts) * kStageTile;
+  const int v_first = (int)(blockIdx.x % vp.parts * vp.views), v_end = min(v_first + (int)vp.views, a.n_cams);
+  uint4* vis_seg = a.vis + vis_base(blockIdx.x, n, a.n_cams, vp);
   const int m = (int)min((int64_t)kStageTile, n - g0);
   // group 0: mu_p, mu_d, the conditioning planes and lambda (phase A);
   // group 1: the SH coefficients, in flight while phase A runs
@@ -446,7 +449,7 @@ __global__ void __launch_bounds__(kThreads ? kThreads : kStageTile, kThreads == 
       if constexpr (kThreads > kStageTile) {
         if (ok) atomicOr(&s_ok[tid >> 5], 1u << (tid & 31));
       } else {
-        queue_visible(a, s_cams, 0, 1, g0, tid, ok, mp, md, cs.A, sym_upper(cs.Sdi), cs.alpha, lam, s_count, s_queue);
+        queue_visible(a, s_cams, v_first, v_end, 1, g0, tid, ok, mp, md, cs.A, sym_upper(cs.Sdi), cs.alpha, lam, s_count, s_queue);
       }
     }
   }
@@ -471,8 +474,8 @@ __global__ void __launch_bounds__(kThreads ? kThreads : kStageTile, kThreads == 
       for (int k = 0; k < 9; ++k) A.m[k] = cp[k * kStageTile];
       const M3 Sdi = load_sym(cp, 9);
       const float alpha = cp[21 * kStageTile], lam = cp[22 * kStageTile];
-      queue_visible(a, s_cams, tid / kStageTile, kThreads / kStageTile, g0, gv, ok, mp, md, A, Sdi, alpha, lam, s_count,
-                    s_queue);
+      queue_visible(a, s_cams, v_first + tid / kStageTile, v_end, kThreads / kStageTile, g0, gv, ok, mp, md, A, Sdi,
+                    alpha, lam, s_count, s_queue);
     }
   }
   if (!stage_wait(s_bars, 1, bulk, a.spin_budget)) raise_status(a.status, SIXDGS_ERR_TIMEOUT);
@@ -505,11 +508,11 @@ __global__ void __launch_bounds__(kThreads ? kThreads : kStageTile, kThreads == 
 
 template <bool kCached, int kThreads>
 static void launch_project(const ProjectArgs& a, cudaStream_t stream) {
-  const int64_t blocks = (a.n + kStageTile - 1) / kStageTile;
+  const int64_t blocks = (a.n + kStageTile - 1) / kStageTile * a.views.parts;
   const ProjPlanes pp = proj_planes(kCached, a.sh_degree, a.lambda_raw != nullptr);
   const size_t smem = sizeof(CamRec) * (size_t)a.n_cams +
                       (kThreads ? (size_t)pp.count * kStageTile * sizeof(float) +
-                                      (size_t)kStageTile * a.n_cams * sizeof(uint16_t)
+                                      (size_t)kStageTile * a.views.views * sizeof(uint16_t)
                                 : 0);
   if (smem > 40 * 1024)   // the static shared memory counts towards the 48 KB as well
     cudaFuncSetAttribute(project_fwd_kernel<kCached, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -520,12 +523,13 @@ static void launch_project(const ProjectArgs& a, cudaStream_t stream) {
 template <bool kCached>
 static void launch_project_views(const ProjectArgs& a, cudaStream_t stream) {
   if (a.n_cams == 1) launch_project<kCached, 0>(a, stream);
-  else if (a.n_cams < kProjWideViews) launch_project<kCached, kStageTile>(a, stream);
+  else if (a.views.views < kProjWideViews) launch_project<kCached, kStageTile>(a, stream);
   else launch_project<kCached, kProjThreads>(a, stream);
 }
 
-void launch_project_fwd(const ProjectArgs& a, cudaStream_t stream) {
+void launch_project_fwd(ProjectArgs a, cudaStream_t stream) {
   if (a.n == 0) return;
+  a.views = view_parts(a.n, a.n_cams);
   if (a.cond_cache) launch_project_views<true>(a, stream);
   else launch_project_views<false>(a, stream);
 }

@@ -44,6 +44,7 @@ def _expected(r):
     ("cube", 1, 1, (64, 64), 1.0),
     ("cube", 127, 2, (33, 17), 1.0),
     ("cube", 3001, 9, (97, 65), 1.0),         # 9 views: the 48-camera set-up launch, three short segments each
+    ("cube", 1500, 7, (97, 65), 1.0),         # views divided among CTAs: 3, 3 and 1
     ("cube", 3000, 1, (1920, 1080), 1.0),     # rectangles of dozens of tiles
     ("shell", 30_000, 1, (128, 128), 1.0),    # lists of several hundred
     ("shell", 9_000, 2, (48, 32), 1.0),       # lists of one to four thousand
