@@ -73,7 +73,7 @@ KERNEL_SOURCES = {
     "blend_fused_kernel": ["raster.cu"], "blend_bwd_kernel": ["raster.cu"], "blend_fwd_kernel": ["raster.cu"],
     "project_fwd_kernel": ["project.cu", "bin.cuh", "cond.cuh", "sh.cuh", "mat3.cuh", "stage.cuh"],
     "bin_scan_kernel": ["sort.cu", "bin.cuh"], "bin_scatter_kernel": ["sort.cu", "bin.cuh"],
-    "bin_sort_kernel": ["sort.cu", "bin.cuh"],
+    "bin_sort_kernel": ["sort.cu", "bin.cuh"], "bin_count_kernel": ["sort.cu", "bin.cuh"],
     "param_bwd_kernel": ["project_bwd.cu", "cond.cuh", "mat3.cuh", "sh.cuh", "stage.cuh"],
     "scale_rotation_kernel": ["scale_rotation.cu", "cond.cuh", "mat3.cuh"],
 }

@@ -146,6 +146,32 @@ bool valid_fwd_scene(const sixdgs_plan* p, const sixdgs_scene* s) {
          (p->n == 0 || (s->mu_p && s->mu_d && s->sh && (s->cond_cache || (s->l_raw && s->opacity_logit))));
 }
 
+BinArgs bin_args(const sixdgs_plan* p, void* ws, int32_t* status_dev) {
+  BinArgs a;
+  a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
+  a.n_cams = p->n_cams;
+  a.n = (uint32_t)p->n;
+  a.total_tiles = (uint32_t)p->total_tiles;
+  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
+  a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
+  a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
+  a.views = view_parts(p->n, p->n_cams);
+  a.segments = (uint32_t)((p->n + kStageTile - 1) / kStageTile) * a.views.parts;
+  a.segment_size = (uint32_t)kStageTile * a.views.views;
+  a.state = ws_ptr<uint32_t>(ws, p, WS_STATE);
+  a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN);
+  a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
+  a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
+  a.capacity = (uint64_t)p->dup_capacity;
+  a.dup = ws_ptr<uint64_t>(ws, p, WS_DUP);
+  a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
+  a.sorted_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTEDKEY);
+  a.counts = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_COUNTS);
+  a.spin_budget = spin_budget(p);
+  a.status = status_dev;
+  return a;
+}
+
 // sixdgs_condition_project; loss (may be null) is set to zero on the way.
 sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, const sixdgs_camera* cams, void* ws,
                             size_t ws_bytes, double* loss, int32_t* status_dev, sixdgs_stream_t stream_) {
@@ -205,7 +231,11 @@ sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, con
                               a.cond_cache ? nullptr : a.l_raw, a.cond_cache ? nullptr : a.opacity_logit});
   a.spin_budget = spin_budget(p);
   a.status = status_dev;
+  a.defer_big = defer_big_rects(p->n, p->n_cams, p->total_tiles);
   launch_project_fwd(a, stream);
+  if (a.defer_big && p->n > 0 &&
+      launch_bin_count(bin_args(p, ws, status_dev), sm_count(), stream) != cudaSuccess)
+    return SIXDGS_ERR_CUDA;
   return launch_status();
 }
 
@@ -317,28 +347,7 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
   sixdgs_status e = check_ws(p, ws, ws_bytes);
   if (e != SIXDGS_OK) return e;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-  BinArgs a;
-  a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
-  a.n_cams = p->n_cams;
-  a.n = (uint32_t)p->n;
-  a.total_tiles = (uint32_t)p->total_tiles;
-  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
-  a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
-  a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
-  a.views = view_parts(p->n, p->n_cams);
-  a.segments = (uint32_t)((p->n + kStageTile - 1) / kStageTile) * a.views.parts;
-  a.segment_size = (uint32_t)kStageTile * a.views.views;
-  a.state = ws_ptr<uint32_t>(ws, p, WS_STATE);
-  a.scan_state = ws_ptr<unsigned long long>(ws, p, WS_SCAN);
-  a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
-  a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
-  a.capacity = (uint64_t)p->dup_capacity;
-  a.dup = ws_ptr<uint64_t>(ws, p, WS_DUP);
-  a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
-  a.sorted_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTEDKEY);
-  a.counts = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_COUNTS);
-  a.spin_budget = spin_budget(p);
-  a.status = status_dev;
+  const BinArgs a = bin_args(p, ws, status_dev);
   if (launch_bin(a, sm_count(), stream) != cudaSuccess) return SIXDGS_ERR_CUDA;
   return launch_status();
 }

@@ -72,6 +72,7 @@ struct ProjectArgs {
   uint4* vis;             // visible queue of the binning (bin.cuh)
   uint32_t* vis_count;
   ViewParts views;        // set by the launch
+  bool defer_big;         // leaves the rectangles of many tiles to bin_count_kernel
   TileCounters* tile;     // their counts are added to
   float* grad_rec;   // zeroed for every visible pair (read by the backward); null: inference plan
   int32_t bulk;      // 1: every parameter plane segment can be staged with bulk copies
@@ -191,6 +192,7 @@ struct ScaleRotationArgs {
 };
 
 void launch_project_fwd(ProjectArgs a, cudaStream_t stream);
+cudaError_t launch_bin_count(BinArgs a, int sms, cudaStream_t stream);
 void launch_scale_rotation(const ScaleRotationArgs& a, cudaStream_t stream);
 void launch_cond_cache(const CondCacheArgs& a, cudaStream_t stream);
 void launch_peak_probe(int kind, int64_t iters, float* out, int blocks, cudaStream_t stream);

@@ -139,7 +139,6 @@ __device__ __forceinline__ M3 load_sym(const float* cp, int k0) {
 // Pairs of a CTA with more tiles than one thread should count alone.
 struct BigRects {
   static constexpr int kMax = 128;
-  static constexpr uint32_t kTiles = 16;   // above: a warp counts them together
   uint32_t count;
   uint4 entry[kMax];
 };
@@ -147,8 +146,9 @@ struct BigRects {
 // Adds one pair's duplicates to the counts of its view's tiles (no result is
 // waited for).
 __device__ __forceinline__ void count_tiles(TileCounters* c, int32_t tiles_x, uint4 e, uint32_t ntiles,
-                                            BigRects& big) {
-  if (ntiles > BigRects::kTiles) {
+                                            bool defer, BigRects& big) {
+  if (ntiles > kBigRect) {
+    if (defer) return;
     const uint32_t k = atomicAdd(&big.count, 1u);
     if (k < BigRects::kMax) {
       big.entry[k] = e;
@@ -253,7 +253,7 @@ __device__ __forceinline__ void project_pair(const ProjectArgs& a, Beta beta, co
       a.rect[pair] =
           make_ushort4((unsigned short)x0, (unsigned short)x1, (unsigned short)y0, (unsigned short)y1);
       entry = vis_entry((uint32_t)pair, __float_as_uint(t[2]), (uint32_t)x0, (uint32_t)x1, (uint32_t)y0, (uint32_t)y1);
-      count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, big);
+      count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, a.defer_big, big);
     }
   }
   a.ntiles[pair] = ntiles;

@@ -88,9 +88,16 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t& total,
 // predecessors and publishes the inclusive prefix.  Returns the exclusive
 // prefix.  The wait is bounded by a clock budget; on expiry the status word
 // gets SIXDGS_ERR_TIMEOUT and the callers carry on with clamped ranges.
+// first: the words of the 32 blocks before, one per lane, as scan_ahead read
+// them before the block's own counts, so that a block whose predecessors are
+// long done does not wait for them a second time.
+__device__ __forceinline__ unsigned long long scan_ahead(const unsigned long long* state, uint32_t tile) {
+  const long long idx = (long long)tile - 1 - (threadIdx.x & 31);
+  return idx >= 0 ? ld_volatile64(&state[idx]) : kScanInc;
+}
 __device__ unsigned long long scan_lookback(unsigned long long* state, uint32_t tile,
-                                            unsigned long long block_total, int64_t budget,
-                                            int32_t* status) {
+                                            unsigned long long block_total, unsigned long long first,
+                                            int64_t budget, int32_t* status) {
   const int lane = threadIdx.x & 31;
   if (tile == 0) {
     if (lane == 0) st_volatile64(&state[0], kScanInc | block_total);
@@ -101,9 +108,8 @@ __device__ unsigned long long scan_lookback(unsigned long long* state, uint32_t 
   long long p = (long long)tile - 1;
   const long long t0 = clock64();
   bool timed_out = false;
+  unsigned long long w = first;
   while (true) {
-    long long idx = p - lane;
-    unsigned long long w = idx >= 0 ? ld_volatile64(&state[idx]) : kScanInc;
     uint32_t flag = (uint32_t)(w >> 62);
     uint32_t inc = __ballot_sync(0xffffffffu, flag == 2u);
     uint32_t not_ready = __ballot_sync(0xffffffffu, flag == 0u);
@@ -115,6 +121,8 @@ __device__ unsigned long long scan_lookback(unsigned long long* state, uint32_t 
         timed_out = true;
         break;
       }
+      const long long idx = p - lane;
+      w = idx >= 0 ? ld_volatile64(&state[idx]) : kScanInc;
       continue;
     }
     unsigned long long val = (lane <= i_inc) ? (w & kScanValMask) : 0ull;
@@ -123,6 +131,8 @@ __device__ unsigned long long scan_lookback(unsigned long long* state, uint32_t 
     excl += val;
     if (i_inc < 32) break;
     p -= 32;
+    const long long idx = p - lane;
+    w = idx >= 0 ? ld_volatile64(&state[idx]) : kScanInc;
   }
   if (lane == 0) {
     if (timed_out) raise_status(status, SIXDGS_ERR_TIMEOUT);
@@ -174,11 +184,12 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   const uint32_t block = blockIdx.x;
   const uint32_t t = block * kScanTile + tid;
   const bool valid = t < a.total_tiles;
+  const unsigned long long ahead = tid < 32 ? scan_ahead(a.scan_state, block) : 0ull;
   const uint32_t cnt = valid ? a.tile[t].count : 0u;
   uint32_t total;
   const uint32_t excl = block_excl_scan<kBinThreads>(cnt, total, s_warp);
   if (tid < 32) {
-    const unsigned long long e = scan_lookback(a.scan_state, block, total, a.spin_budget, a.status);
+    const unsigned long long e = scan_lookback(a.scan_state, block, total, ahead, a.spin_budget, a.status);
     if (tid == 0) s_excl = e;
   }
   // counters of the kernels that follow; the pair counters behind the first two
@@ -209,7 +220,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
 // Duplicates to their tiles, and the tile order
 // --------------------------------------------------------------------------
 // A CTA takes a segment of the visible queue, 256 entries at a time (where there
-// are fewer segments than CTAs, a part of one, down to 32 entries), and
+// are fewer segments than CTAs, a part of one), and
 // spreads their duplicates over its threads whatever the rectangles' sizes:
 // duplicate o goes to thread o % 128, which finds its entry by a binary search
 // of the entries' prefix sums in shared memory.  Bound by L2 requests (one
@@ -220,7 +231,8 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
 constexpr int kScatterThreads = 128;
 constexpr int kScatterEntries = 2 * kScatterThreads;
 constexpr int kScatterBatch = 4;
-__global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a) {
+template <bool kCount>
+__device__ __forceinline__ void scatter(const BinArgs& a) {
   after_previous();
   constexpr int kWarps = kScatterThreads / 32;
   __shared__ uint32_t s_class[kClasses], s_base[kClasses], s_longer[kClasses];
@@ -230,7 +242,7 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
   __shared__ uint32_t s_vis;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) s_vis = 0u;
-  if (blockIdx.x >= a.scatter_grid) {
+  if (!kCount && blockIdx.x >= a.scatter_grid) {
     // these CTAs build the tile order: longest class first, any order within a
     // class (it decides when a tile is worked on, never a result)
     if (warp == 0) {   // tiles of longer classes: a suffix sum over the 64 classes
@@ -287,6 +299,7 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
         const uint32_t i = c0 + 2 * tid + h;
         e[h] = 2 * tid + h < step && i < count ? vis[i] : make_uint4(0u, 0u, 0u, 0u);
         nt[h] = ((e[h].z >> 16) - (e[h].z & 0xffffu)) * ((e[h].w >> 16) - (e[h].w & 0xffffu));
+        if (kCount && nt[h] <= kBigRect) nt[h] = 0u;   // the projection counted them
       }
       uint32_t total;
       const uint32_t excl = block_excl_scan<kScatterThreads>(nt[0] + nt[1], total, s_warp);
@@ -320,21 +333,29 @@ __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a)
             const uint32_t row = rect_row(local, w);
             const uint32_t tile = en.x + row * (en.y >> 16) + (local - row * w);
             key[k] = ((uint64_t)en.w << 32) | en.z;
-            if (tile < a.total_tiles) pos[k] = atomicAdd(&a.tile[tile].cursor, 1u);
+            if (tile < a.total_tiles) {
+              if constexpr (kCount) atomicAdd(&a.tile[tile].count, 1u);
+              else pos[k] = atomicAdd(&a.tile[tile].cursor, 1u);
+            }
           }
         }
 #pragma unroll
         for (int k = 0; k < kScatterBatch; ++k)
-          if (pos[k] < a.capacity) a.dup[pos[k]] = key[k];
+          if (!kCount && pos[k] < a.capacity) a.dup[pos[k]] = key[k];
       }
       __syncthreads();
     }
   }
+  if (kCount) return;
   visible = __reduce_add_sync(0xffffffffu, visible);
   if (lane == 0 && visible) atomicAdd(&s_vis, visible);
   __syncthreads();
   if (tid == 0 && s_vis) atomicAdd(&a.counts[0], s_vis);
 }
+
+__global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a) { scatter<false>(a); }
+// The counts of the rectangles that the projection left (defer_big_rects).
+__global__ void __launch_bounds__(kScatterThreads) bin_count_kernel(BinArgs a) { scatter<true>(a); }
 
 // --------------------------------------------------------------------------
 // Sort of one tile's entries
@@ -742,10 +763,7 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
 // SM, each with the segments of its stride, and one per 128 tiles for the order;
 // the sort, which takes its tiles from a queue, a whole number of clusters, at
 // most 4 CTAs per SM.
-cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream) {
-  const uint32_t blocks = std::max(1u, (a.total_tiles + kScanTile - 1) / kScanTile);
-  cudaError_t e = launch_after(bin_scan_kernel, blocks, kBinThreads, 0, 1, stream, a);
-  if (e != cudaSuccess) return e;
+static void share_segments(BinArgs& a, int sms) {
   // 16 CTAs per SM: with fewer segments, several CTAs take the steps of one in
   // turn (the binning of 20 views of 6,660 Gaussians at 1408^2, 1.1 M duplicates
   // in 53 segments before: 152 -> 78 us; of 4 views 43 -> 29 us, with the
@@ -755,10 +773,22 @@ cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream) {
   a.scatter_step = kScatterEntries;
   if (a.segments && 2u * a.segments <= most_ctas) {
     const uint32_t share = (a.segment_size * a.segments + most_ctas - 1) / most_ctas;
-    a.scatter_step = std::min((share + 31u) & ~31u, (uint32_t)kScatterEntries);
+    a.scatter_step = std::min((share + 1u) & ~1u, (uint32_t)kScatterEntries);
     a.scatter_split = std::min(most_ctas / a.segments, (a.segment_size + a.scatter_step - 1) / a.scatter_step);
   }
   a.scatter_grid = std::min(a.segments * a.scatter_split, most_ctas);
+}
+
+cudaError_t launch_bin_count(BinArgs a, int sms, cudaStream_t stream) {
+  share_segments(a, sms);
+  return launch_after(bin_count_kernel, a.scatter_grid, kScatterThreads, 0, 1, stream, a);
+}
+
+cudaError_t launch_bin(BinArgs a, int sms, cudaStream_t stream) {
+  const uint32_t blocks = std::max(1u, (a.total_tiles + kScanTile - 1) / kScanTile);
+  cudaError_t e = launch_after(bin_scan_kernel, blocks, kBinThreads, 0, 1, stream, a);
+  if (e != cudaSuccess) return e;
+  share_segments(a, sms);
   const uint32_t order = std::max(1u, (a.total_tiles + kScatterThreads - 1) / kScatterThreads);
   e = launch_after(bin_scatter_kernel, a.scatter_grid + order, kScatterThreads, 0, 1, stream, a);
   if (e != cudaSuccess) return e;
