@@ -167,6 +167,7 @@ BinArgs bin_args(const sixdgs_plan* p, void* ws, int32_t* status_dev) {
   a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
   a.sorted_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTEDKEY);
   a.counts = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_COUNTS);
+  a.scan_tickets = false;
   a.spin_budget = spin_budget(p);
   a.status = status_dev;
   return a;

@@ -84,6 +84,7 @@ struct ProjectArgs {
 enum BinWord {
   kBinClass = 0,         // tiles of every list-length class
   kBinCursor = 64,       // next place of every class in the tile order
+  kBinTicket = 128,      // blocks of the list scan that have started (scan_tickets)
   kBinQueue = 129,       // sort work counter
   kBinOver = 130,        // tiles with lists above 16384, 4096, 2048, 1024, 512 and 0 entries
   kBinWords = 192
@@ -102,6 +103,7 @@ struct BinArgs {
   uint32_t segments;               // of the queue
   uint32_t segment_size;           // entries that one can hold
   ViewParts views;
+  bool scan_tickets;               // set by the launch: blocks of the scan number themselves
   // set by the launch: CTAs that share the segments, CTAs of one segment, entries of a step
   uint32_t scatter_grid, scatter_split, scatter_step;
   uint32_t* state;                 // kBinWords words
