@@ -53,24 +53,25 @@ __device__ __forceinline__ void st_volatile64(unsigned long long* p, unsigned lo
 
 // Exclusive block scan of one value per thread; returns the thread's prefix
 // and the block total through `total`.  s_warp needs THREADS/32 + 1 words.
-template <int THREADS>
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t& total, uint32_t* s_warp) {
+// T: wide enough for the total.
+template <int THREADS, typename T>
+__device__ __forceinline__ T block_excl_scan(T v, T& total, T* s_warp) {
   constexpr int WARPS = THREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t incl = v;
+  T incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    T y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
   if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    uint32_t w = lane < WARPS ? s_warp[lane] : 0u;
-    uint32_t wi = w;
+    T w = lane < WARPS ? s_warp[lane] : (T)0;
+    T wi = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
+      T y = __shfl_up_sync(0xffffffffu, wi, o);
       if (lane >= o) wi += y;
     }
     if (lane < WARPS) s_warp[lane] = wi - w;
@@ -78,7 +79,7 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t& total,
   }
   __syncthreads();
   total = s_warp[WARPS];
-  uint32_t r = s_warp[warp] + incl - v;
+  T r = s_warp[warp] + incl - v;
   __syncthreads();
   return r;
 }
@@ -180,7 +181,7 @@ __device__ __forceinline__ uint32_t count_class(uint32_t cls, bool valid, uint32
 // atomic, 0.8 us of 90 for 175k Gaussians at 1408^2, 1.2 of 47 for 6,660.)
 __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   after_previous();
-  __shared__ uint32_t s_warp[kBinWarps + 1];
+  __shared__ unsigned long long s_warp[kBinWarps + 1];
   __shared__ uint32_t s_class[kClasses];
   __shared__ unsigned long long s_excl;
   __shared__ uint32_t s_block;
@@ -197,8 +198,10 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   const bool valid = t < a.total_tiles;
   const unsigned long long ahead = tid < 32 ? scan_ahead(a.scan_state, block) : 0ull;
   const uint32_t cnt = valid ? a.tile[t].count : 0u;
-  uint32_t total;
-  const uint32_t excl = block_excl_scan<kBinThreads>(cnt, total, s_warp);
+  // 64 bits: a block's tiles may hold 2^32 duplicates or more (16.8 million
+  // Gaussians on each), which the capacity check has to see
+  unsigned long long total;
+  const unsigned long long excl = block_excl_scan<kBinThreads>((unsigned long long)cnt, total, s_warp);
   if (tid < 32) {
     const unsigned long long e = scan_lookback(a.scan_state, block, total, ahead, a.spin_budget, a.status);
     if (tid == 0) s_excl = e;
