@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
 // walks its own entry's duplicates needs neither search nor barrier, but more
 // and emptier atomic instructions: 60 instead of 51 us at 300k / 8 x 800^2.)
 constexpr int kScatterThreads = 128;
-constexpr int kScatterEntries = 2 * kScatterThreads;
+static_assert(kScatterEntries == 2 * kScatterThreads, "two entries a thread");
 constexpr int kScatterBatch = 4;
 template <bool kCount>
 __device__ __forceinline__ void scatter(const BinArgs& a) {
@@ -779,19 +779,10 @@ __global__ void __launch_bounds__(kBinThreads, 4) bin_sort_kernel(BinArgs a) {
 // the sort, which takes its tiles from a queue, a whole number of clusters, at
 // most 4 CTAs per SM.
 static void share_segments(BinArgs& a, int sms) {
-  // 16 CTAs per SM: with fewer segments, several CTAs take the steps of one in
-  // turn (the binning of 20 views of 6,660 Gaussians at 1408^2, 1.1 M duplicates
-  // in 53 segments before: 152 -> 78 us; of 4 views 43 -> 29 us, with the
-  // projection's division of the views)
-  const uint32_t most_ctas = (uint32_t)sms * 16u;
-  a.scatter_split = 1u;
-  a.scatter_step = kScatterEntries;
-  if (a.segments && 2u * a.segments <= most_ctas) {
-    const uint32_t share = (a.segment_size * a.segments + most_ctas - 1) / most_ctas;
-    a.scatter_step = std::min((share + 1u) & ~1u, (uint32_t)kScatterEntries);
-    a.scatter_split = std::min(most_ctas / a.segments, (a.segment_size + a.scatter_step - 1) / a.scatter_step);
-  }
-  a.scatter_grid = std::min(a.segments * a.scatter_split, most_ctas);
+  const ScatterShare s = scatter_share(a.segments, a.segment_size, a.total_tiles, sms);
+  a.scatter_grid = s.grid;
+  a.scatter_split = s.split;
+  a.scatter_step = s.step;
 }
 
 cudaError_t launch_bin_count(BinArgs a, int sms, cudaStream_t stream) {
