@@ -384,8 +384,9 @@ sixdgs_status sixdgs_scale_rotation(int64_t n, const float* l_raw_dev, float* ro
  * with a fixed budget), or loops that must never call cudaMalloc.  It runs
  * the same work as sixdgs_condition_project + sixdgs_bin_sort +
  * sixdgs_raster_fwd (no loss) and writes the same images, but keeps the
- * frame's workspace in one array (256 MiB) that lives in the library's device
- * memory.  Every GPU that loads the library
+ * frame's workspace in one array of SIXDGS_STATIC_WS_BYTES (32 MiB) that
+ * lives in the library's device memory (a frame of many tiles is binned and
+ * blended in bands of tiles, with the same result).  Every GPU that loads the library
  * holds that array until the process exits.  The call allocates nothing
  * (no cudaMalloc, cudaFree or allocating library routine).
  *

@@ -151,7 +151,9 @@ BinArgs bin_args(const sixdgs_plan* p, void* ws, int32_t* status_dev) {
   a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
   a.n_cams = p->n_cams;
   a.n = (uint32_t)p->n;
+  a.tile_first = 0;
   a.total_tiles = (uint32_t)p->total_tiles;
+  a.band = -1;
   a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
   a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
   a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
@@ -173,9 +175,48 @@ BinArgs bin_args(const sixdgs_plan* p, void* ws, int32_t* status_dev) {
   return a;
 }
 
+// Byte offsets of the workspace sections, with tile state for tile_slots tiles;
+// returns the size.
+int64_t lay_out(sixdgs_plan* plan, int64_t tile_slots) {
+  const int64_t n_pairs = plan->n_pairs, tiles = tile_slots, dups = plan->dup_capacity;
+  const sixdgs_settings& st = plan->settings;
+  int64_t o = 0;
+  auto take = [&](int section, int64_t bytes) {
+    plan->off[section] = o;
+    o = align_up(o + bytes, 256);
+  };
+  take(SIXDGS_WS_CAMS, (int64_t)plan->n_cams * (int64_t)sizeof(CamRec));
+  take(SIXDGS_WS_REC, n_pairs * (int64_t)sizeof(PairRec));
+  take(SIXDGS_WS_NTILES, align_up(n_pairs, 4) * 4);
+  take(SIXDGS_WS_RECT, n_pairs * 8);
+  take(SIXDGS_WS_DEPTHKEY, n_pairs * 4);
+  take(SIXDGS_WS_GRADREC, st.inference ? 0 : n_pairs * 48);
+  take(SIXDGS_WS_RANGES, tiles * 8);
+  take(SIXDGS_WS_NWALK, st.store_aux ? plan->total_pixels * 4 : 0);
+  take(SIXDGS_WS_COUNTS, 48);
+  take(WS_COUNTERS, 64 * 4);
+  // cleared by condition_project (the binning leaves its own words clean)
+  plan->off[WS_ZERO] = o;
+  take(WS_STATE, kBinWords * 4);
+  take(WS_SCAN, (tiles + kScanTile - 1) / kScanTile * 8);
+  take(WS_TILE, tiles * (int64_t)sizeof(TileCounters));
+  plan->off[WS_ZERO_END] = o;
+  take(WS_ORDER, tiles * 16);
+  take(WS_VIS, n_pairs * 16);
+  take(WS_VIS_COUNT, vis_segments_max(plan->n) * 4);
+  take(WS_DUP, dups * 8);
+  take(WS_SORT_K, dups * 4);
+  take(WS_SORT_V, dups * 4);
+  plan->off[SIXDGS_WS_SORTED] = plan->off[WS_SORT_V];
+  plan->off[SIXDGS_WS_SORTEDKEY] = plan->off[WS_SORT_K];
+  return o;
+}
+
 // sixdgs_condition_project; loss (may be null) is set to zero on the way.
+// banded: the tiles are left uncounted.
 sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, const sixdgs_camera* cams, void* ws,
-                            size_t ws_bytes, double* loss, int32_t* status_dev, sixdgs_stream_t stream_) {
+                            size_t ws_bytes, double* loss, bool banded, int32_t* status_dev,
+                            sixdgs_stream_t stream_) {
   sixdgs_status e = check_ws(p, ws, ws_bytes);
   if (e != SIXDGS_OK) return e;
   if (!valid_fwd_scene(p, scene) || !cams) return SIXDGS_ERR_INVALID_ARG;
@@ -226,13 +267,13 @@ sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, con
   a.depth_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_DEPTHKEY);
   a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
   a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
-  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
+  a.tile = banded ? nullptr : ws_ptr<TileCounters>(ws, p, WS_TILE);
   a.grad_rec = p->settings.inference ? nullptr : ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
   a.bulk = bulk_planes(p->n, {a.mu_p, a.mu_d, a.sh, a.lambda_raw, a.cond_cache,
                               a.cond_cache ? nullptr : a.l_raw, a.cond_cache ? nullptr : a.opacity_logit});
   a.spin_budget = spin_budget(p);
   a.status = status_dev;
-  a.defer_big = defer_big_rects(p->n, p->n_cams, p->total_tiles);
+  a.defer_big = !banded && defer_big_rects(p->n, p->n_cams, p->total_tiles);
   launch_project_fwd(a, stream);
   if (a.defer_big && p->n > 0 &&
       launch_bin_count(bin_args(p, ws, status_dev), sm_count(), stream) != cudaSuccess)
@@ -240,7 +281,73 @@ sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, con
   return launch_status();
 }
 
+BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
+  BlendArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
+  a.n_cams = p->n_cams;
+  a.tile_w = p->settings.tile_w;
+  a.tile_h = p->settings.tile_h;
+  a.batch = p->settings.batch;
+  a.rec = ws_ptr<PairRec>(ws, p, SIXDGS_WS_REC);
+  a.n_pairs = (uint32_t)p->n_pairs;
+  a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
+  a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
+  a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
+  a.n_busy = ws_ptr<uint32_t>(ws, p, WS_STATE) + kBinOver + kBinLevels;
+  for (int i = 0; i < 3; ++i) a.bg[i] = p->settings.bg[i];
+  const double norm = p->settings.loss_norm > 0.f ? (double)p->settings.loss_norm
+                                                   : 3.0 * (double)p->total_pixels;
+  a.inv_count = (float)(1.0 / norm);
+  a.nwalk = p->settings.store_aux ? ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NWALK) : nullptr;
+  a.pair_counts = p->settings.count_pairs
+                      ? reinterpret_cast<unsigned long long*>(ws_ptr<char>(ws, p, SIXDGS_WS_COUNTS) + 16)
+                      : nullptr;
+  a.tile_queue = p->settings.persistent ? ws_ptr<uint32_t>(ws, p, WS_COUNTERS) + 32 : nullptr;
+  a.total_tiles = (uint32_t)p->total_tiles;
+  a.spin_budget = spin_budget(p);
+  return a;
+}
+
 }  // namespace
+
+namespace sixdgs {
+
+int64_t plan_bands(sixdgs_plan* p, int64_t ws_bytes) {
+  const int64_t tiles = p->total_tiles;
+  // per block of the list scan: its tiles' range, counters and order record, and its look-back word
+  constexpr int64_t kPerBlock = kScanTile * (8 + (int64_t)sizeof(TileCounters) + 16) + 8;
+  const int64_t fixed = lay_out(p, 0) + 4 * 256;   // four sections' alignment
+  const int64_t slots = std::min((ws_bytes - fixed) / kPerBlock * kScanTile, tiles);
+  if (slots <= 0) return 0;
+  p->ws_bytes = lay_out(p, slots);
+  return slots;
+}
+
+sixdgs_status render_banded(const sixdgs_plan* p, int64_t slots, const sixdgs_scene* scene, const sixdgs_camera* cams,
+                            void* ws, size_t ws_bytes, float* images_dev, int32_t* status_dev,
+                            sixdgs_stream_t stream_) {
+  sixdgs_status e = project_frame(p, scene, cams, ws, ws_bytes, nullptr, true, status_dev, stream_);
+  if (e != SIXDGS_OK) return e;
+  cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
+  BinArgs b = bin_args(p, ws, status_dev);
+  BlendArgs f = blend_args(p, ws);
+  f.images = images_dev;
+  f.status = status_dev;
+  b.band = 0;
+  for (int64_t first = 0; first < p->total_tiles; first += slots, ++b.band) {
+    b.tile_first = f.tile_first = (uint32_t)first;
+    b.total_tiles = f.total_tiles = (uint32_t)std::min(slots, p->total_tiles - first);
+    if (first > 0 && cudaMemsetAsync(b.tile, 0, b.total_tiles * sizeof(TileCounters), stream) != cudaSuccess)
+      return SIXDGS_ERR_CUDA;
+    if (p->n > 0 && launch_bin_count(b, sm_count(), stream) != cudaSuccess) return SIXDGS_ERR_CUDA;
+    if (launch_bin(b, sm_count(), stream) != cudaSuccess) return SIXDGS_ERR_CUDA;
+    launch_blend_fwd(f, f.total_tiles, stream);
+  }
+  return launch_status();
+}
+
+}  // namespace sixdgs
 
 extern "C" {
 
@@ -301,37 +408,7 @@ sixdgs_status sixdgs_plan_init(int64_t n, int32_t sh_degree, const sixdgs_camera
   while (((int64_t)1 << bits) < tiles) ++bits;
   plan->tile_passes = (bits + 7) / 8;
 
-  const int64_t np4 = align_up(n_pairs, 4);
-  int64_t o = 0;
-  auto take = [&](int section, int64_t bytes) {
-    plan->off[section] = o;
-    o = align_up(o + bytes, 256);
-  };
-  take(SIXDGS_WS_CAMS, (int64_t)n_cams * (int64_t)sizeof(CamRec));
-  take(SIXDGS_WS_REC, n_pairs * (int64_t)sizeof(PairRec));
-  take(SIXDGS_WS_NTILES, np4 * 4);
-  take(SIXDGS_WS_RECT, n_pairs * 8);
-  take(SIXDGS_WS_DEPTHKEY, n_pairs * 4);
-  take(SIXDGS_WS_GRADREC, st->inference ? 0 : n_pairs * 48);
-  take(SIXDGS_WS_RANGES, tiles * 8);
-  take(SIXDGS_WS_NWALK, st->store_aux ? pixels * 4 : 0);
-  take(SIXDGS_WS_COUNTS, 48);
-  take(WS_COUNTERS, 64 * 4);
-  // cleared by condition_project (the binning leaves its own words clean)
-  plan->off[WS_ZERO] = o;
-  take(WS_STATE, kBinWords * 4);
-  take(WS_SCAN, (tiles + kScanTile - 1) / kScanTile * 8);
-  take(WS_TILE, tiles * (int64_t)sizeof(TileCounters));
-  plan->off[WS_ZERO_END] = o;
-  take(WS_ORDER, tiles * 16);
-  take(WS_VIS, n_pairs * 16);
-  take(WS_VIS_COUNT, vis_segments_max(n) * 4);
-  take(WS_DUP, dup_capacity * 8);
-  take(WS_SORT_K, dup_capacity * 4);
-  take(WS_SORT_V, dup_capacity * 4);
-  plan->off[SIXDGS_WS_SORTED] = plan->off[WS_SORT_V];
-  plan->off[SIXDGS_WS_SORTEDKEY] = plan->off[WS_SORT_K];
-  plan->ws_bytes = o;
+  plan->ws_bytes = lay_out(plan, tiles);
   return SIXDGS_OK;
 }
 
@@ -340,7 +417,7 @@ size_t sixdgs_workspace_size(const sixdgs_plan* plan) { return plan ? (size_t)pl
 sixdgs_status sixdgs_condition_project(const sixdgs_plan* p, const sixdgs_scene* scene,
                                        const sixdgs_camera* cams, void* ws, size_t ws_bytes,
                                        int32_t* status_dev, sixdgs_stream_t stream) {
-  return project_frame(p, scene, cams, ws, ws_bytes, nullptr, status_dev, stream);
+  return project_frame(p, scene, cams, ws, ws_bytes, nullptr, false, status_dev, stream);
 }
 
 sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, int32_t* status_dev,
@@ -351,34 +428,6 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
   const BinArgs a = bin_args(p, ws, status_dev);
   if (launch_bin(a, sm_count(), stream) != cudaSuccess) return SIXDGS_ERR_CUDA;
   return launch_status();
-}
-
-static BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
-  BlendArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.cams = ws_ptr<CamRec>(ws, p, SIXDGS_WS_CAMS);
-  a.n_cams = p->n_cams;
-  a.tile_w = p->settings.tile_w;
-  a.tile_h = p->settings.tile_h;
-  a.batch = p->settings.batch;
-  a.rec = ws_ptr<PairRec>(ws, p, SIXDGS_WS_REC);
-  a.n_pairs = (uint32_t)p->n_pairs;
-  a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
-  a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
-  a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
-  a.n_busy = ws_ptr<uint32_t>(ws, p, WS_STATE) + kBinOver + kBinLevels;
-  for (int i = 0; i < 3; ++i) a.bg[i] = p->settings.bg[i];
-  const double norm = p->settings.loss_norm > 0.f ? (double)p->settings.loss_norm
-                                                   : 3.0 * (double)p->total_pixels;
-  a.inv_count = (float)(1.0 / norm);
-  a.nwalk = p->settings.store_aux ? ws_ptr<uint32_t>(ws, p, SIXDGS_WS_NWALK) : nullptr;
-  a.pair_counts = p->settings.count_pairs
-                      ? reinterpret_cast<unsigned long long*>(ws_ptr<char>(ws, p, SIXDGS_WS_COUNTS) + 16)
-                      : nullptr;
-  a.tile_queue = p->settings.persistent ? ws_ptr<uint32_t>(ws, p, WS_COUNTERS) + 32 : nullptr;
-  a.total_tiles = (uint32_t)p->total_tiles;
-  a.spin_budget = spin_budget(p);
-  return a;
 }
 
 sixdgs_status sixdgs_raster_fwd(const sixdgs_plan* p, void* ws, size_t ws_bytes, float* images_dev,
@@ -505,7 +554,7 @@ sixdgs_status sixdgs_render_batched(const sixdgs_plan* p, const sixdgs_scene* sc
     if (p->n > 0 && (!grad_mu_p || !grad_mu_d || !grad_l_raw || !grad_opacity_logit || !grad_sh))
       return SIXDGS_ERR_INVALID_ARG;
   }
-  e = project_frame(p, scene, cams_host, ws, ws_bytes, train ? loss_dev : nullptr, status_dev, stream);
+  e = project_frame(p, scene, cams_host, ws, ws_bytes, train ? loss_dev : nullptr, false, status_dev, stream);
   if (e != SIXDGS_OK) return e;
   e = sixdgs_bin_sort(p, ws, ws_bytes, status_dev, stream);
   if (e != SIXDGS_OK) return e;

@@ -73,7 +73,7 @@ struct ProjectArgs {
   uint32_t* vis_count;
   ViewParts views;        // set by the launch
   bool defer_big;         // leaves the rectangles of many tiles to bin_count_kernel
-  TileCounters* tile;     // their counts are added to
+  TileCounters* tile;     // their counts are added to; null: bin_count_kernel counts
   float* grad_rec;   // zeroed for every visible pair (read by the backward); null: inference plan
   int32_t bulk;      // 1: every parameter plane segment can be staged with bulk copies
   int64_t spin_budget;
@@ -87,16 +87,21 @@ enum BinWord {
   kBinTicket = 128,      // blocks of the list scan that have started (scan_tickets)
   kBinQueue = 129,       // sort work counter
   kBinOver = 130,        // tiles with lists above 16384, 4096, 2048, 1024, 512 and 0 entries
+  kBinBase = 136,        // duplicates of the bands so far, two 64-bit words used in turn
   kBinWords = 192
 };
 constexpr int kBinLevels = 5;   // 16384, 4096, 2048, 1024, 512 entries: what a CTA and its teams sort
 
-// Per-tile lists from the projection's tile counts and visible queue.
+// Per-tile lists from the projection's tile counts and visible queue.  A frame
+// whose tile state does not fit its workspace is taken in bands of consecutive
+// tiles, one after the other (render_banded); any other is one band.
 struct BinArgs {
   const CamRec* cams;
   int32_t n_cams;
   uint32_t n;                      // Gaussians per camera
-  uint32_t total_tiles;
+  uint32_t tile_first;             // first tile of the band
+  uint32_t total_tiles;            // tiles of the band
+  int32_t band;                    // its number; -1: the frame is one band
   TileCounters* tile;
   const uint4* vis;                // visible queue (bin.cuh)
   const uint32_t* vis_count;
@@ -129,6 +134,7 @@ struct BlendArgs {
   const uint2* ranges;
   const uint4* order;       // TileWork of every tile, longest lists first
   const uint32_t* n_busy;   // tiles with a list (the others come last)
+  uint32_t tile_first;      // first tile of the band (kernels.cuh, BinArgs)
   float bg[3];
   float* images;
   const float* targets;
@@ -206,5 +212,15 @@ void launch_param_bwd(const ProjectBwdArgs& a, cudaStream_t stream);
 
 // Tiles per block of the list scan.
 constexpr int kScanTile = 256;
+
+// A forward frame in bands of tiles, in a workspace whose tile state holds one
+// band (api.cu).  plan_bands lays the plan out for at most ws_bytes and returns
+// the tiles of a band, 0 if not even one block of the scan fits.  render_banded
+// projects once, then counts, bins and blends every band; the duplicates of all
+// bands share the capacity, and the images are those of the frame as a whole.
+int64_t plan_bands(sixdgs_plan* plan, int64_t ws_bytes);
+sixdgs_status render_banded(const sixdgs_plan* plan, int64_t band_tiles, const sixdgs_scene* scene,
+                            const sixdgs_camera* cams, void* ws, size_t ws_bytes, float* images_dev,
+                            int32_t* status_dev, sixdgs_stream_t stream);
 
 }  // namespace sixdgs

@@ -253,7 +253,7 @@ __device__ __forceinline__ void project_pair(const ProjectArgs& a, Beta beta, co
       a.rect[pair] =
           make_ushort4((unsigned short)x0, (unsigned short)x1, (unsigned short)y0, (unsigned short)y1);
       entry = vis_entry((uint32_t)pair, __float_as_uint(t[2]), (uint32_t)x0, (uint32_t)x1, (uint32_t)y0, (uint32_t)y1);
-      count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, a.defer_big, big);
+      if (a.tile) count_tiles(a.tile + cam.tile_offset, cam.tiles_x, entry, ntiles, a.defer_big, big);
     }
   }
   a.ntiles[pair] = ntiles;

@@ -760,7 +760,7 @@ __device__ __forceinline__ bool blend_unit(const BlendArgs& a, uint32_t u, Tile 
   const uint4 tw = a.order[min(u, a.total_tiles - 1)];
   const uint32_t busy = min(*a.n_busy, a.total_tiles);
   if (u < busy) {
-    if (tw.x < a.total_tiles) tile(tw);
+    if (tw.x - a.tile_first < a.total_tiles) tile(tw);
     return true;
   }
   const uint32_t first = busy + (u - busy) * (blockDim.x / 32);

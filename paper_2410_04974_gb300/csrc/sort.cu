@@ -198,6 +198,9 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   const bool valid = t < a.total_tiles;
   const unsigned long long ahead = tid < 32 ? scan_ahead(a.scan_state, block) : 0ull;
   const uint32_t cnt = valid ? a.tile[t].count : 0u;
+  // duplicates of the bands before, whose lists come first
+  unsigned long long* base = reinterpret_cast<unsigned long long*>(a.state + kBinBase);
+  const unsigned long long before = a.band > 0 ? base[a.band & 1] : 0ull;
   // 64 bits: a block's tiles may hold 2^32 duplicates or more (16.8 million
   // Gaussians on each), which the capacity check has to see
   unsigned long long total;
@@ -213,7 +216,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   if (block == 0 && tid == 11) a.state[kBinQueue] = 0u;
   __syncthreads();
   // lists beyond the duplicate capacity are cut there (and reported below)
-  const unsigned long long off = s_excl + excl;
+  const unsigned long long off = before + s_excl + excl;
   const uint32_t start = (uint32_t)min(off, (unsigned long long)a.capacity);
   const uint32_t end = (uint32_t)min(off + cnt, (unsigned long long)a.capacity);
   if (valid) {
@@ -224,7 +227,8 @@ __global__ void __launch_bounds__(kBinThreads) bin_scan_kernel(BinArgs a) {
   __syncthreads();
   if (tid < kClasses && s_class[tid]) atomicAdd(&a.state[kBinClass + tid], s_class[tid]);
   if (block == gridDim.x - 1 && tid == 0) {
-    const unsigned long long k = s_excl + total;
+    const unsigned long long k = before + s_excl + total;
+    if (a.band >= 0) base[(a.band + 1) & 1] = k;
     a.counts[1] = (uint32_t)min(k, 0xffffffffull);
     if (k > a.capacity) raise_status(a.status, SIXDGS_ERR_CAPACITY);
   }
@@ -278,7 +282,7 @@ __device__ __forceinline__ void scatter(const BinArgs& a) {
     const uint32_t t = (blockIdx.x - a.scatter_grid) * kScatterThreads + tid;
     const bool valid = t < a.total_tiles;
     const uint2 r = valid ? a.ranges[t] : make_uint2(0u, 0u);
-    const uint32_t cam = valid ? (uint32_t)find_camera(a.cams, a.n_cams, t) : 0u;
+    const uint32_t cam = valid ? (uint32_t)find_camera(a.cams, a.n_cams, a.tile_first + t) : 0u;
     __syncthreads();
     const uint32_t cls = length_class(r.y - r.x);
     const uint32_t rank = count_class(cls, valid, s_class);
@@ -288,7 +292,7 @@ __device__ __forceinline__ void scatter(const BinArgs& a) {
     __syncthreads();
     if (valid) {
       const uint32_t at = s_base[cls] + rank;
-      if (at < a.total_tiles) a.order[at] = tile_work(t, r, cam);
+      if (at < a.total_tiles) a.order[at] = tile_work(a.tile_first + t, r, cam);
     }
     if (blockIdx.x == a.scatter_grid) {
       // tiles with lists above the sort's limits: those of the classes beyond
@@ -314,7 +318,7 @@ __device__ __forceinline__ void scatter(const BinArgs& a) {
         const uint32_t i = c0 + 2 * tid + h;
         e[h] = 2 * tid + h < step && i < count ? vis[i] : make_uint4(0u, 0u, 0u, 0u);
         nt[h] = ((e[h].z >> 16) - (e[h].z & 0xffffu)) * ((e[h].w >> 16) - (e[h].w & 0xffffu));
-        if (kCount && nt[h] <= kBigRect) nt[h] = 0u;   // the projection counted them
+        if (kCount && a.band < 0 && nt[h] <= kBigRect) nt[h] = 0u;   // the projection counted them
       }
       uint32_t total;
       const uint32_t excl = block_excl_scan<kScatterThreads>(nt[0] + nt[1], total, s_warp);
@@ -346,7 +350,7 @@ __device__ __forceinline__ void scatter(const BinArgs& a) {
             const uint32_t w = en.y & 0xffffu;
             const uint32_t local = o - (l ? s_incl[l - 1] : 0u);
             const uint32_t row = rect_row(local, w);
-            const uint32_t tile = en.x + row * (en.y >> 16) + (local - row * w);
+            const uint32_t tile = en.x + row * (en.y >> 16) + (local - row * w) - a.tile_first;
             key[k] = ((uint64_t)en.w << 32) | en.z;
             if (tile < a.total_tiles) {
               if constexpr (kCount) atomicAdd(&a.tile[tile].count, 1u);
@@ -369,7 +373,8 @@ __device__ __forceinline__ void scatter(const BinArgs& a) {
 }
 
 __global__ void __launch_bounds__(kScatterThreads) bin_scatter_kernel(BinArgs a) { scatter<false>(a); }
-// The counts of the rectangles that the projection left (defer_big_rects).
+// The counts of the rectangles that the projection left: large ones
+// (defer_big_rects), or, for a band of a frame, all.
 __global__ void __launch_bounds__(kScatterThreads) bin_count_kernel(BinArgs a) { scatter<true>(a); }
 
 // --------------------------------------------------------------------------

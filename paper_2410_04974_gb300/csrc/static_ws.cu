@@ -15,18 +15,16 @@
 
 namespace {
 
-// Workspace shared by every call of sixdgs_render_fwd_static on a device.  The
-// call's limit counts 8 bytes a tile, the stages keep 56 (range, counters and
-// order record): a frame of the smallest scene and the most tiles that the limit
-// takes (4.19 million) needs 7 times the limit, and one more covers alignment
-// and the scan's words.
-constexpr size_t kArrayBytes = 8 * (size_t)SIXDGS_STATIC_WS_BYTES;
-static __device__ __align__(256) unsigned char g_static_ws[kArrayBytes];
+// Workspace shared by every call of sixdgs_render_fwd_static on a device.
+static __device__ __align__(256) unsigned char g_static_ws[SIXDGS_STATIC_WS_BYTES];
 
 // The size that is held against SIXDGS_STATIC_WS_BYTES: a fixed function of a
 // frame's pairs, duplicates and tiles (about 148.5 bytes a pair and 8 a tile), so
 // that the frames the call takes do not change with what the stages happen to
-// need inside the workspace.
+// need inside the workspace.  The stages keep 56 bytes a tile (range, padded
+// counters, order record): a frame within the limit whose tile state does not fit
+// the array beside its pairs (144 bytes each) is rendered in bands of tiles, at
+// most eight.
 int64_t limit_bytes(const sixdgs_plan& p) {
   int64_t o = 0;
   auto take = [&](int64_t bytes) { o = (o + bytes + 255) / 256 * 256; };
@@ -85,12 +83,18 @@ extern "C" sixdgs_status sixdgs_render_fwd_static(int64_t n, int32_t sh_degree, 
   sixdgs_plan plan;
   sixdgs_status e = sixdgs_plan_init(n, sh_degree, cams, n_cams, &fwd, 0, &plan);
   if (e != SIXDGS_OK) return e;
-  if (limit_bytes(plan) > (int64_t)SIXDGS_STATIC_WS_BYTES || plan.ws_bytes > (int64_t)kArrayBytes)
-    return SIXDGS_ERR_WORKSPACE;
+  if (limit_bytes(plan) > (int64_t)SIXDGS_STATIC_WS_BYTES) return SIXDGS_ERR_WORKSPACE;
+  const size_t bytes = SIXDGS_STATIC_WS_BYTES;
+  int64_t band = 0;
+  if (plan.ws_bytes > (int64_t)bytes) {
+    band = sixdgs::plan_bands(&plan, (int64_t)bytes);
+    if (band <= 0) return SIXDGS_ERR_WORKSPACE;
+  }
   void* ws = nullptr;
   e = static_ws_address(&ws);
   if (e != SIXDGS_OK) return e;
-  const size_t bytes = kArrayBytes;
+  if (band > 0)
+    return sixdgs::render_banded(&plan, band, scene, cams, ws, bytes, images_dev, status_dev, stream);
   e = sixdgs_condition_project(&plan, scene, cams, ws, bytes, status_dev, stream);
   if (e != SIXDGS_OK) return e;
   e = sixdgs_bin_sort(&plan, ws, bytes, status_dev, stream);
