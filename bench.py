@@ -441,11 +441,21 @@ def launches_per_frame(plan, n_cams):
     return (n_cams + 47) // 48 + 1 + 1 + plan.depth_passes + 2 + plan.tile_passes + 1 + 1 + 1 + 1
 
 
-def step_launches(n_cams):
+def step_launches(plan):
     """Kernels of ours one fwd+bwd frame launches: camera upload (one per 48
-    cameras), projection, list scan, scatter and sort, fused blend forward + L1
-    + blend backward, per-Gaussian backward."""
-    return (n_cams + 47) // 48 + 1 + 3 + 1 + 1
+    cameras), projection, the count of large rectangles where few CTAs project
+    many tiles, list scan, scatter and sort, fused blend forward + L1 + blend
+    backward, per-Gaussian backward."""
+    n, V = int(plan.n), int(plan.n_cams)
+    uploads = (V + 47) // 48
+    if n == 0:
+        return uploads + 3 + 1
+    # defer_big_rects of csrc/bin.cuh
+    tiles = -(-n // 128)
+    parts = max(1, min(608 // tiles, V // 2))
+    parts = -(-V // -(-V // parts))
+    count = tiles * parts < 304 and int(plan.total_tiles) > 1024 * V
+    return uploads + 1 + int(count) + 3 + 1 + 1
 
 
 def build_inputs(args):
@@ -618,7 +628,7 @@ def run_ours(args, world, rank, local):
         ms_plain = max_over_ranks(sum(t_plain) / len(t_plain), world)
         rp0 = next(iter(plain_r.values()))
         plain = {"value": V * 1000.0 / ms_plain * world, "unit": UNIT, "ms_per_step": ms_plain,
-                 "launches_per_step": V * step_launches(1), "graph": False}
+                 "launches_per_step": sum(step_launches(plain_r[(c.width, c.height)].plan) for c in cams), "graph": False}
         g_rel = {k: float((grads_p[k] - grads_batched[k]).norm() / grads_batched[k].norm().clamp_min(1e-30))
                  for k in grads_p}
         equiv = {"image_max_abs": float((images - img_batched).abs().max()),
@@ -808,7 +818,7 @@ def run_ours(args, world, rank, local):
         "config": workload_config(w, kw["tile"], world),
         "e2e": e2e, "roofline": roofline, "cpu_baseline": cpu,
         "clocks": {k: clk[k] for k in ("sm_mhz", "sm_max_mhz", "reasons")},
-        "gpu_launches": step_launches(V) * args.steps,
+        "gpu_launches": step_launches(r.plan) * args.steps,
         "megapixels_per_s": round(r.total_pixels * world / (ms_batched * 1e-3) / 1e6, 1),
         "loss": loss_batched,
         "autotuned": None if tuned is None else {k: tuned[k] for k in ("tile", "batch", "persistent", "ms", "cached")},

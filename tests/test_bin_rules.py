@@ -18,7 +18,8 @@ int main() {
     const ViewParts vp = view_parts(n, cams);
     const uint32_t segments = (uint32_t)((n + kStageTile - 1) / kStageTile) * vp.parts;
     const ScatterShare s = scatter_share(segments, (uint32_t)kStageTile * vp.views, (uint32_t)tiles, sms);
-    std::printf("%u %u %u %u %u %u\n", vp.parts, vp.views, segments, s.grid, s.split, s.step);
+    std::printf("%u %u %u %u %u %u %d\n", vp.parts, vp.views, segments, s.grid, s.split, s.step,
+                (int)defer_big_rects(n, cams, tiles));
   }
 }
 """
@@ -42,7 +43,7 @@ def rules(tmp_path_factory):
 def test_a_scatter_step_stays_within_32_bits_and_covers_its_segment(rules):
     frames = [(n, cams, tiles, sms) for n in (1, 127, 129, 5_000, 38_912, 200_000, 3_000_000) for cams in (1, 2, 7, 20, 256)
               for tiles in (1, 2_500, 1 << 20, 1 << 23, (1 << 24) + 3, 1 << 25, (1 << 31) - 1) for sms in (132, 152)]
-    for (n, cams, tiles, sms), (parts, views, segments, grid, split, step) in zip(frames, rules(frames)):
+    for (n, cams, tiles, sms), (parts, views, segments, grid, split, step, _) in zip(frames, rules(frames)):
         assert step >= 1 and step * tiles <= 1 << 31, (n, cams, tiles)     # prefix sums of a step: 32 bits
         size = 128 * views
         assert 1 <= split and 1 <= grid <= min(segments * split, 16 * sms)
@@ -50,3 +51,21 @@ def test_a_scatter_step_stays_within_32_bits_and_covers_its_segment(rules):
         assert split <= -(-size // step)
         # the views of every tile of Gaussians, each once
         assert (parts - 1) * views < cams <= parts * views and segments == -(-n // 128) * parts
+
+
+def test_launch_count_of_a_step_follows_the_rule_for_large_rectangles(rules):
+    import bench
+    import synth
+    from paper_2410_04974_gb300.render import make_plan, make_settings
+
+    frames = [(n, cams, size) for n in (0, 1, 4_000, 17_133, 38_784, 38_785, 300_000) for cams in (1, 2, 3, 8, 20, 64)
+              for size in (128, 512, 513, 1408)]
+    seen = set()
+    for n, cams, size in frames:
+        plan = make_plan(n, 3, synth.ring_cameras(cams, size, size), make_settings())
+        count = n > 0 and bool(rules([(n, cams, int(plan.total_tiles), 152)])[0][6])
+        # upload, projection, count, scan, scatter, sort, fused blend, per-Gaussian backward
+        want = -(-cams // 48) + (n > 0) + count + 3 + 1 + (n > 0)
+        assert bench.step_launches(plan) == want, (n, cams, size)
+        seen.add(count)
+    assert seen == {False, True}

@@ -36,7 +36,7 @@ def test_more_large_rectangles_than_a_cta_lists(rules, n, views, threads):  # no
     scene.l_raw[:3] += np.log(2.0)
     scene.l_raw[:3, ::4] -= np.log(20.0)          # small ones among them
     r = sx.Renderer(n, 1, _cams(views, (400, 272)), tile=(8, 8), lambda_opa=0.0, dup_capacity=32 << 20, inference=True)
-    (parts, per_cta, segments, _, _, _), = rules([(n, views, int(r.plan.total_tiles), 152)])
+    (parts, per_cta, segments, *_), = rules([(n, views, int(r.plan.total_tiles), 152)])
     assert parts == 1 and segments >= FILL // 2 and (per_cta >= WIDE) == (threads == 256)
     r.condition_project(sx.params_to_device(scene))
     r.bin_sort()
@@ -51,7 +51,7 @@ def test_large_rectangles_left_to_their_own_kernel_by_views_divided_among_ctas(r
     scene = synth.scene_cube(n, 5, sh_degree=0)
     r = sx.Renderer(n, 0, _cams(views, (640, 424)), tile=(8, 16), dup_capacity=32 << 20, inference=True)
     tiles = int(r.plan.total_tiles)
-    (parts, per_cta, segments, _, _, _), = rules([(n, views, tiles, 152)])
+    (parts, per_cta, segments, *_), = rules([(n, views, tiles, 152)])
     assert parts > 1 and per_cta == split and segments < FILL // 2 and tiles > 1024 * views
     r.condition_project(sx.params_to_device(scene))
     r.bin_sort()
@@ -71,7 +71,7 @@ def test_staged_projection_with_256_threads_cached_and_not(rules, n, learn):  # 
         scene = synth.with_learnable_lambda(scene, 10)
     cams = _cams(views, (72, 40))
     params = sx.params_to_device(scene)
-    (parts, per_cta, _, _, _, _), = rules([(n, views, 15 * views, 152)])
+    (parts, per_cta, *_), = rules([(n, views, 15 * views, 152)])
     assert parts == 1 and per_cta >= WIDE
     frames = []
     for p in (params, dict(params, cond_cache=sx.condition_cache(params))):
