@@ -9,8 +9,8 @@ render's definition), so the chosen shape is part of the returned settings
 and must be the one any parity check uses.
 
 Results are cached in a JSON file keyed by GPU name, scene size, SH degree,
-camera sizes and the candidate space, so a frame shape is tuned once per
-machine.
+camera sizes, the candidate space, the other render settings and the library's
+sources, so a frame shape is tuned once per machine and version of the kernels.
 """
 
 from __future__ import annotations
@@ -19,6 +19,8 @@ import hashlib
 import json
 import os
 import time
+
+from . import build as _build
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "sixdgs", "autotune.json")
 
@@ -32,10 +34,26 @@ def candidate_space(tiles=((16, 16),), batches=(128, 256, 512, 1024), persistent
     return out
 
 
-def signature(device_name, n, sh_degree, cams, space) -> str:
+def source_digest() -> str:
+    """Digest of the sources that the library is built from (of the library
+    itself where it came without them)."""
+    h = hashlib.sha1()
+    if os.path.isdir(_build.CSRC):
+        paths = sorted(os.path.join(_build.CSRC, f) for f in os.listdir(_build.CSRC))
+        paths.append(os.path.join(_build.INCLUDE, "sixdgs.h"))
+    else:
+        paths = [_build.LIB]
+    for path in paths:
+        if os.path.isfile(path):
+            with open(path, "rb") as f:
+                h.update(os.path.basename(path).encode() + b"\0" + f.read())
+    return h.hexdigest()
+
+
+def signature(device_name, n, sh_degree, cams, space, render_kw=None) -> str:
     sizes = [(int(c.width), int(c.height)) for c in cams]
-    blob = json.dumps({"dev": device_name, "n": int(n), "deg": int(sh_degree), "sizes": sizes,
-                       "space": space}, sort_keys=True)
+    blob = json.dumps({"dev": device_name, "n": int(n), "deg": int(sh_degree), "sizes": sizes, "space": space,
+                       "settings": render_kw or {}, "library": source_digest()}, sort_keys=True, default=str)
     return hashlib.sha1(blob.encode()).hexdigest()
 
 
@@ -92,7 +110,7 @@ def tune(params, n, sh_degree, cams, space=None, cache=DEFAULT_CACHE, force=Fals
     if device_name is None:
         import torch
         device_name = torch.cuda.get_device_name()
-    key = signature(device_name, n, sh_degree, cams, space)
+    key = signature(device_name, n, sh_degree, cams, space, render_kw)
     data = _load(cache) if cache else {}
     if not force and key in data:
         hit = dict(data[key])
