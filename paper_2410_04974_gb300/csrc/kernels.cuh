@@ -128,6 +128,7 @@ struct BlendArgs {
   const CamRec* cams;
   int32_t n_cams;
   int32_t tile_w, tile_h, batch;
+  int32_t short_list;       // set by the launch: lists up to this long are staged by every warp for itself
   const PairRec* rec;
   uint32_t n_pairs;
   const uint32_t* sorted;   // pair index per list entry

@@ -203,6 +203,51 @@ __device__ __forceinline__ void load_batch(const BlendArgs& a, uint32_t start, i
   }
 }
 
+// Sparse frames (below, sparse()): a list of at most a.short_list (32 or fewer)
+// entries is staged by every warp for itself, in places of its own and tested
+// against its own 8x4 sub-block, and walked by the bits of one ballot.  Such a
+// tile is bound by the instructions around its few steps, and waits for the one
+// warp that tests entries against all blocks: no CTA barrier, no ballots and no
+// lists of every block, no padded steps.  2,000 Gaussians of 350 tiles at 4096^2
+// (6.7 entries a tile with a list), against staging by the CTA: forward 208 -> 146
+// us, fused 535 -> 394; tiles of 8x8 pixels 407 -> 204 and 949 -> 521.  (With the
+// walk over the blocks' lists kept, each warp testing its own: forward 220.)
+__host__ __device__ constexpr int short_list(int batch, int warps) {
+  return batch / warps < 32 ? batch / warps : 32;
+}
+// The calling warp's places.
+__device__ __forceinline__ Entry* short_entries(const BlendArgs& a, Entry* s_e) {
+  return s_e + (threadIdx.x >> 5) * a.short_list;
+}
+
+// Stages the short list [range.x, range.y) for the calling warp; returns the
+// entries whose alpha >= 1/255 boxes meet its sub-block, or (kExact, where a
+// backward walk follows) whose ellipses do.
+template <bool kExact>
+__device__ __forceinline__ uint32_t load_short(const BlendArgs& a, uint2 range, float2 npix, Entry* s_e) {
+  const int lane = threadIdx.x & 31;
+  bool reach = false;
+  if (lane < (int)(range.y - range.x)) {
+    const uint32_t p = a.sorted[range.x + lane];
+    Entry& e = short_entries(a, s_e)[lane];
+    if (p < a.n_pairs) {
+      const PairRec& r = a.rec[p];
+      const float4 ra = r.a, rb = r.b, rc = r.c;
+      e.a = ra;
+      e.b = rb;
+      e.c = make_float4(rc.x, rc.y, rc.z, __uint_as_float(p));
+      // first pixel centre of the warp's sub-block
+      const float x0 = -npix.x - (float)((lane >> 4) * kBlkW + (lane & 3)), y0 = -npix.y - (float)((lane >> 2) & 3);
+      reach = kExact ? block_mask<kSubW, 1>(ra, rb, rc, x0, y0) != 0u
+                     : ra.x + rc.y >= x0 && ra.x - rc.y <= x0 + (float)(kSubW - 1) && ra.y + rc.z >= y0 &&
+                           ra.y - rc.z <= y0 + (float)(kSubH - 1);
+    }   // (else unreachable for a consistent sort)
+  }
+  const uint32_t mask = __ballot_sync(0xffffffffu, reach);
+  __syncwarp();
+  return mask;
+}
+
 // The backward walk runs in two passes per warp so that no value has to be
 // summed across the lanes of a warp for every list entry:
 //  1. pixel-parallel (lane = pixel), front to back like the forward: the
@@ -239,18 +284,32 @@ struct __align__(16) WarpScratch {
 // Fills a warp's lists with the batch's entries [c0, c0 + kChunk) (cnt in the
 // batch); returns the number of steps of the longer one, a multiple of kStep.
 // cull: the ballots of the warp's left block (its right one's follow).
+// twin (may be null): whether the two blocks reach nearly the same entries; then
+// both lists get the entries of either (which change nothing at the other block).
 __device__ __forceinline__ int fill_lists(const uint32_t* cull, int batch, int c0, int cnt, WalkLists& lists,
-                                          uint32_t* n_warp = nullptr) {
+                                          uint32_t* n_warp = nullptr, bool* twin = nullptr) {
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
   uint32_t n0 = 0u, n1 = 0u;
   __syncwarp();   // the lists are no longer read
   cull += c0 >> 5;
+  if (twin) {
+    uint32_t both = 0u, either = 0u;
+#pragma unroll
+    for (int g = 0; g < kChunk / 32; ++g)
+      if (c0 + 32 * g < cnt) {
+        const uint32_t m0 = cull[g], m1 = cull[cull_stride(batch) + g];
+        both += __popc(m0 & m1);
+        either += __popc(m0 | m1);
+      }
+    *twin = 16u * (either - both) <= either;
+  }
 #pragma unroll
   for (int g = 0; g < kChunk / 32; ++g) {
     const int base = c0 + 32 * g;
     if (base < cnt) {
-      const uint32_t m0 = cull[g], m1 = cull[cull_stride(batch) + g];
+      uint32_t m0 = cull[g], m1 = cull[cull_stride(batch) + g];
+      if (twin && *twin) m0 = m1 = m0 | m1;
       const uint16_t off = (uint16_t)((base + lane) * (int)sizeof(Entry));
       if ((m0 >> lane) & 1u) lists.off[0][n0 + __popc(m0 & below)] = off;
       if ((m1 >> lane) & 1u) lists.off[1][n1 + __popc(m1 & below)] = off;
@@ -347,6 +406,35 @@ __device__ __forceinline__ FwdPixel fwd_walk(const BlendArgs& a, float2 npix, ui
   return FwdPixel{T, C01.x, C01.y, C2, walked, staged};
 }
 
+// The same for a short list, whose entries in `mask` the warp takes one by one.
+__device__ __forceinline__ FwdPixel fwd_walk_short(const BlendArgs& a, float2 npix, uint2 range, bool inside,
+                                                   Entry* s_e, uint32_t mask) {
+  float T = 1.f, C2 = 0.f;
+  float2 C01 = make_float2(0.f, 0.f);
+  uint32_t walked = range.y - range.x;
+  bool done = !inside;
+  const Entry* e = short_entries(a, s_e);
+  while (mask) {
+    const int j = __ffs(mask) - 1;
+    mask &= mask - 1u;
+    const float4 ra = e[j].a, rb = e[j].b;
+    const float blue = e[j].c.x;
+    float2 d;
+    const float q = entry_q(ra, rb, npix, d);
+    const bool vis = !done && q >= kQMin;
+    const float alpha = vis ? fminf(kAlphaMax, ex2_approx(q)) : 0.f;
+    const float2 tw = __fmul2_rn(make_float2(T, T), make_float2(__fsub_rn(1.f, alpha), alpha));
+    const bool stop = tw.x < kTMin;
+    const float w = stop ? 0.f : tw.y;
+    C01 = __ffma2_rn(make_float2(rb.z, rb.w), make_float2(w, w), C01);
+    C2 = __fmaf_rn(blue, w, C2);
+    T = stop ? T : tw.x;
+    if (stop) walked = (uint32_t)j;
+    done = done || stop;
+  }
+  return FwdPixel{T, C01.x, C01.y, C2, walked, true};
+}
+
 // Sum over the 32 pixels of a sub-block, rows first, then columns from the
 // outermost bit in (an order that does not depend on how the pixels are dealt
 // to the lanes; lane bits: half, row, row, column, column).
@@ -357,7 +445,7 @@ __device__ __forceinline__ float sub_block_sum(float v) {
 }
 
 // Forward blend of tile tw (tile_work) by the calling CTA.
-template <bool kCount, bool kStore>
+template <bool kCount, bool kStore, bool kShort>
 __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
   Entry* s_e = reinterpret_cast<Entry*>(s_mem);
   WalkLists* lists = reinterpret_cast<WalkLists*>(scratch_of(a, s_mem));
@@ -372,8 +460,9 @@ __device__ __forceinline__ void blend_fwd_tile(const BlendArgs& a, uint4 tw, flo
   const int lane = threadIdx.x & 31;
 
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
-  const FwdPixel fp =
-      fwd_walk<kCount>(a, npix, range, inside, s_e, lists[threadIdx.x >> 5], n_eval, n_comp, n_warp);
+  FwdPixel fp;
+  if constexpr (kShort) fp = fwd_walk_short(a, npix, range, inside, s_e, load_short<false>(a, range, npix, s_e));
+  else fp = fwd_walk<kCount>(a, npix, range, inside, s_e, lists[threadIdx.x >> 5], n_eval, n_comp, n_warp);
   float T = fp.T, C0 = fp.C0, C1 = fp.C1, C2 = fp.C2;
   const uint32_t walked = fp.walked;
 
@@ -435,8 +524,11 @@ __device__ __forceinline__ void red_add4(float* addr, float x, float y, float z,
 }
 
 // Pass 2 over slots [0, k) of both halves.  null_off: offset of the null entry.
+// twin (kTwins): both halves' slots hold the same entries, whose sums are added
+// before they go to global memory.
+template <bool kTwins>
 __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws, int k, const Entry* s_e, float2 npix,
-                                            uint32_t null_off) {
+                                            uint32_t null_off, bool twin) {
   static_assert(kSlots == 8 && kBlkW == 4 && kSubH == 4, "two rows of a block per lane");
   __syncwarp();
   const int lane = threadIdx.x & 31;
@@ -473,7 +565,9 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
 #pragma unroll
   for (int q = 0; q < 9; ++q) m[q] += __shfl_xor_sync(0xffffffffu, m[q], kSlots);
   const uint32_t off = reinterpret_cast<const uint16_t*>(ws.slot[h])[s];
-  if (r == 0 && s < k && off != null_off) {
+  const bool mine = r == 0 && s < k && off != null_off;
+  const uint32_t lanes = kTwins ? __ballot_sync(0xffffffffu, mine) : 0u;
+  if (mine) {
     const Entry& en = entry_at(s_e, off);
     // dx = U - c, dy = V - r; the block's centre from this lane's pixel
     const float U = en.a.x + (npix.x + ((float)(lane & 3) - 0.5f * (float)(kBlkW - 1)));
@@ -488,11 +582,17 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
     g[6] = m[6];
     g[7] = m[7];
     g[8] = m[8];
-    float* dst = a.grad_rec + (size_t)__float_as_uint(en.c.w) * 12;
-    // a record is 48 bytes, 16-byte aligned: floats 0-3 and 4-7 as vectors
-    red_add4(dst, g[0], g[1], g[2], g[3]);
-    red_add4(dst + 4, g[4], g[5], g[6], g[7]);
-    if (g[8] != 0.f) red_add(dst + 8, g[8]);
+    if (kTwins && twin) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) g[q] += __shfl_xor_sync(lanes, g[q], 16);
+    }
+    if (!(kTwins && twin) || h == 0) {
+      float* dst = a.grad_rec + (size_t)__float_as_uint(en.c.w) * 12;
+      // a record is 48 bytes, 16-byte aligned: floats 0-3 and 4-7 as vectors
+      red_add4(dst, g[0], g[1], g[2], g[3]);
+      red_add4(dst + 4, g[4], g[5], g[6], g[7]);
+      if (g[8] != 0.f) red_add(dst + 8, g[8]);
+    }
   }
   __syncwarp();
 }
@@ -502,7 +602,13 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
 // kRecompute: re-derive the stop from the transmittance; otherwise the pixel
 // walks `bound` entries.  staged (CTA-uniform): the whole list is already in
 // shared memory (a single batch that the forward of the same CTA staged).
-template <bool kRecompute>
+// kTwins: where a warp's two blocks reach nearly the same entries, they walk the
+// same list and their sums go to global memory together.  In frames of few
+// Gaussians over many tiles every record takes the sums of thousands of blocks,
+// and the reductions to a few records are what bounds the kernel (1,000 Gaussians
+// of 5,600 tiles at 1408^2: blend_bwd 1,117 -> 611 us, fused 1,135 -> 812).  Only
+// in the kernels for sparse frames: elsewhere blocks are seldom twins.
+template <bool kRecompute, bool kTwins>
 __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 range, bool inside, const float* Cf,
                                          const float* dC, uint32_t bound, bool staged, Entry* s_e, WarpScratch& ws) {
   const int B = a.batch;
@@ -520,6 +626,7 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
   // (dC0, dC1, 1, dC2): pass 2 pairs the 1 with dq and dC2 with w
   ws.pix[lane + (lane >> 3)] = make_float4(dC[0], dC[1], 1.f, dC[2]);
   int k0 = 0;         // slots filled (warp-uniform, a multiple of kStep)
+  bool twin = false;  // both halves' slots hold the same entries
 
   for (uint32_t start = range.x; start < range.y; start += B) {
     // a staged list is already in shared memory (read-only): no CTA barrier
@@ -533,7 +640,13 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
     // entries at offsets below lim of this batch lie within the pixel's walk
     const uint32_t lim = min((uint32_t)cnt, bound - min(bound, start - range.x)) * (uint32_t)sizeof(Entry);
     for (int c0 = 0; c0 < cnt; c0 += kChunk) {
-      const int steps = fill_lists(warp_cull(a, s_e), B, c0, cnt, ws.lists);
+      bool same = false;
+      const int steps = fill_lists(warp_cull(a, s_e), B, c0, cnt, ws.lists, nullptr, kTwins ? &same : nullptr);
+      if (kTwins && same != twin) {
+        if (k0) flush_slots<kTwins>(a, ws, k0, s_e, npix, null_off, twin);
+        k0 = 0;
+        twin = same;
+      }
       bool all = false;
 #pragma unroll 1
       for (int i = 0; i < steps && !all; i += kStep) {
@@ -580,7 +693,7 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
         for (int k = 0; k < kStep; ++k) slot[k * 33] = res[k];
         k0 += kStep;
         if (k0 == kSlots) {
-          flush_slots(a, ws, kSlots, s_e, npix, null_off);
+          flush_slots<kTwins>(a, ws, kSlots, s_e, npix, null_off, twin);
           k0 = 0;
         }
         // (a padded list says nothing about the walk's end)
@@ -591,16 +704,60 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
     }
     if (!kRecompute) done = done || start - range.x + cnt >= bound;
     if (k0) {   // the slots refer to this batch's shared-memory records
-      flush_slots(a, ws, k0, s_e, npix, null_off);
+      flush_slots<kTwins>(a, ws, k0, s_e, npix, null_off, twin);
       k0 = 0;
     }
   }
 }
 
+// The same for a short list, whose entries in `mask` the warp takes one by one,
+// both of its blocks the same.
+template <bool kRecompute>
+__device__ __forceinline__ void bwd_walk_short(const BlendArgs& a, float2 npix, bool inside, const float* Cf,
+                                               const float* dC, uint32_t bound, uint32_t mask, Entry* s_e,
+                                               WarpScratch& ws) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t first = (uint32_t)(short_entries(a, s_e) - s_e) * (uint32_t)sizeof(Entry);
+  const float D0 = dC[0] * Cf[0] + dC[1] * Cf[1] + dC[2] * Cf[2];
+  float T = 1.f, Q = 0.f;
+  if (kRecompute || !inside) bound = inside ? 0xffffffffu : 0u;
+  ws.pix[lane + (lane >> 3)] = make_float4(dC[0], dC[1], 1.f, dC[2]);
+  int k = 0;   // slots filled
+  while (mask) {
+    const uint32_t j = (uint32_t)__ffs(mask) - 1u, off = first + j * (uint32_t)sizeof(Entry);
+    mask &= mask - 1u;
+    const Entry& en = entry_at(s_e, off);
+    const float4 ra = en.a, rb = en.b;
+    const float blue = en.c.x;
+    float2 d;
+    const float q = entry_q(ra, rb, npix, d);
+    const bool vis = j < bound && q >= kQMin;
+    const float e = ex2_approx(q);
+    const float alpha = vis ? fminf(kAlphaMax, e) : 0.f;
+    const float om = __fsub_rn(1.f, alpha);
+    const float2 tw = __fmul2_rn(make_float2(T, T), make_float2(om, alpha));
+    const bool stop = kRecompute && tw.x < kTMin;
+    const float w = stop ? 0.f : tw.y;
+    const float G = dC[0] * rb.z + dC[1] * rb.w + dC[2] * blue;
+    Q = fmaf(w, G, Q);
+    const float dLda = T * G - (D0 - Q) * rcp_approx(om);
+    const float dq = (!stop && e <= kAlphaMax) ? dLda * alpha : 0.f;
+    T = stop ? T : tw.x;
+    if (stop) bound = 0u;
+    ws.dqw[k][lane] = make_float2(dq, w);
+    if ((lane & 15) == 0) reinterpret_cast<uint16_t*>(ws.slot[lane >> 4])[k] = (uint16_t)off;
+    if (++k == kSlots) {
+      flush_slots<true>(a, ws, kSlots, s_e, npix, 0xffffffffu, true);
+      k = 0;
+    }
+  }
+  if (k) flush_slots<true>(a, ws, k, s_e, npix, 0xffffffffu, true);
+}
+
 // Backward blend of tile tw by the calling CTA.  kRecompute: re-derive
 // the stop from the transmittance (no per-pixel state); otherwise walk each
 // pixel's stored number of entries.
-template <bool kRecompute>
+template <bool kRecompute, bool kShort, bool kShorts>
 __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
   const CamRec& cam = a.cams[tw.w];
   const uint32_t local = tw.x - (uint32_t)cam.tile_offset;
@@ -624,8 +781,13 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint4 tw, flo
     if (!kRecompute) bound = a.nwalk[cam.pixel_base + pix];
   }
   WarpScratch* ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem));
-  bwd_walk<kRecompute>(a, npix, range, inside, Cf, dC, bound, false, reinterpret_cast<Entry*>(s_mem),
-                       ws[threadIdx.x >> 5]);
+  Entry* s_e = reinterpret_cast<Entry*>(s_mem);
+  if constexpr (kShort) {
+    const uint32_t mask = load_short<true>(a, range, npix, s_e);
+    bwd_walk_short<kRecompute>(a, npix, inside, Cf, dC, bound, mask, s_e, ws[threadIdx.x >> 5]);
+  } else {
+    bwd_walk<kRecompute, kShorts>(a, npix, range, inside, Cf, dC, bound, false, s_e, ws[threadIdx.x >> 5]);
+  }
 }
 
 // Forward blend, fused L1 loss and backward blend of tile tw by the calling
@@ -640,6 +802,7 @@ __device__ __forceinline__ void blend_bwd_tile(const BlendArgs& a, uint4 tw, flo
 // dL/dC, loss and record gradients equal those of raster_fwd followed by
 // blend_bwd in stored-walk mode, bit for bit up to the order of the atomic
 // additions.
+template <bool kShort, bool kShorts>
 __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, float4* s_mem) {
   Entry* s_e = reinterpret_cast<Entry*>(s_mem);
   __shared__ float s_red[16];
@@ -654,8 +817,14 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, f
 
   WarpScratch& ws = reinterpret_cast<WarpScratch*>(scratch_of(a, s_mem))[threadIdx.x >> 5];
   uint32_t n_eval = 0, n_comp = 0, n_warp = 0;
-  const FwdPixel fp =
-      fwd_walk<false>(a, npix, range, inside, s_e, ws.lists, n_eval, n_comp, n_warp);
+  FwdPixel fp;
+  uint32_t mask = 0u;
+  if constexpr (kShort) {
+    mask = load_short<true>(a, range, npix, s_e);
+    fp = fwd_walk_short(a, npix, range, inside, s_e, mask);
+  } else {
+    fp = fwd_walk<false>(a, npix, range, inside, s_e, ws.lists, n_eval, n_comp, n_warp);
+  }
   float Cf[3] = {0.f, 0.f, 0.f}, dC[3] = {0.f, 0.f, 0.f};
   float l1 = 0.f;
   if (inside) {
@@ -683,7 +852,8 @@ __device__ __forceinline__ void blend_fused_tile(const BlendArgs& a, uint4 tw, f
   l1 = sub_block_sum(l1);
   if (lane == 0) s_red[threadIdx.x >> 5] = l1;
   __syncwarp();
-  bwd_walk<false>(a, npix, range, inside, Cf, dC, fp.walked, fp.staged, s_e, ws);
+  if constexpr (kShort) bwd_walk_short<false>(a, npix, inside, Cf, dC, fp.walked, mask, s_e, ws);
+  else bwd_walk<false, kShorts>(a, npix, range, inside, Cf, dC, fp.walked, fp.staged, s_e, ws);
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
@@ -746,6 +916,11 @@ __device__ __forceinline__ void blend_empty(const BlendArgs& a, uint32_t first) 
   }
 }
 
+template <bool kValue>
+struct Bool {
+  static constexpr bool value = kValue;
+};
+
 // Work unit u of a blend launch.  Tiles are taken in the binning's order,
 // longest lists first, so that the launch does not end on a few CTAs that
 // started a long list late (917 -> 858 us for the fused kernel at 300k / 8 x
@@ -755,12 +930,20 @@ __device__ __forceinline__ void blend_empty(const BlendArgs& a, uint32_t first) 
 // that, the one-load tile record and the asynchronous staging of a batch
 // (load_batch): fused kernel 722 -> 663 us at 300k / 8 x 800^2, forward 600 ->
 // 536 us for 20 views of 183k Gaussians at 1024^2.
-template <typename Tile, typename Empty>
+// tile(tw, short): a tile with a list, which is a short one or not.
+template <bool kShorts, typename Tile, typename Empty>
 __device__ __forceinline__ bool blend_unit(const BlendArgs& a, uint32_t u, Tile tile, Empty empty) {
   const uint4 tw = a.order[min(u, a.total_tiles - 1)];
   const uint32_t busy = min(*a.n_busy, a.total_tiles);
   if (u < busy) {
-    if (tw.x - a.tile_first < a.total_tiles) tile(tw);
+    if (tw.x - a.tile_first < a.total_tiles) {
+      if constexpr (kShorts) {
+        if (tw.z - tw.y > (uint32_t)a.short_list) tile(tw, Bool<false>{});
+        else tile(tw, Bool<true>{});
+      } else {
+        tile(tw, Bool<false>{});
+      }
+    }
     return true;
   }
   const uint32_t first = busy + (u - busy) * (blockDim.x / 32);
@@ -769,11 +952,11 @@ __device__ __forceinline__ bool blend_unit(const BlendArgs& a, uint32_t u, Tile 
   return true;
 }
 
-template <typename Tile, typename Empty>
+template <bool kShorts, typename Tile, typename Empty>
 __device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile tile, Empty empty) {
   after_previous();
   if (!a.tile_queue) {
-    blend_unit(a, blockIdx.x, tile, empty);
+    blend_unit<kShorts>(a, blockIdx.x, tile, empty);
     return;
   }
   __shared__ uint32_t s_next;
@@ -781,15 +964,16 @@ __device__ __forceinline__ void for_each_blend_tile(const BlendArgs& a, Tile til
     if (threadIdx.x == 0) s_next = atomicAdd(a.tile_queue, 1u);
     __syncthreads();
     const uint32_t next = s_next;
-    if (!blend_unit(a, next, tile, empty)) break;
+    if (!blend_unit<kShorts>(a, next, tile, empty)) break;
     __syncthreads();
   }
 }
 
+template <bool kShorts>
 __global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  for_each_blend_tile(
-      a, [&](uint4 tw) { blend_fused_tile(a, tw, s_mem); },
+  for_each_blend_tile<kShorts>(
+      a, [&](uint4 tw, auto s) { blend_fused_tile<decltype(s)::value, kShorts>(a, tw, s_mem); },
       [&](uint32_t first) {
         if (a.nwalk) blend_empty<true>(a, first);
         else blend_empty<false>(a, first);
@@ -799,7 +983,7 @@ __global__ void __maxnreg__(SIXDGS_FUSED_MAXNREG) blend_fused_kernel(BlendArgs a
 // One CTA per tile (grid = tiles), or persistent: a grid of as many CTAs as
 // fit on the GPU at once, each taking tiles from a device counter until all
 // cameras' tiles are done.
-template <bool kCount, bool kStore>
+template <bool kCount, bool kStore, bool kShorts>
 // (the forward's registers: 64 / 48 / 40 give 617 / 599 / 606 us for 20 views of
 // 183k Gaussians at 1024^2)
 #ifndef SIXDGS_FWD_MAXNREG
@@ -807,16 +991,16 @@ template <bool kCount, bool kStore>
 #endif
 __global__ void __maxnreg__(SIXDGS_FWD_MAXNREG) blend_fwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  for_each_blend_tile(
-      a, [&](uint4 tw) { blend_fwd_tile<kCount, kStore>(a, tw, s_mem); },
+  for_each_blend_tile<kShorts>(
+      a, [&](uint4 tw, auto s) { blend_fwd_tile<kCount, kStore, decltype(s)::value>(a, tw, s_mem); },
       [&](uint32_t first) { blend_empty<kStore>(a, first); });
 }
 
-template <bool kRecompute>
+template <bool kRecompute, bool kShorts>
 __global__ void __maxnreg__(SIXDGS_BWD_MAXNREG) blend_bwd_kernel(BlendArgs a) {
   extern __shared__ float4 s_mem[];
-  for_each_blend_tile(
-      a, [&](uint4 tw) { blend_bwd_tile<kRecompute>(a, tw, s_mem); }, [](uint32_t) {});
+  for_each_blend_tile<kShorts>(
+      a, [&](uint4 tw, auto s) { blend_bwd_tile<kRecompute, decltype(s)::value, kShorts>(a, tw, s_mem); }, [](uint32_t) {});
 }
 
 // Batches near or above 48 KB of shared memory (with the kernels' static
@@ -835,10 +1019,25 @@ static int resident_grid(const void* fn, int threads, int smem, int64_t tiles) {
   return (int)std::min<int64_t>(g, tiles);
 }
 
+// Frames with fewer (view, Gaussian) pairs a tile than this, whose lists are
+// short or their records few, take kernels compiled with the two paths for them
+// (kShorts); the other kernels are compiled without, as the paths cost registers
+// (fused 652 instead of 648 us at 300k / 8 x 800^2).  With / without them, fused and
+// forward us: 2.4 pairs a tile (4 views of 10,000 volume Gaussians at 1024^2) 136 /
+// 146 and 53 / 57; 4.9: 153 / 161 and 59 / 64; 7.7 (60,000 of a shell at 1408^2):
+// 70.3 / 70.6 and 28.6 / 30.7; 15.5: 93.8 / 92.8 and 38.9 / 38.9; 24: 240 / 241 and
+// 90 / 92; 52: 213 / 211 and 80 / 80.
+constexpr uint32_t kSparsePairs = 8;
+static bool sparse(const BlendArgs& a) { return a.n_pairs / kSparsePairs < a.total_tiles; }
+
 // scratch: the backward walk's per-warp shared memory (the forward: lists only)
 template <typename K>
-static void launch_blend(K kernel, const BlendArgs& a, int64_t total_tiles, bool scratch, cudaStream_t stream) {
+static void launch_blend(K kernel, BlendArgs a, int64_t total_tiles, bool scratch, cudaStream_t stream) {
   const int threads = a.tile_w * a.tile_h;
+  // two warps a CTA: the staging area bounds the CTAs per SM (8 at a batch of 512),
+  // and short lists need little of it
+  if (threads == 64 && sparse(a)) a.batch = std::min(a.batch, 256);
+  a.short_list = short_list(a.batch, threads / 32);
   const int smem = stage_bytes(a.batch, threads / (kBlkW * kSubH)) + threads / 32 * (int)(scratch ? sizeof(WarpScratch) : sizeof(WalkLists));
   allow_smem((const void*)kernel, smem);
   if (a.tile_queue) {
@@ -852,24 +1051,33 @@ static void launch_blend(K kernel, const BlendArgs& a, int64_t total_tiles, bool
 
 void launch_blend_fwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream) {
   if (total_tiles == 0) return;
-  if (a.pair_counts) {
-    if (a.nwalk) launch_blend(blend_fwd_kernel<true, true>, a, total_tiles, false, stream);
-    else launch_blend(blend_fwd_kernel<true, false>, a, total_tiles, false, stream);
+  if (a.pair_counts) {   // counts the general walk's pairs in any frame
+    if (a.nwalk) launch_blend(blend_fwd_kernel<true, true, false>, a, total_tiles, false, stream);
+    else launch_blend(blend_fwd_kernel<true, false, false>, a, total_tiles, false, stream);
+  } else if (sparse(a)) {
+    if (a.nwalk) launch_blend(blend_fwd_kernel<false, true, true>, a, total_tiles, false, stream);
+    else launch_blend(blend_fwd_kernel<false, false, true>, a, total_tiles, false, stream);
   } else {
-    if (a.nwalk) launch_blend(blend_fwd_kernel<false, true>, a, total_tiles, false, stream);
-    else launch_blend(blend_fwd_kernel<false, false>, a, total_tiles, false, stream);
+    if (a.nwalk) launch_blend(blend_fwd_kernel<false, true, false>, a, total_tiles, false, stream);
+    else launch_blend(blend_fwd_kernel<false, false, false>, a, total_tiles, false, stream);
   }
 }
 
 void launch_blend_fused(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream) {
   if (total_tiles == 0) return;
-  launch_blend(blend_fused_kernel, a, total_tiles, true, stream);
+  if (sparse(a)) launch_blend(blend_fused_kernel<true>, a, total_tiles, true, stream);
+  else launch_blend(blend_fused_kernel<false>, a, total_tiles, true, stream);
 }
 
 void launch_blend_bwd(const BlendArgs& a, int64_t total_tiles, cudaStream_t stream) {
   if (total_tiles == 0) return;
-  if (a.recompute) launch_blend(blend_bwd_kernel<true>, a, total_tiles, true, stream);
-  else launch_blend(blend_bwd_kernel<false>, a, total_tiles, true, stream);
+  if (sparse(a)) {
+    if (a.recompute) launch_blend(blend_bwd_kernel<true, true>, a, total_tiles, true, stream);
+    else launch_blend(blend_bwd_kernel<false, true>, a, total_tiles, true, stream);
+  } else {
+    if (a.recompute) launch_blend(blend_bwd_kernel<true, false>, a, total_tiles, true, stream);
+    else launch_blend(blend_bwd_kernel<false, false>, a, total_tiles, true, stream);
+  }
 }
 
 }  // namespace sixdgs
