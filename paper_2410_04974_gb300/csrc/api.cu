@@ -267,15 +267,16 @@ sixdgs_status project_frame(const sixdgs_plan* p, const sixdgs_scene* scene, con
   a.depth_key = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_DEPTHKEY);
   a.vis = ws_ptr<uint4>(ws, p, WS_VIS);
   a.vis_count = ws_ptr<uint32_t>(ws, p, WS_VIS_COUNT);
-  a.tile = banded ? nullptr : ws_ptr<TileCounters>(ws, p, WS_TILE);
+  a.tile = ws_ptr<TileCounters>(ws, p, WS_TILE);
+  a.banded = banded;
   a.grad_rec = p->settings.inference ? nullptr : ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
   a.bulk = bulk_planes(p->n, {a.mu_p, a.mu_d, a.sh, a.lambda_raw, a.cond_cache,
                               a.cond_cache ? nullptr : a.l_raw, a.cond_cache ? nullptr : a.opacity_logit});
   a.spin_budget = spin_budget(p);
   a.status = status_dev;
-  a.defer_big = !banded && defer_big_rects(p->n, p->n_cams, p->total_tiles);
+  a.defer_big = defer_big_rects(p->n, p->n_cams, p->total_tiles);
   launch_project_fwd(a, stream);
-  if (a.defer_big && p->n > 0 &&
+  if (a.defer_big && !banded && p->n > 0 &&
       launch_bin_count(bin_args(p, ws, status_dev), sm_count(), stream) != cudaSuccess)
     return SIXDGS_ERR_CUDA;
   return launch_status();
@@ -304,7 +305,7 @@ BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
                       ? reinterpret_cast<unsigned long long*>(ws_ptr<char>(ws, p, SIXDGS_WS_COUNTS) + 16)
                       : nullptr;
   a.tile_queue = p->settings.persistent ? ws_ptr<uint32_t>(ws, p, WS_COUNTERS) + 32 : nullptr;
-  a.total_tiles = (uint32_t)p->total_tiles;
+  a.total_tiles = a.frame_tiles = (uint32_t)p->total_tiles;
   a.spin_budget = spin_budget(p);
   return a;
 }
@@ -336,7 +337,7 @@ sixdgs_status render_banded(const sixdgs_plan* p, int64_t slots, const sixdgs_sc
   f.status = status_dev;
   b.band = 0;
   for (int64_t first = 0; first < p->total_tiles; first += slots, ++b.band) {
-    b.tile_first = f.tile_first = (uint32_t)first;
+    b.tile_first = (uint32_t)first;
     b.total_tiles = f.total_tiles = (uint32_t)std::min(slots, p->total_tiles - first);
     if (first > 0 && cudaMemsetAsync(b.tile, 0, b.total_tiles * sizeof(TileCounters), stream) != cudaSuccess)
       return SIXDGS_ERR_CUDA;

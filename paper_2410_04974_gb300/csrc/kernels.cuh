@@ -72,8 +72,9 @@ struct ProjectArgs {
   uint4* vis;             // visible queue of the binning (bin.cuh)
   uint32_t* vis_count;
   ViewParts views;        // set by the launch
-  bool defer_big;         // leaves the rectangles of many tiles to bin_count_kernel
-  TileCounters* tile;     // their counts are added to; null: bin_count_kernel counts
+  bool banded;            // leaves all rectangles to bin_count_kernel
+  bool defer_big;         // leaves those of many tiles
+  TileCounters* tile;     // their counts are added to
   float* grad_rec;   // zeroed for every visible pair (read by the backward); null: inference plan
   int32_t bulk;      // 1: every parameter plane segment can be staged with bulk copies
   int64_t spin_budget;
@@ -135,7 +136,6 @@ struct BlendArgs {
   const uint2* ranges;
   const uint4* order;       // TileWork of every tile, longest lists first
   const uint32_t* n_busy;   // tiles with a list (the others come last)
-  uint32_t tile_first;      // first tile of the band (kernels.cuh, BinArgs)
   float bg[3];
   float* images;
   const float* targets;
@@ -151,7 +151,8 @@ struct BlendArgs {
   int32_t recompute;        // 1: re-derive the stop; 0: use nwalk
   // persistent mode: tiles are taken from this counter (NULL: one CTA per tile)
   uint32_t* tile_queue;
-  uint32_t total_tiles;
+  uint32_t total_tiles;     // of the band (BinArgs)
+  uint32_t frame_tiles;     // of the frame
   int64_t spin_budget;      // clock cycles a shared-memory ring wait may take
   int32_t* status;
 };

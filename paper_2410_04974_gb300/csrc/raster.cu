@@ -936,7 +936,7 @@ __device__ __forceinline__ bool blend_unit(const BlendArgs& a, uint32_t u, Tile 
   const uint4 tw = a.order[min(u, a.total_tiles - 1)];
   const uint32_t busy = min(*a.n_busy, a.total_tiles);
   if (u < busy) {
-    if (tw.x - a.tile_first < a.total_tiles) {
+    if (tw.x < (kShorts ? a.frame_tiles : a.total_tiles)) {
       if constexpr (kShorts) {
         if (tw.z - tw.y > (uint32_t)a.short_list) tile(tw, Bool<false>{});
         else tile(tw, Bool<true>{});
@@ -1028,7 +1028,9 @@ static int resident_grid(const void* fn, int threads, int smem, int64_t tiles) {
 // 70.3 / 70.6 and 28.6 / 30.7; 15.5: 93.8 / 92.8 and 38.9 / 38.9; 24: 240 / 241 and
 // 90 / 92; 52: 213 / 211 and 80 / 80.
 constexpr uint32_t kSparsePairs = 8;
-static bool sparse(const BlendArgs& a) { return a.n_pairs / kSparsePairs < a.total_tiles; }
+static bool sparse(const BlendArgs& a) {
+  return a.n_pairs / kSparsePairs < a.total_tiles || a.total_tiles != a.frame_tiles;   // (a band of a frame: always)
+}
 
 // scratch: the backward walk's per-warp shared memory (the forward: lists only)
 template <typename K>

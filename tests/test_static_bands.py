@@ -34,6 +34,7 @@ def test_the_library_holds_no_more_than_the_stated_array():
 @pytest.mark.parametrize("n,log_scale,sizes,bands,status", [
     (150_000, -4.5, [(8192, 8192)], 5, 0),            # 1.05 million tiles
     (700, -5.0, [(4100, 3000), (2051, 4099), (64, 40), (8000, 6001)], 2, 0),      # bands that cross views
+    (12_001, -4.5, [(2000, 1777)] * 10, 2, 0),        # views divided among the projection's CTAs
     (40, -5.5, [(16_000, 13_000)], 6, 0),             # 3.25 million tiles, almost all empty
     (40, 0.0, [(16_000, 13_000)], 6, 1 << _lib.ERR_CAPACITY),
 ])
