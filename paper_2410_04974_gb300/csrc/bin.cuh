@@ -66,7 +66,10 @@ __host__ __device__ inline ScatterShare scatter_share(uint32_t segments, uint32_
   // 16 CTAs per SM: with fewer segments, several CTAs take the steps of one in
   // turn (the binning of 20 views of 6,660 Gaussians at 1408^2, 1.1 M duplicates
   // in 53 segments before: 152 -> 78 us; of 4 views 43 -> 29 us, with the
-  // projection's division of the views)
+  // projection's division of the views); a frame of fewer pairs than CTAs gives
+  // every CTA one, which may have tens of thousands of tiles (count and binning of
+  // 1,000 Gaussians of 22,000 tiles of 8x8 pixels at 1408^2 517 -> 346 us against
+  // two a CTA, of 5,600 of 16x16 166 -> 124)
   const uint32_t most_ctas = (uint32_t)sms * 16u;
   // a step's duplicates are counted in 32 bits: at most 2^31 of them
   uint32_t most_step = total_tiles ? (1u << 31) / total_tiles : kScatterEntries;
@@ -74,7 +77,8 @@ __host__ __device__ inline ScatterShare scatter_share(uint32_t segments, uint32_
   if (most_step < 1u) most_step = 1u;
   ScatterShare s = {0u, 1u, most_step};
   if (segments && 2u * segments <= most_ctas) {
-    const uint32_t share = (segment_size * segments + most_ctas - 1) / most_ctas, step = (share + 1u) & ~1u;
+    const uint32_t share = (segment_size * segments + most_ctas - 1) / most_ctas;
+    const uint32_t step = share > 1u ? (share + 1u) & ~1u : 1u;
     if (step < s.step) s.step = step;
     const uint32_t steps = (segment_size + s.step - 1) / s.step, ctas = most_ctas / segments;
     s.split = ctas < steps ? ctas : steps;
