@@ -131,7 +131,9 @@ typedef struct sixdgs_settings {
                           (no per-pixel auxiliary buffer)                     */
   int64_t spin_budget; /* clock cycles a device-side wait may spin before it
                           reports SIXDGS_ERR_TIMEOUT; <= 0 selects the default
-                          (2^31 cycles, about one second)                     */
+                          (2^31 cycles, about one second).  A wait for a copy
+                          in flight is extended once, by 2^24 cycles or more,
+                          and reported only if the copy has not come by then  */
   float loss_norm;     /* number of values the fused L1 mean divides by; <= 0
                           selects 3 * total_pixels of the plan (use the whole
                           batch's count when one batch is rendered one camera

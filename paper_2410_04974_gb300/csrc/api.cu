@@ -293,7 +293,6 @@ BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
   a.rec = ws_ptr<PairRec>(ws, p, SIXDGS_WS_REC);
   a.n_pairs = (uint32_t)p->n_pairs;
   a.sorted = ws_ptr<uint32_t>(ws, p, SIXDGS_WS_SORTED);
-  a.ranges = ws_ptr<uint2>(ws, p, SIXDGS_WS_RANGES);
   a.order = ws_ptr<uint4>(ws, p, WS_ORDER);
   a.n_busy = ws_ptr<uint32_t>(ws, p, WS_STATE) + kBinOver + kBinLevels;
   for (int i = 0; i < 3; ++i) a.bg[i] = p->settings.bg[i];
@@ -306,7 +305,6 @@ BlendArgs blend_args(const sixdgs_plan* p, void* ws) {
                       : nullptr;
   a.tile_queue = p->settings.persistent ? ws_ptr<uint32_t>(ws, p, WS_COUNTERS) + 32 : nullptr;
   a.total_tiles = a.frame_tiles = (uint32_t)p->total_tiles;
-  a.spin_budget = spin_budget(p);
   return a;
 }
 
@@ -334,7 +332,6 @@ sixdgs_status render_banded(const sixdgs_plan* p, int64_t slots, const sixdgs_sc
   BinArgs b = bin_args(p, ws, status_dev);
   BlendArgs f = blend_args(p, ws);
   f.images = images_dev;
-  f.status = status_dev;
   b.band = 0;
   for (int64_t first = 0; first < p->total_tiles; first += slots, ++b.band) {
     b.tile_first = (uint32_t)first;
@@ -433,7 +430,7 @@ sixdgs_status sixdgs_bin_sort(const sixdgs_plan* p, void* ws, size_t ws_bytes, i
 
 sixdgs_status sixdgs_raster_fwd(const sixdgs_plan* p, void* ws, size_t ws_bytes, float* images_dev,
                                 const float* targets_dev, float* grad_images_dev, double* loss_dev,
-                                int32_t* status_dev, sixdgs_stream_t stream_) {
+                                int32_t* /*status_dev*/, sixdgs_stream_t stream_) {
   sixdgs_status e = check_ws(p, ws, ws_bytes);
   if (e != SIXDGS_OK) return e;
   if (!images_dev) return SIXDGS_ERR_INVALID_ARG;
@@ -445,14 +442,13 @@ sixdgs_status sixdgs_raster_fwd(const sixdgs_plan* p, void* ws, size_t ws_bytes,
   a.targets = targets_dev;
   a.grad_images = grad_images_dev;
   a.loss = loss_dev;
-  a.status = status_dev;
   launch_blend_fwd(a, p->total_tiles, reinterpret_cast<cudaStream_t>(stream_));
   return launch_status();
 }
 
 sixdgs_status sixdgs_raster_fwd_bwd(const sixdgs_plan* p, void* ws, size_t ws_bytes, float* images_dev,
                                     const float* targets_dev, float* grad_images_dev, double* loss_dev,
-                                    int32_t* status_dev, sixdgs_stream_t stream_) {
+                                    int32_t* /*status_dev*/, sixdgs_stream_t stream_) {
   sixdgs_status e = check_ws(p, ws, ws_bytes);
   if (e != SIXDGS_OK) return e;
   if (p->settings.inference || !images_dev || !targets_dev || !loss_dev) return SIXDGS_ERR_INVALID_ARG;
@@ -462,13 +458,12 @@ sixdgs_status sixdgs_raster_fwd_bwd(const sixdgs_plan* p, void* ws, size_t ws_by
   a.grad_images = grad_images_dev;
   a.loss = loss_dev;
   a.grad_rec = ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
-  a.status = status_dev;
   launch_blend_fused(a, p->total_tiles, reinterpret_cast<cudaStream_t>(stream_));
   return launch_status();
 }
 
 sixdgs_status sixdgs_blend_bwd(const sixdgs_plan* p, void* ws, size_t ws_bytes, const float* images_dev,
-                               const float* grad_images_dev, int32_t* status_dev, sixdgs_stream_t stream_) {
+                               const float* grad_images_dev, int32_t* /*status_dev*/, sixdgs_stream_t stream_) {
   sixdgs_status e = check_ws(p, ws, ws_bytes);
   if (e != SIXDGS_OK) return e;
   if (p->settings.inference) return SIXDGS_ERR_INVALID_ARG;
@@ -478,7 +473,6 @@ sixdgs_status sixdgs_blend_bwd(const sixdgs_plan* p, void* ws, size_t ws_bytes, 
   a.grad_in = grad_images_dev;
   a.grad_rec = ws_ptr<float>(ws, p, SIXDGS_WS_GRADREC);
   a.recompute = p->settings.store_aux ? 0 : 1;
-  a.status = status_dev;
   launch_blend_bwd(a, p->total_tiles, reinterpret_cast<cudaStream_t>(stream_));
   return launch_status();
 }

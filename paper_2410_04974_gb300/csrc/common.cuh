@@ -109,23 +109,4 @@ __device__ __forceinline__ float entry_q(const float4& a, const float4& b, float
   return __fmaf_rn(t1, d.x, t2);
 }
 
-// Decoupled look-back status words: 2-bit flag in the top bits.
-constexpr uint32_t kFlagAgg = 1u << 30;
-constexpr uint32_t kFlagInc = 2u << 30;
-constexpr uint32_t kFlagMask = 3u << 30;
-constexpr uint32_t kValMask = ~kFlagMask;
-
-__device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) {
-  return *reinterpret_cast<const volatile uint32_t*>(p);
-}
-__device__ __forceinline__ void st_volatile(uint32_t* p, uint32_t v) {
-  *reinterpret_cast<volatile uint32_t*>(p) = v;
-}
-
-__device__ __forceinline__ uint32_t lane_id() {
-  uint32_t l;
-  asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
-  return l;
-}
-
 }  // namespace sixdgs

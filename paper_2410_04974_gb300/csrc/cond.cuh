@@ -39,11 +39,6 @@ __device__ __forceinline__ void cholesky_from(Plane plane, float L[6][6]) {
     }
 }
 
-__device__ __forceinline__ void load_cholesky(const float* __restrict__ l_raw, int64_t n, int64_t g,
-                                              float L[6][6]) {
-  cholesky_from([&](int p) { return __ldg(l_raw + p * n + g); }, L);
-}
-
 // Sigma_p = Lpp Lpp^T, Sigma_pd = Lpp Ldp^T, Sigma_d = Ldp Ldp^T + Ldd Ldd^T.
 __device__ __forceinline__ void sigma_blocks(const float L[6][6], M3& Sp, M3& Spd, M3& Sd) {
 #pragma unroll

@@ -9,7 +9,7 @@ namespace sixdgs {
 // stream capture it may be set up while the kernel before it in the stream
 // ends, which hides most of the gap between two small kernels: 59 -> 43 us for
 // the seven kernels of a 4,096-Gaussian training step, 67 -> 52 us for the six
-// of a 6,660-Gaussian frame, 964 -> 945 us at 300k / 8 x 800^2.  A captured
+// (now seven) of a 6,660-Gaussian frame, 964 -> 945 us at 300k / 8 x 800^2.  A captured
 // graph keeps the plain dependency: it hides the gaps itself (no difference
 // measured).
 template <typename... Params, typename... Args>
@@ -133,7 +133,6 @@ struct BlendArgs {
   const PairRec* rec;
   uint32_t n_pairs;
   const uint32_t* sorted;   // pair index per list entry
-  const uint2* ranges;
   const uint4* order;       // TileWork of every tile, longest lists first
   const uint32_t* n_busy;   // tiles with a list (the others come last)
   float bg[3];
@@ -153,8 +152,6 @@ struct BlendArgs {
   uint32_t* tile_queue;
   uint32_t total_tiles;     // of the band (BinArgs)
   uint32_t frame_tiles;     // of the frame
-  int64_t spin_budget;      // clock cycles a shared-memory ring wait may take
-  int32_t* status;
 };
 
 struct ProjectBwdArgs {

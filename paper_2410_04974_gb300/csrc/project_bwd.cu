@@ -27,7 +27,6 @@
 // two kernels, geometry and colour, in Gaussian order: 146 -> 130 us at 300k /
 // 8 x 800^2 (3.3 of 8 views see a Gaussian), 546 -> 456 us at 2M / 4 views
 // (0.3 of 4), 1354 -> 1236 us at 500k / 64 views.
-#include "bin.cuh"
 #include "common.cuh"
 #include "cond.cuh"
 #include "kernels.cuh"

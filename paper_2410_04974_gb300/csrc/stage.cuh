@@ -102,14 +102,14 @@ __device__ __forceinline__ void stage_issue(float* tile, int np, int split, Src 
   }
 }
 
-// Waits for group `grp` of stage_issue (bulk mode; a no-op otherwise).  False
-// when the bounded wait ran out, after which that group's contents are
-// unspecified.
+// Waits for group `grp` of stage_issue (bulk mode; a no-op otherwise).  A wait
+// that runs out of its budget is extended once, as the copies land in this CTA's
+// memory: true if they came then (nothing is reported), false if not, after which
+// that group's contents are unspecified.
 __device__ __forceinline__ bool stage_wait(uint64_t* bars, int grp, bool bulk, int64_t budget) {
   if (!bulk) return true;
   bool ok = mbar_wait(&bars[grp], 0, budget);
-  // the copies land in this CTA's memory: let them finish, for at least 2^24
-  // cycles (about 8 ms) however short the budget
+  // at least 2^24 cycles (about 8 ms), however short the budget
   if (!ok) ok = mbar_wait(&bars[grp], 0, budget > (1 << 24) ? budget : (1 << 24));
   return ok;
 }

@@ -68,10 +68,11 @@ def test_launch_count_of_a_step_follows_the_rule_for_large_rectangles(rules):
 
     frames = [(n, cams, size) for n in (0, 1, 4_000, 17_133, 38_784, 38_785, 300_000) for cams in (1, 2, 3, 8, 20, 64)
               for size in (128, 512, 513, 1408)]
+    plans = [make_plan(n, 3, synth.ring_cameras(cams, size, size), make_settings()) for n, cams, size in frames]
+    asked = rules([(n, cams, int(p.total_tiles), 152) for (n, cams, _), p in zip(frames, plans)])
     seen = set()
-    for n, cams, size in frames:
-        plan = make_plan(n, 3, synth.ring_cameras(cams, size, size), make_settings())
-        count = n > 0 and bool(rules([(n, cams, int(plan.total_tiles), 152)])[0][6])
+    for (n, cams, size), plan, rule in zip(frames, plans, asked):
+        count = n > 0 and bool(rule[6])
         # upload, projection, count, scan, scatter, sort, fused blend, per-Gaussian backward
         want = -(-cams // 48) + (n > 0) + count + 3 + 1 + (n > 0)
         assert bench.step_launches(plan) == want, (n, cams, size)
