@@ -284,32 +284,22 @@ struct __align__(16) WarpScratch {
 // Fills a warp's lists with the batch's entries [c0, c0 + kChunk) (cnt in the
 // batch); returns the number of steps of the longer one, a multiple of kStep.
 // cull: the ballots of the warp's left block (its right one's follow).
-// twin (may be null): whether the two blocks reach nearly the same entries; then
-// both lists get the entries of either (which change nothing at the other block).
+// kTwin: both lists get the entries of either block (which change nothing at the
+// other).
+template <bool kTwin>
 __device__ __forceinline__ int fill_lists(const uint32_t* cull, int batch, int c0, int cnt, WalkLists& lists,
-                                          uint32_t* n_warp = nullptr, bool* twin = nullptr) {
+                                          uint32_t* n_warp = nullptr) {
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
   uint32_t n0 = 0u, n1 = 0u;
   __syncwarp();   // the lists are no longer read
   cull += c0 >> 5;
-  if (twin) {
-    uint32_t both = 0u, either = 0u;
-#pragma unroll
-    for (int g = 0; g < kChunk / 32; ++g)
-      if (c0 + 32 * g < cnt) {
-        const uint32_t m0 = cull[g], m1 = cull[cull_stride(batch) + g];
-        both += __popc(m0 & m1);
-        either += __popc(m0 | m1);
-      }
-    *twin = 16u * (either - both) <= either;
-  }
 #pragma unroll
   for (int g = 0; g < kChunk / 32; ++g) {
     const int base = c0 + 32 * g;
     if (base < cnt) {
       uint32_t m0 = cull[g], m1 = cull[cull_stride(batch) + g];
-      if (twin && *twin) m0 = m1 = m0 | m1;
+      if (kTwin) m0 = m1 = m0 | m1;
       const uint16_t off = (uint16_t)((base + lane) * (int)sizeof(Entry));
       if ((m0 >> lane) & 1u) lists.off[0][n0 + __popc(m0 & below)] = off;
       if ((m1 >> lane) & 1u) lists.off[1][n1 + __popc(m1 & below)] = off;
@@ -366,7 +356,7 @@ __device__ __forceinline__ FwdPixel fwd_walk(const BlendArgs& a, float2 npix, ui
     if (__all_sync(0xffffffffu, done)) continue;
     uint32_t stop_off = 0xffffffffu;   // of the entry this pixel stopped at in this batch
     for (int c0 = 0; c0 < cnt; c0 += kChunk) {
-      const int steps = fill_lists(warp_cull(a, s_e), B, c0, cnt, lists, kCount ? &n_warp : nullptr);
+      const int steps = fill_lists<false>(warp_cull(a, s_e), B, c0, cnt, lists, kCount ? &n_warp : nullptr);
       bool all = false;
 #pragma unroll 1
       for (int i = 0; i < steps && !all; i += kStep) {
@@ -524,11 +514,11 @@ __device__ __forceinline__ void red_add4(float* addr, float x, float y, float z,
 }
 
 // Pass 2 over slots [0, k) of both halves.  null_off: offset of the null entry.
-// twin (kTwins): both halves' slots hold the same entries, whose sums are added
-// before they go to global memory.
+// kTwins: both halves' slots hold the same entries, whose sums are added before
+// they go to global memory.
 template <bool kTwins>
 __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws, int k, const Entry* s_e, float2 npix,
-                                            uint32_t null_off, bool twin) {
+                                            uint32_t null_off) {
   static_assert(kSlots == 8 && kBlkW == 4 && kSubH == 4, "two rows of a block per lane");
   __syncwarp();
   const int lane = threadIdx.x & 31;
@@ -582,11 +572,11 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
     g[6] = m[6];
     g[7] = m[7];
     g[8] = m[8];
-    if (kTwins && twin) {
+    if (kTwins) {
 #pragma unroll
       for (int q = 0; q < 9; ++q) g[q] += __shfl_xor_sync(lanes, g[q], 16);
     }
-    if (!(kTwins && twin) || h == 0) {
+    if (!kTwins || h == 0) {
       float* dst = a.grad_rec + (size_t)__float_as_uint(en.c.w) * 12;
       // a record is 48 bytes, 16-byte aligned: floats 0-3 and 4-7 as vectors
       red_add4(dst, g[0], g[1], g[2], g[3]);
@@ -602,12 +592,12 @@ __device__ __forceinline__ void flush_slots(const BlendArgs& a, WarpScratch& ws,
 // kRecompute: re-derive the stop from the transmittance; otherwise the pixel
 // walks `bound` entries.  staged (CTA-uniform): the whole list is already in
 // shared memory (a single batch that the forward of the same CTA staged).
-// kTwins: where a warp's two blocks reach nearly the same entries, they walk the
-// same list and their sums go to global memory together.  In frames of few
-// Gaussians over many tiles every record takes the sums of thousands of blocks,
-// and the reductions to a few records are what bounds the kernel (1,000 Gaussians
-// of 5,600 tiles at 1408^2: blend_bwd 1,117 -> 611 us, fused 1,135 -> 812).  Only
-// in the kernels for sparse frames: elsewhere blocks are seldom twins.
+// kTwins (the kernels for sparse frames): a warp's two blocks walk the same list,
+// and their sums go to global memory together.  In frames of few Gaussians over
+// many tiles a warp's blocks reach much the same entries, and every record takes
+// the sums of thousands of blocks, which bounds the kernel: 1,000 Gaussians of
+// 5,600 tiles at 1408^2 blend_bwd 1,117 -> 597 us, fused 1,135 -> 813.  (Deciding
+// it list by list gained nothing: 611 and 812.)
 template <bool kRecompute, bool kTwins>
 __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 range, bool inside, const float* Cf,
                                          const float* dC, uint32_t bound, bool staged, Entry* s_e, WarpScratch& ws) {
@@ -626,7 +616,6 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
   // (dC0, dC1, 1, dC2): pass 2 pairs the 1 with dq and dC2 with w
   ws.pix[lane + (lane >> 3)] = make_float4(dC[0], dC[1], 1.f, dC[2]);
   int k0 = 0;         // slots filled (warp-uniform, a multiple of kStep)
-  bool twin = false;  // both halves' slots hold the same entries
 
   for (uint32_t start = range.x; start < range.y; start += B) {
     // a staged list is already in shared memory (read-only): no CTA barrier
@@ -640,13 +629,7 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
     // entries at offsets below lim of this batch lie within the pixel's walk
     const uint32_t lim = min((uint32_t)cnt, bound - min(bound, start - range.x)) * (uint32_t)sizeof(Entry);
     for (int c0 = 0; c0 < cnt; c0 += kChunk) {
-      bool same = false;
-      const int steps = fill_lists(warp_cull(a, s_e), B, c0, cnt, ws.lists, nullptr, kTwins ? &same : nullptr);
-      if (kTwins && same != twin) {
-        if (k0) flush_slots<kTwins>(a, ws, k0, s_e, npix, null_off, twin);
-        k0 = 0;
-        twin = same;
-      }
+      const int steps = fill_lists<kTwins>(warp_cull(a, s_e), B, c0, cnt, ws.lists);
       bool all = false;
 #pragma unroll 1
       for (int i = 0; i < steps && !all; i += kStep) {
@@ -693,7 +676,7 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
         for (int k = 0; k < kStep; ++k) slot[k * 33] = res[k];
         k0 += kStep;
         if (k0 == kSlots) {
-          flush_slots<kTwins>(a, ws, kSlots, s_e, npix, null_off, twin);
+          flush_slots<kTwins>(a, ws, kSlots, s_e, npix, null_off);
           k0 = 0;
         }
         // (a padded list says nothing about the walk's end)
@@ -704,7 +687,7 @@ __device__ __forceinline__ void bwd_walk(const BlendArgs& a, float2 npix, uint2 
     }
     if (!kRecompute) done = done || start - range.x + cnt >= bound;
     if (k0) {   // the slots refer to this batch's shared-memory records
-      flush_slots<kTwins>(a, ws, k0, s_e, npix, null_off, twin);
+      flush_slots<kTwins>(a, ws, k0, s_e, npix, null_off);
       k0 = 0;
     }
   }
@@ -747,11 +730,11 @@ __device__ __forceinline__ void bwd_walk_short(const BlendArgs& a, float2 npix, 
     ws.dqw[k][lane] = make_float2(dq, w);
     if ((lane & 15) == 0) reinterpret_cast<uint16_t*>(ws.slot[lane >> 4])[k] = (uint16_t)off;
     if (++k == kSlots) {
-      flush_slots<true>(a, ws, kSlots, s_e, npix, 0xffffffffu, true);
+      flush_slots<true>(a, ws, kSlots, s_e, npix, 0xffffffffu);
       k = 0;
     }
   }
-  if (k) flush_slots<true>(a, ws, k, s_e, npix, 0xffffffffu, true);
+  if (k) flush_slots<true>(a, ws, k, s_e, npix, 0xffffffffu);
 }
 
 // Backward blend of tile tw by the calling CTA.  kRecompute: re-derive
