@@ -332,6 +332,7 @@ sixdgs_status render_banded(const sixdgs_plan* p, int64_t slots, const sixdgs_sc
   BinArgs b = bin_args(p, ws, status_dev);
   BlendArgs f = blend_args(p, ws);
   f.images = images_dev;
+  f.pair_counts = nullptr;   // (nobody could read them)
   b.band = 0;
   for (int64_t first = 0; first < p->total_tiles; first += slots, ++b.band) {
     b.tile_first = (uint32_t)first;

@@ -38,14 +38,15 @@ def test_the_library_holds_no_more_than_the_stated_array():
     (40, -5.5, [(16_000, 13_000)], 6, 0),             # 3.25 million tiles, almost all empty
     (40, 0.0, [(16_000, 13_000)], 6, 1 << _lib.ERR_CAPACITY),
 ])
-def test_banded_frames_equal_the_staged_calls(n, log_scale, sizes, bands, status):
+@pytest.mark.parametrize("extra", [{}, {"count_pairs": True, "persistent": True, "store_aux": True}], ids=["plain", "extra"])
+def test_banded_frames_equal_the_staged_calls(n, log_scale, sizes, bands, status, extra):
     tile = (8, 8)
     scene = synth.scene_cube(n, 3)
     scene.l_raw[:3] += log_scale                      # a few tiles a Gaussian: the call plans 4 a pair and 4,096
     scene.l_raw[6:] = 0.0
     scene.opacity_logit += 3.0
     cams = [synth.look_at_camera((4.0, 0.3 * k, 0.2), *s) for k, s in enumerate(sizes)]
-    settings = make_settings(tile=tile)
+    settings = make_settings(tile=tile, **extra)
     params = sx.params_to_device(scene)
     r = sx.Renderer(scene.n, scene.sh_degree, cams, tile=tile, inference=True)
     ref = r.forward(params, check=False)
